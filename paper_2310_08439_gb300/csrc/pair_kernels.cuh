@@ -7,13 +7,25 @@
 //                   fly); ScatterSum into forces, virial
 //                                        -- Eqs. dP_abkd, U_abck, F1_abcx, F2_abcx
 //
+// The moments are kept in 16 components, not the 20 monomials of Eq. T_dm.  On
+// the unit sphere the monomials of rank 2 and 3 repeat those of rank 0 and 1
+// (xx + yy + zz = 1, xxx + xyy + xzz = x, ...), so the rank-m sum
+// sum_d T_dm P_d^2, which is the double sum of (u_j . u_k)^m, splits into
+// harmonics: (u.v)^2 = 1/3 + (5 terms of degree 2), (u.v)^3 = 3/5 u.v + (7
+// terms of degree 3).  harmonics16 lists the polynomials, c_W their weights:
+//   G_0 = |A_0|                     G_1 = sum_{1..3} A_c^2
+//   G_2 = A_0^2 / 3 + sum_{4..8} w_c A_c^2
+//   G_3 = 3/5 G_1 + sum_{9..15} w_c A_c^2
+// The sums are the same numbers with 16 instead of 20 multiply-adds per
+// channel, pair and pass, and every term is a square with a positive weight.
+//
 // One warp owns one centre atom.  The in-cutoff pairs of each atom come from
 // the pair cache (filled by k_screen in screen.cu, read by both passes) or,
 // without a cache, from screening the table in the pass itself, compacted
 // through a per-warp shared-memory queue; either way every lane works on an
 // in-cutoff pair.  Each lane computes H and M for one
 // neighbour and stages them in shared memory; the warp then accumulates the
-// per-atom P[b][k][d] outer products with each lane owning a (K/8 x 5) block
+// per-atom P[b][k][d] outer products with each lane owning a (K/8 x 4) block
 // of P in registers.  In k_force each lane owns one cached pair and reads the
 // atom's P' from shared memory with broadcast loads.
 //
@@ -30,16 +42,19 @@ namespace {
 constexpr int PW = PAIR_WARPS;   // warps per block in the pair kernels
 constexpr float PI_F = 3.14159265358979323846f;
 
-// multiplicities T_d and ranks m(d) in the row order of Eq. T_dm:
-// 1 | x y z | xx xy xz yy yz zz | xxx xxy xxz xyy xyz xzz yyy yyz yzz zzz
-__constant__ float c_T[NMOM] = {1, 1, 1, 1, 1, 2, 2, 1, 2, 1, 1, 3, 3, 3, 6, 3, 1, 3, 3, 1};
+// weights w_c of the squared sums A_c, in the order of harmonics16
+__constant__ float c_W[NHAR] = {1.f, 1.f, 1.f, 1.f, 2.f, 2.f, 2.f, 0.5f, 1.5f, 0.1f, 0.15f, 0.15f, 1.5f, 6.f, 0.25f, 0.25f};
 
-__device__ __forceinline__ void moments20(float x, float y, float z, float *M) {
-    M[0] = 1.f;
-    M[1] = x; M[2] = y; M[3] = z;
-    M[4] = x * x; M[5] = x * y; M[6] = x * z; M[7] = y * y; M[8] = y * z; M[9] = z * z;
-    M[10] = M[4] * x; M[11] = M[4] * y; M[12] = M[4] * z; M[13] = x * M[7]; M[14] = M[5] * z;
-    M[15] = x * M[9]; M[16] = M[7] * y; M[17] = M[7] * z; M[18] = y * M[9]; M[19] = M[9] * z;
+// 1 | x y z | xy yz xz x^2-y^2 | z^2-1/3, z(5z^2-3) x(5z^2-1) y(5z^2-1) | z(x^2-y^2) xyz x(x^2-3y^2) y(3x^2-y^2)
+// of a unit vector (degrees 0; 1; 2; 3)
+__device__ __forceinline__ void harmonics16(float x, float y, float z, float *Y) {
+    const float xx = x * x, yy = y * y, zz = z * z, d = xx - yy, q = fmaf(5.f, zz, -1.f);
+    Y[0] = 1.f;
+    Y[1] = x; Y[2] = y; Y[3] = z;
+    Y[4] = x * y; Y[5] = y * z; Y[6] = x * z; Y[7] = d;
+    Y[8] = zz - (1.f / 3.f);
+    Y[9] = z * fmaf(5.f, zz, -3.f); Y[10] = x * q; Y[11] = y * q;
+    Y[12] = z * d; Y[13] = Y[4] * z; Y[14] = x * fmaf(-3.f, yy, xx); Y[15] = y * fmaf(3.f, xx, -yy);
 }
 
 // 2^x and 1/sqrt(x) from the special-function unit (PTX ex2.approx /
@@ -357,8 +372,25 @@ struct PairStream {
     }
 };
 
+// G_m of one channel, m = g, from the sums A of the four lanes g = 0..3 that
+// hold components 4g .. 4g + 3 of it (lane 0: degrees 0 and 1; lane 1: four of
+// degree 2; lane 2: the fifth of degree 2 and three of degree 3; lane 3: four
+// of degree 3).  m = 0 is |A_0| and not the root of its square, so that a
+// channel's tiny sum (|A_0| < 1e-19, whose square underflows in FP32) is not
+// read as 0.
+__device__ __forceinline__ float desc_value(const float (&A)[4], const float (&Wg)[4], int g) {
+    const float s0 = Wg[0] * A[0] * A[0];
+    const float s13 = Wg[1] * A[1] * A[1] + Wg[2] * A[2] * A[2] + Wg[3] * A[3] * A[3];
+    const int quad = (threadIdx.x & 31) & ~3;
+    const float a00 = __shfl_sync(0xffffffffu, s0, quad);     // A_0^2
+    const float one = __shfl_sync(0xffffffffu, s13, quad);    // G_1
+    const float up = __shfl_up_sync(0xffffffffu, g == 1 ? s0 + s13 : s13, 1);
+    const float val2 = fmaf(1.f / 3.f, a00, up + s0), val3 = fmaf(0.6f, one, up + (s0 + s13));
+    return g == 0 ? fabsf(A[0]) : (g == 1 ? one : (g == 2 ? val2 : val3));
+}
+
 // ---------------------------------------------------------------------------
-// descriptor forward: P and G per atom
+// descriptor forward: A and G per atom
 // ---------------------------------------------------------------------------
 // CACHED: the atom's in-cutoff pairs come from the pair cache filled by
 // k_screen; otherwise the pass screens the table itself (for_pairs).  K > 32
@@ -377,18 +409,18 @@ __global__ void __launch_bounds__(PW * 32) k_desc(DevModel m, DevNlist nl, const
     __shared__ float4 s_q[PW][64];
     __shared__ float2 s_q2[PW][64];
     // staged pair data, one column per pair: H_k in row (k % KPL) 8 + k / KPL,
-    // M_d in row (d % 5) 4 + d / 5, so that the lane owning k-group kg and
-    // d-group g reads four pairs of a row with one conflict-free vector load
+    // Y_c in row (c % 4) 4 + c / 4, so that the lane owning k-group kg and
+    // component group g reads four pairs of a row with one conflict-free vector load
     __shared__ __align__(16) float s_H[PW][KC * RS];
-    __shared__ __align__(16) float s_M[PW][NMOM * RS];
+    __shared__ __align__(16) float s_M[PW][NHAR * RS];
     stage_rad2(s_rad2, m.radial, S * S * K);
     __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int kg = lane >> 2, g = lane & 3;
     const unsigned lt = (1u << lane) - 1u;
-    float Tg[5];
+    float Wg[4];
 #pragma unroll
-    for (int dd = 0; dd < 5; ++dd) Tg[dd] = c_T[5 * g + dd];
+    for (int dd = 0; dd < 4; ++dd) Wg[dd] = c_W[4 * g + dd];
     const int64_t total = (int64_t)gridDim.x * PW;
     // CACHED: the pair-cache batches are read one batch ahead, across chunk
     // and atom boundaries (the next atom's segment one atom ahead, its perm
@@ -403,13 +435,13 @@ __global__ void __launch_bounds__(PW * 32) k_desc(DevModel m, DevNlist nl, const
         for (int k0 = 0; k0 < K; k0 += KC) {
         // two partial sums per P entry (even and odd pair slots), so that
         // the accumulation runs on packed FP32x2 multiply-adds
-        float2 acc2[S][KPL][5];
+        float2 acc2[S][KPL][4];
 #pragma unroll
         for (int s = 0; s < S; ++s)
 #pragma unroll
             for (int kk = 0; kk < KPL; ++kk)
 #pragma unroll
-                for (int dd = 0; dd < 5; ++dd) acc2[s][kk][dd] = make_float2(0.f, 0.f);
+                for (int dd = 0; dd < 4; ++dd) acc2[s][kk][dd] = make_float2(0.f, 0.f);
         float *sH = s_H[warp];
         float *sM = s_M[warp];
         auto pair_fn = [&](const float4 e, const float2 e2, bool valid, int) {
@@ -428,7 +460,7 @@ __global__ void __launch_bounds__(PW * 32) k_desc(DevModel m, DevNlist nl, const
                       if (valid) {
                           float r_hi, r_lo, ir;
                           split_sqrt(e2.x, e2.y, r_hi, r_lo, ir);
-                          float H[KC], M[NMOM];
+                          float H[KC], M[NHAR];
                           if (TAB)
                               radial_tab<KC, false>(m.rtab + (size_t)(ti * S + b) * m.rtab_n * 4 * K, K, k0,
                                                     m.rtab_scale, r_hi, r_lo, H, nullptr);
@@ -445,11 +477,11 @@ __global__ void __launch_bounds__(PW * 32) k_desc(DevModel m, DevNlist nl, const
                                   H[k + 1] = o.H.y;
                               }
                           }
-                          moments20(e.x * ir, e.y * ir, e.z * ir, M);
+                          harmonics16(e.x * ir, e.y * ir, e.z * ir, M);
 #pragma unroll
                           for (int k = 0; k < KC; ++k) sH[((k % KPL) * 8 + k / KPL) * RS + slot] = H[k];
 #pragma unroll
-                          for (int d = 0; d < NMOM; ++d) sM[((d % 5) * 4 + d / 5) * RS + slot] = M[d];
+                          for (int d = 0; d < NHAR; ++d) sM[((d % 4) * 4 + d / 4) * RS + slot] = M[d];
                       }
                       __syncwarp();
                       // P[b][k][d] += H_k M_d: four pairs per step, the rest one at a time
@@ -459,17 +491,17 @@ __global__ void __launch_bounds__(PW * 32) k_desc(DevModel m, DevNlist nl, const
                           const int stop = start + cnt[s];
                           int q = start;
                           for (; q + 4 <= stop; q += 4) {
-                              float4 hv[KPL], mv[5];
+                              float4 hv[KPL], mv[4];
 #pragma unroll
                               for (int kk = 0; kk < KPL; ++kk)
                                   hv[kk] = *reinterpret_cast<const float4 *>(&sH[(kk * 8 + kg) * RS + q]);
 #pragma unroll
-                              for (int dd = 0; dd < 5; ++dd)
+                              for (int dd = 0; dd < 4; ++dd)
                                   mv[dd] = *reinterpret_cast<const float4 *>(&sM[(dd * 4 + g) * RS + q]);
 #pragma unroll
                               for (int kk = 0; kk < KPL; ++kk)
 #pragma unroll
-                                  for (int dd = 0; dd < 5; ++dd) {
+                                  for (int dd = 0; dd < 4; ++dd) {
                                       float2 x = acc2[s][kk][dd];
                                       x = __ffma2_rn(make_float2(hv[kk].x, hv[kk].y), make_float2(mv[dd].x, mv[dd].y), x);
                                       x = __ffma2_rn(make_float2(hv[kk].z, hv[kk].w), make_float2(mv[dd].z, mv[dd].w), x);
@@ -477,15 +509,15 @@ __global__ void __launch_bounds__(PW * 32) k_desc(DevModel m, DevNlist nl, const
                                   }
                           }
                           for (; q < stop; ++q) {
-                              float hv[KPL], mv[5];
+                              float hv[KPL], mv[4];
 #pragma unroll
                               for (int kk = 0; kk < KPL; ++kk) hv[kk] = sH[(kk * 8 + kg) * RS + q];
 #pragma unroll
-                              for (int dd = 0; dd < 5; ++dd) mv[dd] = sM[(dd * 4 + g) * RS + q];
+                              for (int dd = 0; dd < 4; ++dd) mv[dd] = sM[(dd * 4 + g) * RS + q];
 #pragma unroll
                               for (int kk = 0; kk < KPL; ++kk)
 #pragma unroll
-                                  for (int dd = 0; dd < 5; ++dd)
+                                  for (int dd = 0; dd < 4; ++dd)
                                       acc2[s][kk][dd].x = fmaf(hv[kk], mv[dd], acc2[s][kk][dd].x);
                           }
                           start += (cnt[s] + 3) & ~3;
@@ -504,48 +536,26 @@ __global__ void __launch_bounds__(PW * 32) k_desc(DevModel m, DevNlist nl, const
         } else {
             for_pairs(nl, a, nl.beg[a], nl.end[a], m.rc2h, m.rc2l, s_q[warp], s_q2[warp], lane, pair_fn);
         }
-        float acc[S][KPL][5];
+        float acc[S][KPL][4];
 #pragma unroll
         for (int s = 0; s < S; ++s)
 #pragma unroll
             for (int kk = 0; kk < KPL; ++kk)
 #pragma unroll
-                for (int dd = 0; dd < 5; ++dd) acc[s][kk][dd] = acc2[s][kk][dd].x + acc2[s][kk][dd].y;
-        // P[b][k][d] for the backward pass
-        float *Pa = Pout + (size_t)p * (S * K * NMOM);   // workspaces are indexed by perm position
+                for (int dd = 0; dd < 4; ++dd) acc[s][kk][dd] = acc2[s][kk][dd].x + acc2[s][kk][dd].y;
+        // A[b][k][c] for the backward pass
+        float *Pa = Pout + (size_t)p * (S * K * NHAR);   // workspaces are indexed by perm position
 #pragma unroll
         for (int s = 0; s < S; ++s)
 #pragma unroll
             for (int kk = 0; kk < KPL; ++kk)
+                *reinterpret_cast<float4 *>(Pa + (s * K + k0 + kg * KPL + kk) * NHAR + 4 * g) =
+                    make_float4(acc[s][kk][0], acc[s][kk][1], acc[s][kk][2], acc[s][kk][3]);
 #pragma unroll
-                for (int dd = 0; dd < 5; ++dd)
-                    Pa[(s * K + k0 + kg * KPL + kk) * NMOM + 5 * g + dd] = acc[s][kk][dd];
-        // G[b][k][m] = sigma(sum_{d in rank m} T_d P^2)
+        for (int s = 0; s < S; ++s)
 #pragma unroll
-        for (int s = 0; s < S; ++s) {
-#pragma unroll
-            for (int kk = 0; kk < KPL; ++kk) {
-                float sq[5];
-#pragma unroll
-                for (int dd = 0; dd < 5; ++dd) sq[dd] = Tg[dd] * acc[s][kk][dd] * acc[s][kk][dd];
-                const float tot = sq[0] + sq[1] + sq[2] + sq[3] + sq[4];
-                // rank m of the four lanes g = 0..3 of this k: lane 0 holds
-                // d = 0 (m = 0), d = 1..3 (m = 1) and d = 4 (m = 2); lane 1
-                // d = 5..9 (m = 2); lanes 2 and 3 d = 10..19 (m = 3).  Lane g
-                // writes G for m = g: m = 2 and m = 3 are pair sums (xor 1),
-                // and lanes 1 and 2 fetch theirs from lane 0.
-                const float s123 = sq[1] + sq[2] + sq[3];
-                const float a = (g == 0) ? sq[4] : tot;
-                const float asum = a + __shfl_xor_sync(0xffffffffu, a, 1);    // lanes 0, 1: m = 2; lanes 2, 3: m = 3
-                const float m1 = __shfl_xor_sync(0xffffffffu, s123, 1);      // lane 1: lane 0's d = 1..3
-                const float m2 = __shfl_xor_sync(0xffffffffu, asum, 2);      // lane 2: lane 0's m = 2
-                // m = 0: sqrt(T_0 P^2) = |P| (T_0 = 1), taken as |P| so that a
-                // channel's tiny P (|P| < 1e-19, whose square underflows in
-                // FP32) is not read as 0; elsewhere bitwise the same value
-                const float val = (g == 0) ? fabsf(acc[s][kk][0]) : ((g == 1) ? m1 : ((g == 2) ? m2 : asum));
-                G[(size_t)p * Dd + (s * K + k0 + kg * KPL + kk) * 4 + g] = val;
-            }
-        }
+            for (int kk = 0; kk < KPL; ++kk)
+                G[(size_t)p * Dd + (s * K + k0 + kg * KPL + kk) * 4 + g] = desc_value(acc[s][kk], Wg, g);
         }
         if constexpr (CACHED) ps.atom_ends();
     }
@@ -588,44 +598,45 @@ __device__ __forceinline__ void kahan_add(float &sum, float &comp, float x) {
     sum = t;
 }
 
-// The rest of g_ij once V_d and W_d of the pair are known, as packed pairs
-// (d, d + 1).  The moments are formed in the same pairs, so that
-// dE/dr = sum_d W_d M_d runs on FP32x2 multiply-adds.
-__device__ __forceinline__ void pair_grad_tail(const float2 (&V2)[NMOM / 2], const float2 (&W2)[NMOM / 2], float ux,
-                                               float uy, float uz, float ir, float &gxs, float &gys, float &gzs) {
-    // M2[q] = (M_2q, M_2q+1) in the row order of moments20
-    float2 M2[NMOM / 2];
-    M2[0] = make_float2(1.f, ux);
-    M2[1] = make_float2(uy, uz);
-    M2[2] = make_float2(ux * ux, ux * uy);
-    M2[3] = make_float2(ux * uz, uy * uy);
-    M2[4] = make_float2(uy * uz, uz * uz);
-    M2[5] = make_float2(M2[2].x * ux, M2[2].x * uy);
-    M2[6] = make_float2(M2[2].x * uz, ux * M2[3].y);
-    M2[7] = make_float2(M2[2].y * uz, ux * M2[4].y);
-    M2[8] = make_float2(M2[3].y * uy, M2[3].y * uz);
-    M2[9] = make_float2(uy * M2[4].y, M2[4].y * uz);
+// The rest of g_ij once V_c and W_c of the pair are known, as packed pairs
+// (c, c + 1).  The harmonics are formed in the same pairs, so that
+// dE/dr = sum_c W_c Y_c runs on FP32x2 multiply-adds.
+__device__ __forceinline__ void pair_grad_tail(const float2 (&V2)[NHAR / 2], const float2 (&W2)[NHAR / 2], float x,
+                                               float y, float z, float ir, float &gxs, float &gys, float &gzs) {
+    const float xx = x * x, yy = y * y, zz = z * z, d = xx - yy, q = fmaf(5.f, zz, -1.f);
+    const float xy = x * y, yz = y * z, xz = x * z;
+    const float p14 = fmaf(-3.f, yy, xx), p15 = fmaf(3.f, xx, -yy);
+    const float2 Y2[NHAR / 2] = {make_float2(1.f, x),
+                                 make_float2(y, z),
+                                 make_float2(xy, yz),
+                                 make_float2(xz, d),
+                                 make_float2(zz - (1.f / 3.f), z * fmaf(5.f, zz, -3.f)),
+                                 make_float2(x * q, y * q),
+                                 make_float2(z * d, xy * z),
+                                 make_float2(x * p14, y * p15)};
     float2 s0 = make_float2(0.f, 0.f), s1 = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int q = 0; q < NMOM / 2; q += 2) {
-        s0 = __ffma2_rn(W2[q], M2[q], s0);
-        s1 = __ffma2_rn(W2[q + 1], M2[q + 1], s1);
+    for (int t = 0; t < NHAR / 2; t += 2) {
+        s0 = __ffma2_rn(W2[t], Y2[t], s0);
+        s1 = __ffma2_rn(W2[t + 1], Y2[t + 1], s1);
     }
     const float dEdr = (s0.x + s0.y) + (s1.x + s1.y);
-    // F2 = V M': dE/du_y = sum_d V_d dM_d/du_y (M' formed on the fly)
-    const float xx = M2[2].x, xy = M2[2].y, xz = M2[3].x, yy = M2[3].y, yz = M2[4].x, zz = M2[4].y;
-    auto V = [&](int d) { return (d & 1) ? V2[d >> 1].y : V2[d >> 1].x; };
-    const float gx = V(1) + 2.f * ux * V(4) + uy * V(5) + uz * V(6) + 3.f * xx * V(10) +
-                     2.f * xy * V(11) + 2.f * xz * V(12) + yy * V(13) + yz * V(14) + zz * V(15);
-    const float gy = V(2) + ux * V(5) + 2.f * uy * V(7) + uz * V(8) + xx * V(11) + 2.f * xy * V(13) +
-                     xz * V(14) + 3.f * yy * V(16) + 2.f * yz * V(17) + zz * V(18);
-    const float gz = V(3) + ux * V(6) + uy * V(8) + 2.f * uz * V(9) + xx * V(12) + xy * V(14) +
-                     2.f * xz * V(15) + yy * V(17) + 2.f * yz * V(18) + 3.f * zz * V(19);
-    const float ug = ux * gx + uy * gy + uz * gz;
+    // F2 = V M': dE/du = sum_c V_c grad Y_c.  Only its part tangent to the
+    // sphere is used below, on which the gradients of the polynomials agree
+    // with those of any other form of the same functions on the sphere.
+    auto V = [&](int c) { return (c & 1) ? V2[c >> 1].y : V2[c >> 1].x; };
+    const float b = 3.f * d;
+    float gx = V(1) + y * V(4) + z * V(6) + q * V(10) + yz * V(13);
+    float gy = V(2) + x * V(4) + z * V(5) + q * V(11) + xz * V(13);
+    float gz = V(3) + y * V(5) + x * V(6) + 2.f * z * V(8) + fmaf(15.f, zz, -3.f) * V(9) + 10.f * xz * V(10) +
+               10.f * yz * V(11) + d * V(12) + xy * V(13);
+    gx += 2.f * x * (V(7) + z * V(12)) + b * V(14) + 6.f * xy * V(15);
+    gy += -2.f * y * (V(7) + z * V(12)) - 6.f * xy * V(14) + b * V(15);
+    const float ug = x * gx + y * gy + z * gz;
     // g_ij = dE/dD_ij = dE/dr u + (I - u u^T) dE/du / r
-    gxs = fmaf(dEdr, ux, (gx - ux * ug) * ir);
-    gys = fmaf(dEdr, uy, (gy - uy * ug) * ir);
-    gzs = fmaf(dEdr, uz, (gz - uz * ug) * ir);
+    gxs = fmaf(dEdr, x, (gx - x * ug) * ir);
+    gys = fmaf(dEdr, y, (gy - y * ug) * ir);
+    gzs = fmaf(dEdr, z, (gz - z * ug) * ir);
 }
 
 // g_ij = dE/dD_ij of one in-cutoff pair (Eqs. dP_abkd, U_abck, F1_abcx,
@@ -642,9 +653,9 @@ __device__ __forceinline__ void pair_grad(const DevModel &m, const float4 e, con
     // F1 = U H' R' = sum_d W_d M_d and F2 = V M'
     // V and W as packed pairs (d, d + 1): every multiply-add of the channel
     // loop is one FP32x2 instruction (each half rounded as fmaf)
-    float2 V2[NMOM / 2], W2[NMOM / 2];
+    float2 V2[NHAR / 2], W2[NHAR / 2];
 #pragma unroll
-    for (int d = 0; d < NMOM / 2; ++d) V2[d] = W2[d] = make_float2(0.f, 0.f);
+    for (int d = 0; d < NHAR / 2; ++d) V2[d] = W2[d] = make_float2(0.f, 0.f);
     float fc = 0.f, dfc = 0.f;
     TabCell tc;
     if (TAB)
@@ -673,8 +684,8 @@ __device__ __forceinline__ void pair_grad(const DevModel &m, const float4 e, con
         for (int c = 0; c < 2; ++c) {
             const float2 h2 = make_float2(Hk[c], Hk[c]), d2 = make_float2(dHk[c], dHk[c]);
 #pragma unroll
-            for (int q4 = 0; q4 < NMOM / 4; ++q4) {
-                const float4 pd = *reinterpret_cast<const float4 *>(Pb + (k + c) * NMOM + 4 * q4);
+            for (int q4 = 0; q4 < NHAR / 4; ++q4) {
+                const float4 pd = *reinterpret_cast<const float4 *>(Pb + (k + c) * NHAR + 4 * q4);
                 const float2 plo = make_float2(pd.x, pd.y), phi = make_float2(pd.z, pd.w);
                 V2[2 * q4] = __ffma2_rn(plo, h2, V2[2 * q4]);
                 V2[2 * q4 + 1] = __ffma2_rn(phi, h2, V2[2 * q4 + 1]);
@@ -687,16 +698,26 @@ __device__ __forceinline__ void pair_grad(const DevModel &m, const float4 e, con
 }
 
 
-// P'_bkd = 2 T_d sigma'_m P_bkd G'_bkm (for m = 0: G'_bk0 sign(P)) of the
-// atom at perm position p (P and G' are indexed by perm position) into a
-// shared slot, each lane its (K/8 x 5) block  (Eq. dP_abkd)
+// A'_bkc = dE/dA_bkc (Eq. dP_abkd) of the atom at perm position p (A and G'
+// are indexed by perm position) into a shared slot, each lane its (K/8 x 4)
+// block: 2 w_c A_c G'_m(c) with, from the parts that ranks 2 and 3 hold of the
+// lower degrees, G'_0 sign(A_0) + 2/3 G'_2 A_0 (c = 0) and G'_1 + 3/5 G'_3 in
+// the place of G'_1 (c = 1..3).
+__device__ __forceinline__ float4 aprime(const float4 A, const float4 gm, const float (&Wg)[4], int g) {
+    const float h0 = g == 1 || g == 2 ? gm.z : gm.w;                      // c = 4g
+    const float h = g == 0 ? fmaf(0.6f, gm.w, gm.y) : (g == 1 ? gm.z : gm.w);
+    float4 o = make_float4(2.f * Wg[0] * A.x * h0, 2.f * Wg[1] * A.y * h, 2.f * Wg[2] * A.z * h, 2.f * Wg[3] * A.w * h);
+    if (g == 0) o.x = fmaf(2.f / 3.f * gm.z, A.x, (A.x > 0.f) ? gm.x : ((A.x < 0.f) ? -gm.x : 0.f));
+    return o;
+}
+
 template <int K, int S>
-__device__ __forceinline__ void pprime_setup(const float *__restrict__ Pin, const float *__restrict__ dG, int p,
-                                             float *slot, int kg, int g, const float (&Tg)[5]) {
+__device__ __forceinline__ void pprime_setup(const float *__restrict__ Pin, const float *__restrict__ dG, int64_t p,
+                                             float *slot, int kg, int g, const float (&Wg)[4]) {
     constexpr int KPL = K / 8;
-    constexpr int PSTR = K * NMOM + 4;
+    constexpr int PSTR = K * NHAR + 4;
     constexpr int Dd = S * K * 4;
-    const float *Pa = Pin + (size_t)p * (S * K * NMOM);
+    const float *Pa = Pin + (size_t)p * (S * K * NHAR);
     const float *dGa = dG + (size_t)p * Dd;
 #pragma unroll
     for (int s = 0; s < S; ++s)
@@ -704,18 +725,8 @@ __device__ __forceinline__ void pprime_setup(const float *__restrict__ Pin, cons
         for (int kk = 0; kk < KPL; ++kk) {
             const int k = kg * KPL + kk;
             const float4 gm = *reinterpret_cast<const float4 *>(dGa + (s * K + k) * 4);
-#pragma unroll
-            for (int dd = 0; dd < 5; ++dd) {
-                const int d = 5 * g + dd;
-                const float pv = Pa[(s * K + k) * NMOM + d];
-                float gg;
-                if (g == 0) gg = (dd == 0) ? gm.x : ((dd < 4) ? gm.y : gm.z);
-                else gg = (g == 1) ? gm.z : gm.w;
-                float v;
-                if (g == 0 && dd == 0) v = (pv > 0.f) ? gg : ((pv < 0.f) ? -gg : 0.f);
-                else v = 2.f * Tg[dd] * pv * gg;
-                slot[s * PSTR + k * NMOM + d] = v;
-            }
+            const float4 A = *reinterpret_cast<const float4 *>(Pa + (s * K + k) * NHAR + 4 * g);
+            *reinterpret_cast<float4 *>(slot + s * PSTR + k * NHAR + 4 * g) = aprime(A, gm, Wg, g);
         }
 }
 
@@ -744,7 +755,7 @@ __global__ void __launch_bounds__(PW * 32, 4) k_force_merged(DevModel m, DevNlis
                                                           const float *__restrict__ Pin, const float *__restrict__ dG,
                                                           unsigned long long *__restrict__ Fq,
                                                           double *__restrict__ part_w) {
-    constexpr int PSTR = K * NMOM + 4;
+    constexpr int PSTR = K * NHAR + 4;
     __shared__ float4 s_rad[S * S * K];
     __shared__ __align__(16) float s_Pd[PW][2][S * PSTR];
     __shared__ double s_w[PW][9];
@@ -753,9 +764,9 @@ __global__ void __launch_bounds__(PW * 32, 4) k_force_merged(DevModel m, DevNlis
     if (lane < 9) s_w[warp][lane] = 0.0;
     __syncthreads();
     const int kg = lane >> 2, g = lane & 3;
-    float Tg[5];
+    float Wg[4];
 #pragma unroll
-    for (int dd = 0; dd < 5; ++dd) Tg[dd] = c_T[5 * g + dd];
+    for (int dd = 0; dd < 4; ++dd) Wg[dd] = c_W[4 * g + dd];
     // virial: each lane's pairs summed in FP32 over VFLUSH atoms, then the
     // warp's total added to an FP64 accumulator in shared memory
     float wacc[9];
@@ -769,7 +780,7 @@ __global__ void __launch_bounds__(PW * 32, 4) k_force_merged(DevModel m, DevNlis
     if (p < pend) {
         int slot = 0;
         int a = nl.perm[p], ta = types[a];
-        pprime_setup<K, S>(Pin, dG, (int)p, s_Pd[warp][0], kg, g, Tg);
+        pprime_setup<K, S>(Pin, dG, p, s_Pd[warp][0], kg, g, Wg);
         int64_t cb = nl.beg[a];
         int cr = nl.npair[a];
         long long fcx = 0, fcy = 0, fcz = 0;
@@ -781,7 +792,7 @@ __global__ void __launch_bounds__(PW * 32, 4) k_force_merged(DevModel m, DevNlis
             if (has_n) {   // bring in the next atom
                 an = nl.perm[p + 1];
                 tn = types[an];
-                pprime_setup<K, S>(Pin, dG, (int)p + 1, s_Pd[warp][slot ^ 1], kg, g, Tg);
+                pprime_setup<K, S>(Pin, dG, p + 1, s_Pd[warp][slot ^ 1], kg, g, Wg);
                 nb = nl.beg[an];
                 nr = nl.npair[an];
                 take_n = min(nr, 32 - cr);
@@ -845,7 +856,7 @@ __global__ void __launch_bounds__(PW * 32, 4) k_force_merged(DevModel m, DevNlis
                         __syncwarp();
                         a = nl.perm[p];
                         ta = types[a];
-                        pprime_setup<K, S>(Pin, dG, (int)p, s_Pd[warp][slot], kg, g, Tg);
+                        pprime_setup<K, S>(Pin, dG, p, s_Pd[warp][slot], kg, g, Wg);
                         cb = nl.beg[a];
                         cr = nl.npair[a];
                         fcx = fcy = fcz = 0;
@@ -872,7 +883,7 @@ __global__ void __launch_bounds__(PW * 32, 4) k_force_merged(DevModel m, DevNlis
 // pairs, columns = k) times P' (k x d).  Each warp takes its atom's cached
 // pairs 32 at a time: every lane forms H and H' of its pair into a shared
 // 64 x K tile (rows 0-31 H, rows 32-63 H'), the warp multiplies the tile by P'
-// with mma.sync m16n8k8 on TF32 operands (d padded to 24 with zeros), and
+// with mma.sync m16n8k8 on TF32 operands, and
 // every lane reads back the V and W rows of its pair for the rest of g_ij.
 // FP32 accuracy from TF32 products: each operand x is split into
 // x_hi = tf32(x) and x_lo = tf32(x - x_hi), and a product is accumulated as
@@ -901,8 +912,8 @@ __global__ void __launch_bounds__(PW * 32, 4) k_force_tc(DevModel m, DevNlist nl
     static_assert(K % 8 == 0 && K <= 32, "k steps of 8, one pass");
     constexpr int KS = K / 8;        // k steps of the product
     constexpr int AS = K + 4;        // row stride of the H / H' tile (conflict-free fragment loads)
-    constexpr int CS = 28;           // row stride of the V / W tile (24 columns, 16-byte rows)
-    constexpr int PSTR = K * NMOM + 4;
+    constexpr int CS = 20;           // row stride of the V / W tile (16 columns, 16-byte rows)
+    constexpr int PSTR = K * NHAR + 4;
     // the V / W tile is written over the H / H' tile, one m tile at a time,
     // in descending order when its rows are longer (CS > AS) and ascending
     // otherwise: the words a tile's results land on then hold only H / H'
@@ -917,9 +928,9 @@ __global__ void __launch_bounds__(PW * 32, 4) k_force_tc(DevModel m, DevNlist nl
     __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int kg = lane >> 2, g = lane & 3;   // P' setup block; also the fragment row / column group
-    float Tg[5];
+    float Wg[4];
 #pragma unroll
-    for (int dd = 0; dd < 5; ++dd) Tg[dd] = c_T[5 * g + dd];
+    for (int dd = 0; dd < 4; ++dd) Wg[dd] = c_W[4 * g + dd];
     float wsum[9], wcmp[9];
 #pragma unroll
     for (int t = 0; t < 9; ++t) { wsum[t] = 0.f; wcmp[t] = 0.f; }
@@ -928,18 +939,18 @@ __global__ void __launch_bounds__(PW * 32, 4) k_force_tc(DevModel m, DevNlist nl
     const int64_t total = (int64_t)gridDim.x * PW;
     for (int64_t p = (int64_t)blockIdx.x * PW + warp; p < nl.n; p += total) {
         const int a = nl.perm[p];
-        pprime_setup<K, 1>(Pin, dG, (int)p, sPd, kg, g, Tg);
+        pprime_setup<K, 1>(Pin, dG, p, sPd, kg, g, Wg);
         __syncwarp();
         // B fragments of P' (k x 24), hi and lo parts: b0 = (k = t, n = g), b1 = (k = t + 4, n = g)
-        uint32_t bh[KS][3][2], bl[KS][3][2];
+        uint32_t bh[KS][2][2], bl[KS][2][2];
 #pragma unroll
         for (int ks = 0; ks < KS; ++ks)
 #pragma unroll
-            for (int nt = 0; nt < 3; ++nt)
+            for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const int k = ks * 8 + g + 4 * h, d = nt * 8 + kg;
-                    split_tf32(d < NMOM ? sPd[k * NMOM + d] : 0.f, bh[ks][nt][h], bl[ks][nt][h]);
+                    split_tf32(sPd[k * NHAR + d], bh[ks][nt][h], bl[ks][nt][h]);
                 }
         const int np = nl.npair[a];
         const int64_t pb = nl.beg[a];
@@ -986,9 +997,9 @@ __global__ void __launch_bounds__(PW * 32, 4) k_force_tc(DevModel m, DevNlist nl
             for (int i = 0; i < 4; ++i) {
                 const int mt = ASCENDING ? i : 3 - i;
                 if ((mt & 1) >= mt_used) continue;
-                float c[3][4];
+                float c[2][4];
 #pragma unroll
-                for (int nt = 0; nt < 3; ++nt)
+                for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
                     for (int q = 0; q < 4; ++q) c[nt][q] = 0.f;
 #pragma unroll
@@ -1001,7 +1012,7 @@ __global__ void __launch_bounds__(PW * 32, 4) k_force_tc(DevModel m, DevNlist nl
                     split_tf32(r0[4], ah[2], al[2]);
                     split_tf32(r1[4], ah[3], al[3]);
 #pragma unroll
-                    for (int nt = 0; nt < 3; ++nt) {
+                    for (int nt = 0; nt < 2; ++nt) {
                         mma_tf32(c[nt], al, bh[ks][nt][0], bh[ks][nt][1]);
                         mma_tf32(c[nt], ah, bl[ks][nt][0], bl[ks][nt][1]);
                         mma_tf32(c[nt], ah, bh[ks][nt][0], bh[ks][nt][1]);
@@ -1009,7 +1020,7 @@ __global__ void __launch_bounds__(PW * 32, 4) k_force_tc(DevModel m, DevNlist nl
                 }
                 __syncwarp();   // every lane's fragment loads of this tile precede the stores below
 #pragma unroll
-                for (int nt = 0; nt < 3; ++nt) {
+                for (int nt = 0; nt < 2; ++nt) {
                     float *c0 = sT + (mt * 16 + kg) * CS + nt * 8 + 2 * g;
                     *reinterpret_cast<float2 *>(c0) = make_float2(c[nt][0], c[nt][1]);
                     *reinterpret_cast<float2 *>(c0 + 8 * CS) = make_float2(c[nt][2], c[nt][3]);
@@ -1017,10 +1028,10 @@ __global__ void __launch_bounds__(PW * 32, 4) k_force_tc(DevModel m, DevNlist nl
                 __syncwarp();
             }
             if (valid) {
-                float2 V2[NMOM / 2], W2[NMOM / 2];
+                float2 V2[NHAR / 2], W2[NHAR / 2];
                 const float *vr = sT + lane * CS, *wr = sT + (32 + lane) * CS;
 #pragma unroll
-                for (int q4 = 0; q4 < NMOM / 4; ++q4) {
+                for (int q4 = 0; q4 < NHAR / 4; ++q4) {
                     const float4 v = *reinterpret_cast<const float4 *>(vr + 4 * q4);
                     const float4 w = *reinterpret_cast<const float4 *>(wr + 4 * q4);
                     V2[2 * q4] = make_float2(v.x, v.y); V2[2 * q4 + 1] = make_float2(v.z, v.w);
@@ -1090,7 +1101,7 @@ __global__ void __launch_bounds__(PW * 32, 4) k_force(DevModel m, DevNlist nl, c
                                                    unsigned long long *__restrict__ Fq,
                                                    double *__restrict__ part_w, float *__restrict__ w_atom) {
     constexpr int KPL = K / 8;
-    constexpr int PSTR = K * NMOM + 4;   // per-species stride of P' (bank offset between species)
+    constexpr int PSTR = K * NHAR + 4;   // per-species stride of P' (bank offset between species)
     constexpr int Dd = S * K * 4;
     __shared__ float4 s_rad[S * S * K];
     __shared__ float4 s_q[PW][64];
@@ -1101,9 +1112,9 @@ __global__ void __launch_bounds__(PW * 32, 4) k_force(DevModel m, DevNlist nl, c
     __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int kg = lane >> 2, g = lane & 3;
-    float Tg[5];
+    float Wg[4];
 #pragma unroll
-    for (int dd = 0; dd < 5; ++dd) Tg[dd] = c_T[5 * g + dd];
+    for (int dd = 0; dd < 4; ++dd) Wg[dd] = c_W[4 * g + dd];
     float wsum[9], wcmp[9];
 #pragma unroll
     for (int t = 0; t < 9; ++t) { wsum[t] = 0.f; wcmp[t] = 0.f; }
@@ -1112,29 +1123,7 @@ __global__ void __launch_bounds__(PW * 32, 4) k_force(DevModel m, DevNlist nl, c
     for (int64_t p = (int64_t)blockIdx.x * PW + warp; p < nl.n; p += total) {
         const int a = nl.perm[p];
         const int ti = types[a];
-        // P'_bkd = 2 T_d sigma'_m P_bkd G'_bkm; for m = 0: G'_bk0 sign(P)  (Eq. dP_abkd)
-        const float *Pa = Pin + (size_t)p * (S * K * NMOM);
-        const float *dGa = dG + (size_t)p * Dd;
-#pragma unroll
-        for (int s = 0; s < S; ++s)
-#pragma unroll
-            for (int kk = 0; kk < KPL; ++kk) {
-                const int k = kg * KPL + kk;
-                const float4 gm = *reinterpret_cast<const float4 *>(dGa + (s * K + k) * 4);
-#pragma unroll
-                for (int dd = 0; dd < 5; ++dd) {
-                    const int d = 5 * g + dd;
-                    const float pv = Pa[(s * K + k) * NMOM + d];
-                    // rank of d: g==0 -> {0,1,1,1,2}, g==1 -> 2, g>=2 -> 3
-                    float gg;
-                    if (g == 0) gg = (dd == 0) ? gm.x : ((dd < 4) ? gm.y : gm.z);
-                    else gg = (g == 1) ? gm.z : gm.w;
-                    float v;
-                    if (g == 0 && dd == 0) v = (pv > 0.f) ? gg : ((pv < 0.f) ? -gg : 0.f);
-                    else v = 2.f * Tg[dd] * pv * gg;
-                    sPd[s * PSTR + k * NMOM + d] = v;
-                }
-            }
+        pprime_setup<K, S>(Pin, dG, p, sPd, kg, g, Wg);
         __syncwarp();
         long long fx = 0, fy = 0, fz = 0;
         float wa[9];  // this lane's pairs of this atom

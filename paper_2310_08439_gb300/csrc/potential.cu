@@ -1356,7 +1356,7 @@ tmd_status reserve_compute(const DevModel &dm, tmd_nlist *nl, int64_t n_total, i
     const int64_t nt = std::max<int64_t>(n_total, 1), na = std::max<int64_t>(n_active, 1);
     if ((st = grow(&nl->G, &nl->cap_G, na * dm.Dd)) != TMD_OK) return st;
     if ((st = grow(&nl->dG, &nl->cap_dG, na * dm.Dd)) != TMD_OK) return st;
-    if ((st = grow(&nl->P, &nl->cap_P, na * dm.S * dm.K * NMOM)) != TMD_OK) return st;
+    if ((st = grow(&nl->P, &nl->cap_P, na * dm.S * dm.K * NHAR)) != TMD_OK) return st;
     if ((st = grow(&nl->Fq, &nl->cap_Fq, 3 * nt)) != TMD_OK) return st;
     if ((st = grow(&nl->ph, &nl->cap_ph, nt)) != TMD_OK) return st;
     if ((st = grow(&nl->pl, &nl->cap_pl, nt)) != TMD_OK) return st;
@@ -1388,7 +1388,7 @@ tmd_status run_descriptors(const tmd_model *model, tmd_nlist *nl, const double *
     if (st != TMD_OK) return st;
     if (n == 0) return TMD_OK;
     const DevModel &dm = model->dm;
-    if ((st = grow(&nl->P, &nl->cap_P, n * dm.S * dm.K * NMOM)) != TMD_OK) return st;
+    if ((st = grow(&nl->P, &nl->cap_P, n * dm.S * dm.K * NHAR)) != TMD_OK) return st;
     if ((st = grow(&nl->G, &nl->cap_G, n * dm.Dd)) != TMD_OK) return st;
     if (dEdG && (st = grow(&nl->dG, &nl->cap_dG, n * dm.Dd)) != TMD_OK) return st;
     const int nblk = pair_blocks(dm, n);
@@ -1424,7 +1424,7 @@ tmd_status run_compute(const tmd_model *model, tmd_nlist *nl, const double *pos,
     const int64_t Dd = dm.Dd;
     if ((st = grow(&nl->G, &nl->cap_G, n * Dd)) != TMD_OK) return st;
     if ((st = grow(&nl->dG, &nl->cap_dG, n * Dd)) != TMD_OK) return st;
-    if ((st = grow(&nl->P, &nl->cap_P, n * dm.S * dm.K * NMOM)) != TMD_OK) return st;
+    if ((st = grow(&nl->P, &nl->cap_P, n * dm.S * dm.K * NHAR)) != TMD_OK) return st;
     if ((st = grow(&nl->Fq, &nl->cap_Fq, 3 * n)) != TMD_OK) return st;
     const int nblk = pair_blocks(dm, n);
     const int ntile = (int)((n + MT - 1) / MT);
@@ -1605,7 +1605,7 @@ tmd_status noalloc_capacity(const tmd_model *model, int64_t n, size_t *need) {
     size_t b = 0;
     b += al(sizeof(int32_t) * n);                              // identity order
     b += 2 * al(sizeof(float4) * n);                           // positions hi / lo
-    b += al(sizeof(float) * n * dm.S * dm.K * NMOM);           // P
+    b += al(sizeof(float) * n * dm.S * dm.K * NMOM);           // P (with room for NMOM components: the documented limit)
     b += 2 * al(sizeof(float) * n * dm.Dd);                    // G, G'
     b += al(sizeof(unsigned long long) * 3 * n);               // force accumulator
     b += al(sizeof(double) * (ntile + 9 * nblk + 16 + RED_PART));         // block partials
@@ -1681,7 +1681,7 @@ tmd_status run_compute_noalloc(const tmd_model *model, const int64_t *off, const
     w.perm = static_cast<int32_t *>(take(sizeof(int32_t) * n));
     w.ph = static_cast<float4 *>(take(sizeof(float4) * n));
     w.pl = static_cast<float4 *>(take(sizeof(float4) * n));
-    w.P = static_cast<float *>(take(sizeof(float) * n * dm.S * dm.K * NMOM));
+    w.P = static_cast<float *>(take(sizeof(float) * n * dm.S * dm.K * NHAR));
     w.G = static_cast<float *>(take(sizeof(float) * n * dm.Dd));
     w.dG = static_cast<float *>(take(sizeof(float) * n * dm.Dd));
     w.Fq = static_cast<unsigned long long *>(take(sizeof(unsigned long long) * 3 * n));
@@ -1770,7 +1770,7 @@ tmd_status run_compute_batch(const tmd_model *model, tmd_nlist *nl, const double
         // P, G and G' are indexed by perm position: room for the active atoms only
         if ((st = grow(&nl->G, &nl->cap_G, na * dm.Dd)) != TMD_OK) return st;
         if ((st = grow(&nl->dG, &nl->cap_dG, na * dm.Dd)) != TMD_OK) return st;
-        if ((st = grow(&nl->P, &nl->cap_P, na * dm.S * dm.K * NMOM)) != TMD_OK) return st;
+        if ((st = grow(&nl->P, &nl->cap_P, na * dm.S * dm.K * NHAR)) != TMD_OK) return st;
         if ((st = grow(&nl->Fq, &nl->cap_Fq, 3 * n_total)) != TMD_OK) return st;
         const int nblk = pair_blocks(dm, na);
         const int ntile = (int)((na + MT - 1) / MT);

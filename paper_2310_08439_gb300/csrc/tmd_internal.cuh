@@ -13,6 +13,7 @@
 namespace tmd {
 
 constexpr int NMOM = 20;        // moment components d, ranks 0..3 (Eq. T_dm)
+constexpr int NHAR = 16;        // independent components of the moments on the unit sphere (pair_kernels.cuh)
 constexpr int WARP = 32;
 constexpr int MAX_LAYERS = TMD_MAX_HIDDEN + 1;
 
@@ -173,7 +174,7 @@ struct tmd_nlist {
     // compute workspace
     float *G = nullptr;       int64_t cap_G = 0;    // [n][Dd]
     float *dG = nullptr;      int64_t cap_dG = 0;   // [n][Dd]
-    float *P = nullptr;       int64_t cap_P = 0;    // [n][S][K][20]
+    float *P = nullptr;       int64_t cap_P = 0;    // [n][S][K][NHAR]
     unsigned long long *Fq = nullptr; int64_t cap_Fq = 0; // [n][3] forces, 2^-32 fixed point
     float4 *ph = nullptr;     int64_t cap_ph = 0;   // [n] positions hi
     float4 *pl = nullptr;     int64_t cap_pl = 0;   // [n] positions lo
