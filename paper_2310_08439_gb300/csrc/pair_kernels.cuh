@@ -33,6 +33,8 @@
 // pair_k<K>.cu translation unit instantiates one K (compiled in parallel).
 #pragma once
 
+#include <algorithm>
+
 #include "tmd_internal.cuh"
 
 namespace tmd {
@@ -55,6 +57,22 @@ __device__ __forceinline__ void harmonics16(float x, float y, float z, float *Y)
     Y[8] = zz - (1.f / 3.f);
     Y[9] = z * fmaf(5.f, zz, -3.f); Y[10] = x * q; Y[11] = y * q;
     Y[12] = z * d; Y[13] = Y[4] * z; Y[14] = x * fmaf(-3.f, yy, xx); Y[15] = y * fmaf(3.f, xx, -yy);
+}
+
+__device__ __forceinline__ float2 bc2(float x) { return make_float2(x, x); }
+
+// harmonics16 of two vectors (packed FP32x2)
+__device__ __forceinline__ void harmonics16x2(float2 x, float2 y, float2 z, float2 *Y) {
+    const float2 xx = __fmul2_rn(x, x), yy = __fmul2_rn(y, y), zz = __fmul2_rn(z, z);
+    const float2 d = __ffma2_rn(yy, bc2(-1.f), xx), q = __ffma2_rn(zz, bc2(5.f), bc2(-1.f));
+    Y[0] = bc2(1.f);
+    Y[1] = x; Y[2] = y; Y[3] = z;
+    Y[4] = __fmul2_rn(x, y); Y[5] = __fmul2_rn(y, z); Y[6] = __fmul2_rn(x, z); Y[7] = d;
+    Y[8] = __fadd2_rn(zz, bc2(-1.f / 3.f));
+    Y[9] = __fmul2_rn(z, __fadd2_rn(q, bc2(-2.f))); Y[10] = __fmul2_rn(x, q); Y[11] = __fmul2_rn(y, q);
+    Y[12] = __fmul2_rn(z, d); Y[13] = __fmul2_rn(Y[4], z);
+    Y[14] = __fmul2_rn(x, __ffma2_rn(yy, bc2(-3.f), xx));
+    Y[15] = __fmul2_rn(y, __ffma2_rn(xx, bc2(3.f), __fmul2_rn(yy, bc2(-1.f))));
 }
 
 // 2^x and 1/sqrt(x) from the special-function unit (PTX ex2.approx /
@@ -189,6 +207,26 @@ __device__ __forceinline__ void split_sqrt(float r2_hi, float r2_lo, float &r_hi
     ir = fmaf(y, e, y);
 }
 
+// split_sqrt and f_c (cutoff_fn) of two pairs (packed FP32x2)
+__device__ __forceinline__ void split_sqrt2(float2 r2h, float2 r2l, float2 &r_hi, float2 &r_lo, float2 &ir) {
+    const float2 y = make_float2(rsqrt_ftz(r2h.x), rsqrt_ftz(r2h.y));
+    r_hi = __fmul2_rn(r2h, y);
+    const float2 nr = __fmul2_rn(r_hi, bc2(-1.f));
+    r_lo = __fmul2_rn(__fadd2_rn(__ffma2_rn(nr, r_hi, r2h), r2l), __fmul2_rn(y, bc2(0.5f)));
+    const float2 e = __ffma2_rn(__fmul2_rn(r_lo, bc2(-1.f)), y, __ffma2_rn(nr, y, bc2(1.f)));
+    ir = __ffma2_rn(y, e, y);
+}
+__device__ __forceinline__ float2 cutoff2(float2 r, float inv_rc) {
+    const float2 y = __fmul2_rn(bc2(PI_F), __ffma2_rn(r, bc2(inv_rc), bc2(-0.5f))), u = __fmul2_rn(y, y);
+    float2 p = bc2(1.f / 6227020800.f);
+    p = __ffma2_rn(p, u, bc2(-1.f / 39916800.f));
+    p = __ffma2_rn(p, u, bc2(1.f / 362880.f));
+    p = __ffma2_rn(p, u, bc2(-1.f / 5040.f));
+    p = __ffma2_rn(p, u, bc2(1.f / 120.f));
+    p = __ffma2_rn(p, u, bc2(-1.f / 6.f));
+    return __ffma2_rn(__ffma2_rn(__fmul2_rn(y, u), p, y), bc2(-0.5f), bc2(0.5f));
+}
+
 // Double-float helpers: a value is carried as an unevaluated sum hi + lo of two
 // floats.  two_sum is Knuth's error-free addition.
 __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
@@ -250,17 +288,21 @@ __device__ __forceinline__ void pair_geom(const float4 jh, const float4 jl, cons
 // The queue holds (Dx, Dy, Dz, j | b<<28) rounded to FP32 and r^2 as hi/lo.
 // Used when there is no pair cache (k_screen in screen.cu fills the cache
 // with the same pairs, in the same order, by the same arithmetic).
-template <typename F>
-__device__ __forceinline__ int for_pairs(const DevNlist &nl, int a, int64_t beg, int64_t end, float rc2h, float rc2l,
-                                         float4 *q, float2 *q2, int lane, F &&f) {
-    int qn = 0, kept = 0;
+//
+// f(q, q2, nb) takes the first nb pairs of the queue (nb = 32 NL but for the
+// atom's last batch).
+template <int NL, typename F>
+__device__ __forceinline__ void queue_pairs(const DevNlist &nl, int a, int64_t beg, int64_t end, float rc2h, float rc2l,
+                                            float4 *q, float2 *q2, int lane, F &&f) {
+    constexpr int NB = 32 * NL;
+    int qn = 0;
     const unsigned lt = (1u << lane) - 1u;
     const float4 ih = nl.ph[a], il = nl.pl[a];
     float Lh[3], Ll[3];
     pair_box(nl, a, Lh, Ll);
     int64_t base = beg;
     while (true) {
-        while (qn < 32 && base < end) {
+        while (qn < NB && base < end) {
             const int64_t c = base + lane;
             bool v = false;
             float4 e = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -282,23 +324,29 @@ __device__ __forceinline__ int for_pairs(const DevNlist &nl, int a, int64_t beg,
                 q2[slot] = e2;
             }
             qn += __popc(m);
-            kept += __popc(m);
             base += 32;
         }
         if (qn == 0) break;
         // one call site: full batches while entries remain, then the tail
-        const int nb = min(qn, 32);
+        const int nb = min(qn, NB);
         __syncwarp();
-        f(q[lane], q2[lane], lane < nb, nb);
+        f(q, q2, nb);
         __syncwarp();
         if (lane < qn - nb) {
-            q[lane] = q[lane + 32];
-            q2[lane] = q2[lane + 32];
+            q[lane] = q[lane + NB];
+            q2[lane] = q2[lane + NB];
         }
         __syncwarp();
         qn -= nb;
     }
-    return kept;
+}
+
+// the same, one pair per lane: f(pair, r^2, valid, nb)
+template <typename F>
+__device__ __forceinline__ void for_pairs(const DevNlist &nl, int a, int64_t beg, int64_t end, float rc2h, float rc2l,
+                                          float4 *q, float2 *q2, int lane, F &&f) {
+    queue_pairs<1>(nl, a, beg, end, rc2h, rc2l, q, q2, lane,
+                   [&](const float4 *p, const float2 *p2, int nb) { f(p[lane], p2[lane], lane < nb, nb); });
 }
 
 // The in-cutoff pairs of atom a from the pair cache written by k_screen, in
@@ -318,56 +366,71 @@ __device__ __forceinline__ void cached_pairs(const DevNlist &nl, int a, int np, 
     }
 }
 
-// A warp's stream of pair-cache batches over its atoms p, p + total, ...
-// (perm order), read one batch ahead.
+// Two neighbouring pairs of a lane (pairs 2 lane and 2 lane + 1 of a batch of 64).
+struct PairTwo {
+    float4 e0, e1;
+    float2 q0, q1;
+};
+// pairs i and i + 1 of the n >= 1 at p, p2 (the last pair again past the end)
+__device__ __forceinline__ PairTwo load_two(const float4 *p, const float2 *p2, int i, int n) {
+    const int i0 = min(i, n - 1), i1 = min(i + 1, n - 1);
+    PairTwo t;
+    t.e0 = p[i0];
+    t.e1 = p[i1];
+    t.q0 = p2[i0];
+    t.q1 = p2[i1];
+    return t;
+}
+
+// A warp's stream of pair-cache batches (64 pairs, two per lane) over its atoms
+// p, p + total, ... (perm order), read one batch ahead.
 struct PairStream {
     int a = -1, np = 0;          // current atom and its in-cutoff pair count
     int64_t pb = 0;
     int an = -1, npn = 0;        // next atom (segment start and count read one atom ahead)
     int64_t pbn = 0;
     int an2 = -1;                // the atom after next (perm entry read two atoms ahead)
-    float4 pf = make_float4(0.f, 0.f, 0.f, 0.f);
-    float2 pf2 = make_float2(1.f, 0.f);
+    int ty = 0, tyn = 0;         // species of the current and the next atom (0 unless asked for)
+    PairTwo pf;                  // the batch that is taken next
 
-    __device__ __forceinline__ void load(const DevNlist &nl, int64_t at, bool ok) {
-        pf = make_float4(0.f, 0.f, 0.f, 0.f);
-        pf2 = make_float2(1.f, 0.f);
-        if (ok) {
-            pf = nl.pq[at];
-            pf2 = nl.pq2[at];
-        }
+    __device__ __forceinline__ void load(const DevNlist &nl, int64_t at, int n, int lane) {
+        if (n > 0) pf = load_two(nl.pq + at, nl.pq2 + at, 2 * lane, n);
     }
-    __device__ __forceinline__ void start(const DevNlist &nl, int64_t p, int64_t total, int lane) {
+    __device__ __forceinline__ void start(const DevNlist &nl, const int32_t *types, int64_t p, int64_t total, int lane) {
+        pf.e0 = pf.e1 = make_float4(1.f, 0.f, 0.f, 0.f);
+        pf.q0 = pf.q1 = make_float2(1.f, 0.f);
         if (p < nl.n) {
             a = nl.perm[p];
+            if (types) ty = types[a];
             pb = nl.beg[a];
             np = nl.npair[a];
-            load(nl, pb + lane, lane < np);
+            load(nl, pb, np, lane);
         }
         an = p + total < nl.n ? nl.perm[p + total] : -1;
     }
     // at the start of atom p: the next atom's segment, the perm entry after it
-    __device__ __forceinline__ void atom_begins(const DevNlist &nl, int64_t p, int64_t total) {
+    __device__ __forceinline__ void atom_begins(const DevNlist &nl, const int32_t *types, int64_t p, int64_t total) {
+        npn = 0;
         if (an >= 0) {
+            if (types) tyn = types[an];
             pbn = nl.beg[an];
             npn = nl.npair[an];
         }
         an2 = p + 2 * total < nl.n ? nl.perm[p + 2 * total] : -1;
     }
-    // the batch after the one starting at base: the atom's next batch, its
-    // first batch again (another channel chunk follows), or the next atom's first
-    __device__ __forceinline__ void advance(const DevNlist &nl, int base, bool again, int lane) {
-        if (base + 32 < np)
-            load(nl, pb + base + 32 + lane, lane < np - base - 32);
-        else if (again)
-            load(nl, pb + lane, lane < np);
+    // the batch after the one starting at base: the atom's next batch, or the
+    // next atom's first
+    __device__ __forceinline__ void advance(const DevNlist &nl, int base, int lane) {
+        if (base + 64 < np)
+            load(nl, pb + base + 64, np - base - 64, lane);
         else
-            load(nl, pbn + lane, an >= 0 && lane < npn);
+            load(nl, pbn, npn, lane);
     }
     __device__ __forceinline__ void atom_ends() {
         a = an;
+        ty = tyn;
         pb = pbn;
-        np = an >= 0 ? npn : 0;
+        np = npn;
         an = an2;
     }
 };
@@ -392,171 +455,298 @@ __device__ __forceinline__ float desc_value(const float (&A)[4], const float (&W
 // ---------------------------------------------------------------------------
 // descriptor forward: A and G per atom
 // ---------------------------------------------------------------------------
+__device__ __forceinline__ void split_tf32(float x, uint32_t &hi, uint32_t &lo) {
+    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(hi) : "f"(x));
+    const float rest = x - __uint_as_float(hi);   // exact
+    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(lo) : "f"(rest));
+}
+
+// c += a b for one m16n8k8 tile (a: 16 x 8 row-major, b: 8 x 8, c: 16 x 8)
+__device__ __forceinline__ void mma_tf32(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+        "{%0, %1, %2, %3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// c = a b for one m16n8k8 tile
+__device__ __forceinline__ void mma_tf32_first(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+        "{%10, %10, %10, %10};"
+        : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
+}
+
+// Two values as operands of a split product: x_h = x rounded to TF32 (11
+// significant bits, ties away) and x_l = x - x_h (exact, 12 bits or fewer), of
+// which the tensor cores read the TF32 part, dropping at most the last bit of
+// x.  Integer operations: the conversion cvt.rna.tf32 issues at the rate of
+// the special functions and made it the bound of the descriptor pass.
+struct Split2 {
+    uint32_t h0, h1, l0, l1;
+};
+
+__device__ __forceinline__ Split2 split2(const float2 x) {
+    Split2 o;
+    o.h0 = (__float_as_uint(x.x) + 0x1000u) & 0xffffe000u;
+    o.h1 = (__float_as_uint(x.y) + 0x1000u) & 0xffffe000u;
+    const float2 r = __ffma2_rn(make_float2(__uint_as_float(o.h0), __uint_as_float(o.h1)), make_float2(-1.f, -1.f), x);
+    o.l0 = __float_as_uint(r.x);
+    o.l1 = __float_as_uint(r.y);
+    return o;
+}
+
+// The contraction A[k][c] = sum_j H_jk Y_jc of one atom is a K x 16 product
+// over its pairs, run on the tensor cores (mma.sync) 8 pairs at a time: rows =
+// 16 channels, columns = the 16 components in two tiles of 8.  Every lane forms
+// the H of its own operand elements (two channels, two pairs of the 8), so H
+// is never staged; r, f_c and the 16 harmonics of a pair are formed once, by
+// the lane that holds the pair, and staged in shared memory, one row per
+// quantity and one column per pair.
+//
+// FP32 accuracy from split operands: x = x_h + x_l + O(2^-23 x), both parts
+// TF32, and x y = x_l y_h + x_h y_l + x_h y_h (the products are exact in FP32).
+// The tensor cores truncate as they accumulate: the sums of 8 pairs therefore
+// start from zero, small terms first, and are added to the totals in FP32,
+// times 1 + 2^-23.  That factor makes up for the truncated parts, which are
+// lost from the magnitude of each such sum (twice half a unit in its last place
+// on average): without it G is 1.8e-7 too small on average, with it 1e-8 (rms
+// error of G 2.0e-7 and 1.4e-7; the FP32 sums before: 1.3e-7 and 1.6e-7).
+//
+// A lane stages two pairs (2 l, 2 l + 1 of a batch of 64) on packed FP32x2
+// arithmetic, so that most atoms need one batch.
+//
+// What bounds it: instruction issue (61 % of the slots; 760 warp instructions
+// per atom at 53 pairs and K = 16; FMA pipe 41 %, ALU 35 %, tensor 27 %).  The
+// pass before it (packed FP32 multiply-adds on a (K/8 x 4) block per lane)
+// staged H as well, read 6 shared float4 per 16 multiply-add instructions and
+// waited on shared memory.  1,048,576 atoms, K = 16: 1.60 -> 1.02 ms; 148,176
+// atoms, K = 32: 0.356 -> 0.285; 39,366 atoms, K = 128: 0.487 -> 0.338 ms.
+//
 // CACHED: the atom's in-cutoff pairs come from the pair cache filled by
-// k_screen; otherwise the pass screens the table itself (for_pairs).  K > 32
-// runs in chunks of 32 channels, each chunk going over the atom's pairs again,
-// so that the per-lane accumulators and the staged columns stay those of
-// K = 32.
+// k_screen; otherwise the pass screens the table itself (for_pairs).
+// Blocks per SM asked for (registers): measured 7 of 5 .. 10 at K = 16, S = 1
+// (1.02 ms for 1M atoms; 5 blocks 1.20, 9 blocks 1.17), 5 at K = 32 (0.285 ms
+// for 148,176 atoms; without a bound 0.290, 6 blocks 0.308) and at K = 16, S = 3
+// (0.369 against 0.399 and 0.480); the totals of larger S K leave no choice.
+constexpr int desc_min_blocks(int sk) { return sk <= 16 ? 7 : (sk <= 48 ? 5 : 1); }
+
 template <int K, int S, bool TAB, bool CACHED>
-__global__ void __launch_bounds__(PW * 32) k_desc(DevModel m, DevNlist nl, const double *__restrict__ pos,
+__global__ void __launch_bounds__(PW * 32, desc_min_blocks(S * K)) k_desc(DevModel m, DevNlist nl, const double *__restrict__ pos,
                                                   const int32_t *__restrict__ types, float *__restrict__ G,
                                                   float *__restrict__ Pout) {
-    constexpr int KC = K > 32 ? 32 : K;   // channels per chunk
-    constexpr int KPL = KC / 8;           // k values per lane
-    constexpr int RS = 44;       // row stride of the staged pair columns (>= 32 + 3 (S - 1) slots)
+    constexpr int MT = (K + 15) / 16;     // tiles of 16 channels
+    constexpr int NC = K < 16 ? 1 : 2;    // channels of a lane per tile (rows g and g + 8)
+    // slots of a batch of 64 pairs: groups of the neighbour species, each a
+    // multiple of 8; row stride 8 mod 32 so that the float2 operand reads are
+    // conflict-free
+    constexpr int RS = S <= 2 ? 72 : 104;
     constexpr int Dd = S * K * 4;
-    __shared__ float4 s_rad2[S * S * K];
-    __shared__ float4 s_q[PW][64];
-    __shared__ float2 s_q2[PW][64];
-    // staged pair data, one column per pair: H_k in row (k % KPL) 8 + k / KPL,
-    // Y_c in row (c % 4) 4 + c / 4, so that the lane owning k-group kg and
-    // component group g reads four pairs of a row with one conflict-free vector load
-    __shared__ __align__(16) float s_H[PW][KC * RS];
-    __shared__ __align__(16) float s_M[PW][NHAR * RS];
-    stage_rad2(s_rad2, m.radial, S * S * K);
-    __syncthreads();
+    constexpr bool HOIST = MT <= 2;       // channel parameters in registers (per species group)
+    const float2 untrunc = bc2(1.00000012f);   // 1 + 2^-23
+    constexpr bool RSH = S * S * K <= 512;   // the channel parameters fit beside the staging
+    __shared__ float4 s_rad[RSH ? S * S * K : 1];   // (-mu_hi, -mu_lo, -eta log2 e, 0)
+    __shared__ float4 s_q[CACHED ? 1 : PW][CACHED ? 1 : 96];
+    __shared__ float2 s_q2[CACHED ? 1 : PW][CACHED ? 1 : 96];
+    // rows: r_hi, r_lo, f_c (TAB: t, interval, 1), then component c in row
+    // 3 + 8 ((c >> 1) & 1) + 2 (c >> 2) + (c & 1): operand column n of tile i
+    // is component 4 (n >> 1) + 2 i + (n & 1), which leaves the lane t of a
+    // quad with components 4t .. 4t + 3 of its channels
+    __shared__ __align__(16) float s_st[PW][(3 + NHAR) * RS];
+    if constexpr (RSH)
+        for (int i = threadIdx.x; i < S * S * K; i += blockDim.x) {
+            const float4 a = m.radial[i];
+            s_rad[i] = make_float4(-a.x, -a.y, -a.z, 0.f);
+        }
+    auto channel = [&](int i) {
+        if constexpr (RSH) return s_rad[i];
+        const float4 a = __ldg(m.radial + i);
+        return make_float4(-a.x, -a.y, -a.z, 0.f);
+    };
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int kg = lane >> 2, g = lane & 3;
+    const int g = lane >> 2, t = lane & 3;   // operand row (channel) / column (pairs 2t, 2t + 1)
     const unsigned lt = (1u << lane) - 1u;
-    float Wg[4];
+    float *const st = s_st[warp];
+    // unused slots hold f_c = 0 and finite values; component 0 is 1
+    for (int i = lane; i < (3 + NHAR) * RS; i += 32) st[i] = (i / RS == 3) ? 1.f : 0.f;
+    __syncthreads();
+    float Wt[4];
 #pragma unroll
-    for (int dd = 0; dd < 4; ++dd) Wg[dd] = c_W[4 * g + dd];
+    for (int dd = 0; dd < 4; ++dd) Wt[dd] = c_W[4 * t + dd];
     const int64_t total = (int64_t)gridDim.x * PW;
-    // CACHED: the pair-cache batches are read one batch ahead, across chunk
-    // and atom boundaries (the next atom's segment one atom ahead, its perm
-    // entry two atoms ahead), so that the pass waits on no load of its own
-    // stream.  pf / pf2 hold the batch the next pair_fn call takes.
+    // CACHED: the pair-cache batches are read one batch ahead, across atom
+    // boundaries (the next atom's segment one atom ahead, its perm entry two
+    // atoms ahead), so that the pass waits on no load of its own stream.
     PairStream ps;
-    if constexpr (CACHED) ps.start(nl, (int64_t)blockIdx.x * PW + warp, total, lane);
+    const int32_t *const tys = S > 1 ? types : nullptr;
+    if constexpr (CACHED) ps.start(nl, tys, (int64_t)blockIdx.x * PW + warp, total, lane);
     for (int64_t p = (int64_t)blockIdx.x * PW + warp; p < nl.n; p += total) {
         const int a = CACHED ? ps.a : nl.perm[p];
-        const int ti = types[a];
-        if constexpr (CACHED) ps.atom_begins(nl, p, total);
-        for (int k0 = 0; k0 < K; k0 += KC) {
-        // two partial sums per P entry (even and odd pair slots), so that
-        // the accumulation runs on packed FP32x2 multiply-adds
-        float2 acc2[S][KPL][4];
+        const int ti = S == 1 ? 0 : (CACHED ? ps.ty : types[a]);
+        if constexpr (CACHED) ps.atom_begins(nl, tys, p, total);
+        // totals: tile i, channel g (x, y of [i]) and g + 8 ([2 + i])
+        float2 acc[S][MT][4];
 #pragma unroll
         for (int s = 0; s < S; ++s)
 #pragma unroll
-            for (int kk = 0; kk < KPL; ++kk)
+            for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
-                for (int dd = 0; dd < 4; ++dd) acc2[s][kk][dd] = make_float2(0.f, 0.f);
-        float *sH = s_H[warp];
-        float *sM = s_M[warp];
-        auto pair_fn = [&](const float4 e, const float2 e2, bool valid, int) {
-                      const uint32_t jb = __float_as_uint(e.w);
-                      const int b = valid ? (int)(jb >> 28) : S;
-                      // columns grouped by neighbour species, each group starting
-                      // on a multiple of 4
-                      int cnt[S], slot = 0, start = 0;
+                for (int i = 0; i < 4; ++i) acc[s][mt][i] = make_float2(0.f, 0.f);
+        auto pair_fn = [&](const PairTwo &w, int nb) {   // pairs 2 lane, 2 lane + 1 of nb
+            const bool v0 = 2 * lane < nb, v1 = 2 * lane + 1 < nb;
+            int slot0 = 2 * lane, slot1 = 2 * lane + 1, cnt[S];
+            if constexpr (S == 1) {
+                cnt[0] = nb;
+            } else {
+                const int b0 = v0 ? (int)(__float_as_uint(w.e0.w) >> 28) : S;
+                const int b1 = v1 ? (int)(__float_as_uint(w.e1.w) >> 28) : S;
+                int start = 0;
 #pragma unroll
-                      for (int s = 0; s < S; ++s) {
-                          const unsigned ms = __ballot_sync(0xffffffffu, b == s);
-                          if (b == s) slot = start + __popc(ms & lt);
-                          cnt[s] = __popc(ms);
-                          start += (cnt[s] + 3) & ~3;
-                      }
-                      if (valid) {
-                          float r_hi, r_lo, ir;
-                          split_sqrt(e2.x, e2.y, r_hi, r_lo, ir);
-                          float H[KC], M[NHAR];
-                          if (TAB)
-                              radial_tab<KC, false>(m.rtab + (size_t)(ti * S + b) * m.rtab_n * 4 * K, K, k0,
-                                                    m.rtab_scale, r_hi, r_lo, H, nullptr);
-                          else {
-                              float fc, dfc;
-                              cutoff_fn(r_hi, m.inv_rc, fc, dfc);
-                              const float4 *rad2 = &s_rad2[(ti * S + b) * K + k0];
+                for (int s = 0; s < S; ++s) {
+                    const unsigned m0 = __ballot_sync(0xffffffffu, b0 == s), m1 = __ballot_sync(0xffffffffu, b1 == s);
+                    const int before = start + __popc(m0 & lt) + __popc(m1 & lt);
+                    if (b0 == s) slot0 = before;
+                    if (b1 == s) slot1 = before + (b0 == s);
+                    cnt[s] = __popc(m0) + __popc(m1);
+                    start += (cnt[s] + 7) & ~7;
+                }
+                // f_c of every slot: the groups' padding contributes nothing
 #pragma unroll
-                              for (int k = 0; k < KC; k += 2) {
-                                  const Radial2 o = radial2<false>(rad2, k, make_float2(r_hi, r_hi),
-                                                                   make_float2(r_lo, r_lo), make_float2(fc, fc),
-                                                                   make_float2(dfc, dfc));
-                                  H[k] = o.H.x;
-                                  H[k + 1] = o.H.y;
-                              }
-                          }
-                          harmonics16(e.x * ir, e.y * ir, e.z * ir, M);
-#pragma unroll
-                          for (int k = 0; k < KC; ++k) sH[((k % KPL) * 8 + k / KPL) * RS + slot] = H[k];
-#pragma unroll
-                          for (int d = 0; d < NHAR; ++d) sM[((d % 4) * 4 + d / 4) * RS + slot] = M[d];
-                      }
-                      __syncwarp();
-                      // P[b][k][d] += H_k M_d: four pairs per step, the rest one at a time
-                      start = 0;
-#pragma unroll
-                      for (int s = 0; s < S; ++s) {
-                          const int stop = start + cnt[s];
-                          int q = start;
-                          for (; q + 4 <= stop; q += 4) {
-                              float4 hv[KPL], mv[4];
-#pragma unroll
-                              for (int kk = 0; kk < KPL; ++kk)
-                                  hv[kk] = *reinterpret_cast<const float4 *>(&sH[(kk * 8 + kg) * RS + q]);
-#pragma unroll
-                              for (int dd = 0; dd < 4; ++dd)
-                                  mv[dd] = *reinterpret_cast<const float4 *>(&sM[(dd * 4 + g) * RS + q]);
-#pragma unroll
-                              for (int kk = 0; kk < KPL; ++kk)
-#pragma unroll
-                                  for (int dd = 0; dd < 4; ++dd) {
-                                      float2 x = acc2[s][kk][dd];
-                                      x = __ffma2_rn(make_float2(hv[kk].x, hv[kk].y), make_float2(mv[dd].x, mv[dd].y), x);
-                                      x = __ffma2_rn(make_float2(hv[kk].z, hv[kk].w), make_float2(mv[dd].z, mv[dd].w), x);
-                                      acc2[s][kk][dd] = x;
-                                  }
-                          }
-                          for (; q < stop; ++q) {
-                              float hv[KPL], mv[4];
-#pragma unroll
-                              for (int kk = 0; kk < KPL; ++kk) hv[kk] = sH[(kk * 8 + kg) * RS + q];
-#pragma unroll
-                              for (int dd = 0; dd < 4; ++dd) mv[dd] = sM[(dd * 4 + g) * RS + q];
-#pragma unroll
-                              for (int kk = 0; kk < KPL; ++kk)
-#pragma unroll
-                                  for (int dd = 0; dd < 4; ++dd)
-                                      acc2[s][kk][dd].x = fmaf(hv[kk], mv[dd], acc2[s][kk][dd].x);
-                          }
-                          start += (cnt[s] + 3) & ~3;
-                      }
-                      __syncwarp();
-                  };
-        if constexpr (CACHED) {
-            for (int base = 0; base < ps.np; base += 32) {
-                const float4 e = ps.pf;
-                const float2 e2 = ps.pf2;
-                const int nb = min(32, ps.np - base);
-                ps.advance(nl, base, k0 + KC < K, lane);
-                pair_fn(e, e2, lane < nb, nb);
+                for (int i = 0; i < RS; i += 32)
+                    if (i + lane < RS) st[2 * RS + i + lane] = 0.f;
+                __syncwarp();
             }
-            if (ps.np == 0 && k0 + KC >= K) ps.advance(nl, 0, false, lane);
+            auto put = [&](int row, const float2 v) {
+                if constexpr (S == 1) {
+                    *reinterpret_cast<float2 *>(st + row * RS + 2 * lane) = v;
+                } else {
+                    if (v0) st[row * RS + slot0] = v.x;
+                    if (v1) st[row * RS + slot1] = v.y;
+                }
+            };
+            float2 r_hi, r_lo, ir;
+            split_sqrt2(make_float2(w.q0.x, w.q1.x), make_float2(w.q0.y, w.q1.y), r_hi, r_lo, ir);
+            if constexpr (TAB) {
+                const float2 x = __fmul2_rn(r_hi, bc2(m.rtab_scale)), gf = make_float2(floorf(x.x), floorf(x.y));
+                put(0, __ffma2_rn(r_lo, bc2(m.rtab_scale), __ffma2_rn(gf, bc2(-1.f), x)));
+                // as tab_cell; a place without a pair reads interval 0
+                put(1, make_float2(__int_as_float(v0 ? __float_as_int(gf.x + 12582912.0f) - 0x4B400000 : 0),
+                                   __int_as_float(v1 ? __float_as_int(gf.y + 12582912.0f) - 0x4B400000 : 0)));
+                put(2, make_float2(v0 ? 1.f : 0.f, v1 ? 1.f : 0.f));
+            } else {
+                const float2 fc = cutoff2(r_hi, m.inv_rc);
+                put(0, r_hi);
+                put(1, r_lo);
+                put(2, make_float2(v0 ? fc.x : 0.f, v1 ? fc.y : 0.f));
+            }
+            float2 Y[NHAR];
+            harmonics16x2(__fmul2_rn(make_float2(w.e0.x, w.e1.x), ir), __fmul2_rn(make_float2(w.e0.y, w.e1.y), ir),
+                          __fmul2_rn(make_float2(w.e0.z, w.e1.z), ir), Y);
+#pragma unroll
+            for (int c = 1; c < NHAR; ++c) put(3 + 8 * ((c >> 1) & 1) + 2 * (c >> 2) + (c & 1), Y[c]);
+            __syncwarp();
+            int start = 0;
+#pragma unroll
+            for (int s = 0; s < S; ++s) {
+                const int stop = start + cnt[s];
+                const int rad = (ti * S + s) * K;
+                const float *tab = TAB ? m.rtab + (size_t)(ti * S + s) * m.rtab_n * 4 * K : nullptr;
+                float2 mh[HOIST ? MT : 1][NC], ml[HOIST ? MT : 1][NC], et[HOIST ? MT : 1][NC];
+                if constexpr (HOIST && !TAB) {
+#pragma unroll
+                    for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+                        for (int h = 0; h < NC; ++h) {
+                            const float4 q = channel(rad + 16 * mt + 8 * h + g);
+                            mh[mt][h] = make_float2(q.x, q.x);
+                            ml[mt][h] = make_float2(q.y, q.y);
+                            et[mt][h] = make_float2(q.z, q.z);
+                        }
+                }
+#pragma unroll 1
+                for (int q0 = start; q0 < stop; q0 += 8) {
+                    const int q = q0 + 2 * t;   // this lane's pairs q, q + 1
+                    const float2 r0 = *reinterpret_cast<const float2 *>(st + q);
+                    const float2 r1 = *reinterpret_cast<const float2 *>(st + RS + q);
+                    const float2 fc = *reinterpret_cast<const float2 *>(st + 2 * RS + q);
+                    Split2 y[2];
+#pragma unroll
+                    for (int i = 0; i < 2; ++i)
+                        y[i] = split2(*reinterpret_cast<const float2 *>(st + (3 + 8 * i + g) * RS + q));
+#pragma unroll
+                    for (int mt = 0; mt < MT; ++mt) {
+                        Split2 x[2];
+                        x[1] = Split2{0u, 0u, 0u, 0u};
+#pragma unroll
+                        for (int h = 0; h < NC; ++h) {
+                            float2 H;
+                            if constexpr (TAB) {
+                                const int k = 16 * mt + 8 * h + g;
+                                const float4 *c = reinterpret_cast<const float4 *>(tab);
+                                const float4 u = __ldg(c + (size_t)__float_as_int(r1.x) * K + k);
+                                const float4 v = __ldg(c + (size_t)__float_as_int(r1.y) * K + k);
+                                H.x = fmaf(r0.x, fmaf(r0.x, fmaf(r0.x, u.w, u.z), u.y), u.x);
+                                H.y = fmaf(r0.y, fmaf(r0.y, fmaf(r0.y, v.w, v.z), v.y), v.x);
+                                H = __fmul2_rn(H, fc);
+                            } else {
+                                float2 qh, ql, qe;
+                                if constexpr (HOIST) {
+                                    qh = mh[mt][h]; ql = ml[mt][h]; qe = et[mt][h];
+                                } else {
+                                    const float4 u = channel(rad + 16 * mt + 8 * h + g);
+                                    qh = bc2(u.x); ql = bc2(u.y); qe = bc2(u.z);
+                                }
+                                const float2 d = __fadd2_rn(__fadd2_rn(r0, qh), __fadd2_rn(r1, ql));
+                                const float2 ex = __fmul2_rn(__fmul2_rn(qe, d), d);
+                                H = __fmul2_rn(make_float2(ex2_ftz(ex.x), ex2_ftz(ex.y)), fc);
+                            }
+                            x[h] = split2(H);
+                        }
+#pragma unroll
+                        for (int i = 0; i < 2; ++i) {
+                            float c[4];
+                            const uint32_t xl[4] = {x[0].l0, x[1].l0, x[0].l1, x[1].l1};
+                            const uint32_t xh[4] = {x[0].h0, x[1].h0, x[0].h1, x[1].h1};
+                            mma_tf32_first(c, xl, y[i].h0, y[i].h1);
+                            mma_tf32(c, xh, y[i].l0, y[i].l1);
+                            mma_tf32(c, xh, y[i].h0, y[i].h1);
+                            acc[s][mt][i] = __ffma2_rn(make_float2(c[0], c[1]), untrunc, acc[s][mt][i]);
+                            if (NC == 2) acc[s][mt][2 + i] = __ffma2_rn(make_float2(c[2], c[3]), untrunc, acc[s][mt][2 + i]);
+                        }
+                    }
+                }
+                start += (cnt[s] + 7) & ~7;
+            }
+            __syncwarp();
+        };
+        if constexpr (CACHED) {
+            for (int base = 0; base < ps.np; base += 64) {
+                const PairTwo w = ps.pf;
+                ps.advance(nl, base, lane);
+                pair_fn(w, min(64, ps.np - base));
+            }
+            if (ps.np == 0) ps.advance(nl, 0, lane);
         } else {
-            for_pairs(nl, a, nl.beg[a], nl.end[a], m.rc2h, m.rc2l, s_q[warp], s_q2[warp], lane, pair_fn);
+            queue_pairs<2>(nl, a, nl.beg[a], nl.end[a], m.rc2h, m.rc2l, s_q[warp], s_q2[warp], lane,
+                           [&](const float4 *p, const float2 *p2, int nb) {
+                               pair_fn(load_two(p, p2, 2 * lane, nb), nb);
+                           });
         }
-        float acc[S][KPL][4];
-#pragma unroll
-        for (int s = 0; s < S; ++s)
-#pragma unroll
-            for (int kk = 0; kk < KPL; ++kk)
-#pragma unroll
-                for (int dd = 0; dd < 4; ++dd) acc[s][kk][dd] = acc2[s][kk][dd].x + acc2[s][kk][dd].y;
-        // A[b][k][c] for the backward pass
+        // A[b][k][c] for the backward pass, and G
         float *Pa = Pout + (size_t)p * (S * K * NHAR);   // workspaces are indexed by perm position
+        float *Ga = G + (size_t)p * Dd;
 #pragma unroll
         for (int s = 0; s < S; ++s)
 #pragma unroll
-            for (int kk = 0; kk < KPL; ++kk)
-                *reinterpret_cast<float4 *>(Pa + (s * K + k0 + kg * KPL + kk) * NHAR + 4 * g) =
-                    make_float4(acc[s][kk][0], acc[s][kk][1], acc[s][kk][2], acc[s][kk][3]);
+            for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
-        for (int s = 0; s < S; ++s)
-#pragma unroll
-            for (int kk = 0; kk < KPL; ++kk)
-                G[(size_t)p * Dd + (s * K + k0 + kg * KPL + kk) * 4 + g] = desc_value(acc[s][kk], Wg, g);
-        }
+                for (int h = 0; h < NC; ++h) {
+                    const int row = s * K + 16 * mt + 8 * h + g;
+                    const float A[4] = {acc[s][mt][2 * h].x, acc[s][mt][2 * h].y, acc[s][mt][2 * h + 1].x,
+                                        acc[s][mt][2 * h + 1].y};
+                    *reinterpret_cast<float4 *>(Pa + row * NHAR + 4 * t) = make_float4(A[0], A[1], A[2], A[3]);
+                    Ga[row * 4 + t] = desc_value(A, Wt, t);
+                }
         if constexpr (CACHED) ps.atom_ends();
     }
 }
@@ -889,20 +1079,6 @@ __global__ void __launch_bounds__(PW * 32, 4) k_force_merged(DevModel m, DevNlis
 // x_hi = tf32(x) and x_lo = tf32(x - x_hi), and a product is accumulated as
 // a_lo b_hi + a_hi b_lo + a_hi b_hi in FP32 (the dropped a_lo b_lo and the
 // split remainders are about 2^-22 of |a b|).
-__device__ __forceinline__ void split_tf32(float x, uint32_t &hi, uint32_t &lo) {
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(hi) : "f"(x));
-    const float rest = x - __uint_as_float(hi);   // exact
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(lo) : "f"(rest));
-}
-
-// c += a b for one m16n8k8 tile (a: 16 x 8 row-major, b: 8 x 8, c: 16 x 8)
-__device__ __forceinline__ void mma_tf32(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-    asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
-        "{%0, %1, %2, %3};"
-        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
 // One species, direct radial basis, pair cache present.
 template <int K>
 __global__ void __launch_bounds__(PW * 32, 4) k_force_tc(DevModel m, DevNlist nl, const float *__restrict__ Pin,
@@ -1100,9 +1276,7 @@ __global__ void __launch_bounds__(PW * 32, 4) k_force(DevModel m, DevNlist nl, c
                                                    const float *__restrict__ dG,
                                                    unsigned long long *__restrict__ Fq,
                                                    double *__restrict__ part_w, float *__restrict__ w_atom) {
-    constexpr int KPL = K / 8;
     constexpr int PSTR = K * NHAR + 4;   // per-species stride of P' (bank offset between species)
-    constexpr int Dd = S * K * 4;
     __shared__ float4 s_rad[S * S * K];
     __shared__ float4 s_q[PW][64];
     __shared__ float2 s_q2[PW][64];
@@ -1202,6 +1376,35 @@ __global__ void __launch_bounds__(PW * 32, 4) k_force(DevModel m, DevNlist nl, c
     }
 }
 
+// Blocks of the descriptor pass (or the caller's tuning): what the GPU holds at
+// once, and more once every warp would run over 512 channels (atoms x S x K),
+// so that blocks that finish early are replaced (1M atoms, K = 16: 1.12 ms with
+// the resident 7 blocks per SM, 1.04 with 4 times, 1.02 with 8 times and 1.05
+// with 64 times as many; 39,366 atoms, K = 128: 0.51 ms with the resident
+// blocks, 0.34 with 4 atoms per warp; 16,384 atoms, K = 16: 0.041 ms with the
+// resident blocks, 0.045 with 8 times as many).
+constexpr int CHANNELS_PER_WARP = 512;
+template <auto KERNEL>
+int desc_blocks(const DevModel &dm, int64_t n, int nblk) {
+    if (dm.pair_bps > 0) return nblk;
+    static const int resident = [] {
+        int dev = 0, nsm = 0, per_sm = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, KERNEL, PW * 32, 0);
+        return std::max(1, nsm) * std::max(1, per_sm);
+    }();
+    const int64_t most = (n + PW - 1) / PW;
+    return (int)std::max<int64_t>(1, std::min<int64_t>(most, std::max<int64_t>(resident, n * dm.S * dm.K / (PW * CHANNELS_PER_WARP))));
+}
+
+template <int K, int S, bool TAB, bool CACHED>
+void launch_desc(const DevModel &dm, const DevNlist &dn, const double *pos, const int32_t *types, tmd_nlist *nl,
+                 int nblk, cudaStream_t s) {
+    const int nb = desc_blocks<k_desc<K, S, TAB, CACHED>>(dm, dn.n, nblk);
+    TMD_LAUNCH("k_desc", s, k_desc<K, S, TAB, CACHED><<<nb, PW * 32, 0, s>>>(dm, dn, pos, types, nl->G, nl->P));
+}
+
 template <int K, int S>
 tmd_status launch_pair_kernels(const DevModel &dm, const DevNlist &dn, const double *pos, const int32_t *types,
                                tmd_nlist *nl, double *part_w, int nblk, cudaStream_t s, bool forward,
@@ -1209,14 +1412,12 @@ tmd_status launch_pair_kernels(const DevModel &dm, const DevNlist &dn, const dou
     if (forward && dn.pq) {   // screen into the pair cache, then stream it
         const tmd_status st = launch_screen(dm, dn, s);
         if (st != TMD_OK) return st;
-        if (dm.rtab)
-            TMD_LAUNCH("k_desc", s, k_desc<K, S, true, true><<<nblk, PW * 32, 0, s>>>(dm, dn, pos, types, nl->G, nl->P));
-        else
-            TMD_LAUNCH("k_desc", s, k_desc<K, S, false, true><<<nblk, PW * 32, 0, s>>>(dm, dn, pos, types, nl->G, nl->P));
+        if (dm.rtab) launch_desc<K, S, true, true>(dm, dn, pos, types, nl, nblk, s);
+        else launch_desc<K, S, false, true>(dm, dn, pos, types, nl, nblk, s);
     } else if (forward && dm.rtab)
-        TMD_LAUNCH("k_desc", s, k_desc<K, S, true, false><<<nblk, PW * 32, 0, s>>>(dm, dn, pos, types, nl->G, nl->P));
+        launch_desc<K, S, true, false>(dm, dn, pos, types, nl, nblk, s);
     else if (forward)
-        TMD_LAUNCH("k_desc", s, k_desc<K, S, false, false><<<nblk, PW * 32, 0, s>>>(dm, dn, pos, types, nl->G, nl->P));
+        launch_desc<K, S, false, false>(dm, dn, pos, types, nl, nblk, s);
     else if (w_atom && dm.rtab)   // batched evaluations always run with the pair cache
         TMD_LAUNCH("k_force", s, k_force<K, S, true, true, true><<<nblk, PW * 32, 0, s>>>(dm, dn, pos, types, nl->P,
                                                                                         nl->dG, nl->Fq, part_w, w_atom));
