@@ -224,16 +224,15 @@ int64_t tmd_graph_replays(void);
 
 /*
  * Tile shapes of this implementation's kernels (the paper has no counterpart:
- * they are launch choices of the GPU path).  32 and 64 give the same results
- * up to the order of FP64 partial sums; 128 runs the network's FP32 sums in
- * another order (results agree to FP32 rounding).
- *  tile_rows           atoms per tile of the FP32 network kernel: 32 or 64
- *                      (weights streamed through shared memory), 128
- *                      (weights resident in shared memory; networks whose
- *                      descriptor length and hidden widths are all 64, one or
- *                      two hidden layers; other networks fall back to the
- *                      built-in choice), 0 = built-in choice (128 where it
- *                      applies, else 32);
+ * they are launch choices of the GPU path).  The results are the same up to
+ * the order of FP64 partial sums.
+ *  tile_rows           atoms per tile of the FP32 network kernel on the FP32
+ *                      pipes: 32 or 64; 128 (networks whose descriptor length
+ *                      and hidden widths are all 64, one or two hidden layers)
+ *                      and 0 = built-in choice.  Networks that run on the
+ *                      tensor cores (hidden widths multiples of 16 up to 128,
+ *                      activations of a tile within an SM's shared memory)
+ *                      have 128-atom tiles with each of them;
  *  pair_blocks_per_sm  blocks per SM of the persistent descriptor / force
  *                      grids (0 = built-in 16);
  *  ms                  output of the tuners: measured milliseconds of one

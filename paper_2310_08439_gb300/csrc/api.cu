@@ -524,19 +524,18 @@ tmd_status tmd_model_create(const tmd_model_desc *d, tmd_model **out) {
     m->eta.assign(d->eta, d->eta + (size_t)S * S * K);
     m->rc_exact = d->rc;
     {
-        const tmd_status su = tmd::mlp_umma_build(m, d->weights);
-        if (su != TMD_OK) { cudaFree(m->dev_block); delete m; return su; }
+        tmd_status su = tmd::mlp_umma_build(m, d->weights);
+        if (su == TMD_OK) su = tmd::mlp_tf32_build(m, d->weights);
+        if (su != TMD_OK) { tmd_model_destroy(m); return su; }
     }
     if (tmd::mlp_smem_tr_public(m->dm, 32) > 227 * 1024) {
         set_error("network too wide: the activations of a 32-atom tile exceed the shared memory of an SM");
-        cudaFree(m->dev_block);
-        if (m->dev_umma) cudaFree(m->dev_umma);
-        delete m;
+        tmd_model_destroy(m);
         return TMD_ERR_UNIMPLEMENTED;
     }
     if (d->precision == TMD_PREC_BF16) {
         tmd_status st = tmd_model_set_precision(m, TMD_PREC_BF16);
-        if (st != TMD_OK) { cudaFree(m->dev_block); if (m->dev_umma) cudaFree(m->dev_umma); delete m; return st; }
+        if (st != TMD_OK) { tmd_model_destroy(m); return st; }
     }
     *out = m;
     return TMD_OK;
@@ -547,6 +546,7 @@ tmd_status tmd_model_destroy(tmd_model *m) {
     if (m->dev_block) cudaFree(m->dev_block);
     if (m->dev_rtab) cudaFree(m->dev_rtab);
     if (m->dev_umma) cudaFree(m->dev_umma);
+    if (m->dev_tf32) cudaFree(m->dev_tf32);
     delete m;
     return TMD_OK;
 }

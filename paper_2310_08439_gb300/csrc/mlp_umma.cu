@@ -696,6 +696,8 @@ uint16_t bf16_bits(double x) {
     return (uint16_t)((v + 0x7fffu + ((v >> 16) & 1u)) >> 16);   // round to nearest even
 }
 
+#include "mlp_tf32.cuh"
+
 }  // namespace
 
 int g_network_kernel = 0;
@@ -793,6 +795,125 @@ tmd_status mlp_umma_build(tmd_model *m, const double *const *weights) {
     }
     m->dev_umma = dev;
     for (int s = 0; s < S; ++s) dm.ub[s] = static_cast<const uint16_t *>(dev) + per * s;
+    return TMD_OK;
+}
+
+bool mlp_tf32_ok(const DevModel &dm) {
+    Tf32Net u;
+    return dm.precision == TMD_PREC_FP32 && tf32_plan(dm, u);
+}
+
+tmd_status mlp_tf32_launch(const char *name, const DevModel &dm, const int32_t *perm, const int32_t *types, int64_t n,
+                           const float *G, float *dG, float *e_atom, double *part_e, int *ntile_out, cudaStream_t s) {
+    Tf32Net u;
+    if (!tf32_plan(dm, u)) {
+        set_error("network shapes outside the split-TF32 kernel");
+        return TMD_ERR_UNIMPLEMENTED;
+    }
+    static const cudaError_t set =
+        cudaFuncSetAttribute(k_mlp_tf32, cudaFuncAttributeMaxDynamicSharedMemorySize, TF_SMEM_MAX);
+    TMD_CUDA(set);
+    const int ntile = (int)((n + UM - 1) / UM);
+    int dev = 0, nsm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    const int grid = std::max(1, std::min(ntile, std::max(1, nsm) * u.blocks_per_sm));
+    TMD_LAUNCH(name, s, k_mlp_tf32<<<grid, UTHREADS, u.smem, s>>>(dm, u, perm, types, n, G, dG, e_atom, part_e, ntile));
+    TMD_CUDA(cudaGetLastError());
+    *ntile_out = ntile;
+    return TMD_OK;
+}
+
+// FP32 weights split into two TF32 planes in the operand layout of k_mlp_tf32
+// (product order as mlp_umma_build; leaves dm.tb null when the widths have no
+// such form)
+tmd_status mlp_tf32_build(tmd_model *m, const double *const *weights) {
+    DevModel &dm = m->dm;
+    const int L = dm.L, S = dm.S;
+    if (m->dev_tf32) {
+        cudaFree(m->dev_tf32);
+        m->dev_tf32 = nullptr;
+    }
+    for (int s = 0; s < TMD_MAX_SPECIES; ++s) dm.tb[s] = nullptr;
+    TfShape sh;
+    if (!tf32_shape(dm, sh)) return TMD_OK;
+    size_t off = 0;
+    for (int pr = 0; pr < 2 * L; ++pr) {
+        dm.toff[pr] = (int)off;
+        off += (size_t)sh.npass[pr] * sh.nk[pr] * sh.np[pr] * TKC * 2;
+    }
+    const size_t per = (off + 255) & ~size_t(255);   // 1 KiB aligned species blocks
+    std::vector<float> h(per * S, 0.f);
+    for (int s = 0; s < S; ++s) {
+        const double *w = weights[s];
+        size_t lo[MAX_LAYERS], o = 0;
+        for (int l = 0; l <= L; ++l) {
+            lo[l] = o;
+            o += (size_t)dm.dims[l] * dm.dims[l + 1] + dm.dims[l + 1];
+        }
+        for (int pr = 0; pr < 2 * L; ++pr) {
+            const bool fwd = pr < L;
+            const int l = fwd ? pr : 2 * L - 1 - pr;
+            const int in = dm.dims[l];
+            const int K = fwd ? dm.dims[l] : dm.dims[l + 1], N = fwd ? dm.dims[l + 1] : dm.dims[l];
+            float *b = h.data() + per * s + dm.toff[pr];
+            const int np = sh.np[pr];
+            for (int nn = 0; nn < N; ++nn)
+                for (int k = 0; k < K; ++k) {
+                    const double v = fwd ? w[lo[l] + (size_t)nn * in + k] : w[lo[l] + (size_t)k * in + nn];
+                    const int P = nn / np, r = nn % np, c = k / TKC, kk = k % TKC;
+                    const size_t plane = (size_t)np * TKC;
+                    const size_t idx = ((size_t)P * sh.nk[pr] + c) * plane * 2 + (size_t)(r >> 3) * (8 * TKC) +
+                                       (size_t)(kk >> 2) * 32 + (r & 7) * 4 + (kk & 3);
+                    const float hi = tf32_value(v);
+                    b[idx] = hi;
+                    b[idx + plane] = tf32_value(v - (double)hi);
+                }
+        }
+    }
+    // the copies of a species in the order in which the kernel takes them
+    std::vector<int2> ck;
+    for (int pr = 0; pr < 2 * L; ++pr) {
+        const int K = pr < L ? dm.dims[pr] : dm.dims[2 * L - pr], kg = pr == 0 ? sh.ka : K, np = sh.np[pr];
+        for (int P = 0; P < sh.npass[pr]; ++P)
+            for (int k0 = 0; k0 < K; k0 += kg) {
+                const int nk = (std::min(kg, K - k0) + TKC - 1) / TKC, half = (nk + 1) >> 1;
+                for (int hh = 0; hh < 2; ++hh)
+                    for (int plane = 1; plane >= 0; --plane)
+                        for (int c = hh ? half : 0; c < (hh ? nk : half); ++c)
+                            ck.push_back(make_int2(
+                                dm.toff[pr] + ((P * sh.nk[pr] + k0 / TKC + c) * 2 + plane) * np * TKC, np * TKC * 4));
+            }
+    }
+    int at[MAX_LAYERS + 1];
+    const int cstride = tf32_consts(dm, at);
+    const size_t c0 = h.size();
+    h.resize(c0 + ((size_t)cstride * S + 1) / 2 * 2, 0.f);
+    for (int s = 0; s < S; ++s) {
+        const double *w = weights[s];
+        float *c = h.data() + c0 + (size_t)s * cstride;
+        for (int l = 0; l <= L; ++l) {   // layer L: the output (weights, then its bias)
+            const size_t nw = (size_t)dm.dims[l] * dm.dims[l + 1];
+            for (int j = 0; j < dm.dims[l + 1]; ++j) c[l < L ? at[l] + j : at[L + 1]] = (float)w[nw + j];
+            if (l == L)
+                for (int j = 0; j < dm.dims[L]; ++j) c[at[L] + j] = (float)w[j];
+            w += nw + dm.dims[l + 1];
+        }
+    }
+    void *dev = nullptr;
+    cudaError_t e = cudaMalloc(&dev, sizeof(float) * h.size() + sizeof(int2) * ck.size());
+    if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc split weights");
+    e = cudaMemcpy(dev, h.data(), sizeof(float) * h.size(), cudaMemcpyHostToDevice);
+    int2 *const ck_dev = reinterpret_cast<int2 *>(static_cast<float *>(dev) + h.size());
+    if (e == cudaSuccess) e = cudaMemcpy(ck_dev, ck.data(), sizeof(int2) * ck.size(), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) {
+        cudaFree(dev);
+        return cuda_fail(e, "cudaMemcpy split weights");
+    }
+    m->dev_tf32 = dev;
+    dm.tck = ck_dev;
+    dm.tconst = static_cast<const float *>(dev) + c0;
+    for (int s = 0; s < S; ++s) dm.tb[s] = static_cast<const float *>(dev) + per * s;
     return TMD_OK;
 }
 

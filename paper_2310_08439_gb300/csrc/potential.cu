@@ -415,343 +415,6 @@ __global__ void __launch_bounds__(MLP_THREADS, TR == 64 ? 4 : 2) k_mlp(DevModel 
 }
 
 // ---------------------------------------------------------------------------
-// network, FP32 SIMT with resident weights (E_a = NNP(G_a) and G' = dE_a/dG_a,
-// Sec. "The Tensor Formalism"): networks whose descriptor length and hidden
-// widths are all 64, with one or two hidden layers.
-//
-// A persistent block of 256 threads keeps one species' weight matrices in
-// shared memory and walks a contiguous range of 128-atom tiles (perm order,
-// so the species changes at most S - 1 times per block).  Every product of
-// the chain (forward layers, then the input-gradient chain) is
-// [128 x 64] x [64 x 64]: each thread owns an 8 x 4 block of the result
-// (atoms 4 rb .. 4 rb + 3 and 64 + 4 rb .. 64 + 4 rb + 3, columns 4 cb ..
-// 4 cb + 3) and runs 32 multiply-adds (16 packed FP32x2 instructions) per
-// two float4 activation loads and one float4 weight load.  Each weight matrix is stored once in 4 x 4
-// blocks: the forward products read rows of a block, the backward products
-// (which multiply by W^T) read its columns from the same copy after loading
-// the whole block.  The rows inside a block are XOR-swizzled so that the
-// four column groups of a warp read distinct banks in both directions.  The
-// output layer (E_a and dz_L) is formed in the epilogue of the last forward
-// product.
-//
-// Two activation buffers X and Y alternate their roles from tile to tile.
-// A tile starts with its G rows already in X (row-major, copied by cp.async
-// while the previous tile ran its last product); they are transposed into Y,
-// and the chain runs Y -> X (a_1) -> Y (dz_2) -> X (dz_1 over a_1) -> G'
-// (one hidden layer: Y -> X (dz_1) -> G').  The last product reads only X,
-// so the next tile's G rows are copied into Y meanwhile, and Y becomes the
-// next tile's X.
-// ---------------------------------------------------------------------------
-constexpr int RW_TR = 128;              // atoms per tile
-constexpr int RW_THREADS = 256;         // 8 warps, an 8 x 4 result block per thread
-constexpr int RW_N = 64;                // descriptor length and every hidden width
-constexpr int RW_LDT = RW_TR + 4;       // row stride of the transposed activations
-constexpr int RW_LDG = RW_N + 4;        // row stride of staged G rows (conflict-free float4 reads)
-constexpr int RW_MAXL = 2;              // hidden layers
-constexpr int RW_WF = RW_N * RW_N;      // floats per weight matrix
-constexpr int RW_BUF = (RW_N * RW_LDT > RW_TR * RW_LDG) ? RW_N * RW_LDT : RW_TR * RW_LDG;
-constexpr int RW_CG = 4;                // column groups: energy partials of a row come from 4 warp pairs
-
-// dynamic shared memory: weights, two activation buffers, biases, output
-// weights and bias, the energy partials of the column groups
-constexpr size_t RW_SMEM_FLOATS =
-    (size_t)RW_MAXL * RW_WF + 2 * (size_t)RW_BUF + RW_MAXL * RW_N + RW_N + 4 + RW_CG * RW_TR;
-
-// place of element (k, o) of a 64 x 64 matrix in the blocked, swizzled layout
-__device__ __forceinline__ int rw_widx(int k, int o) {
-    const int kb = k >> 2, ob = o >> 2, f = (kb ^ (ob >> 1)) & 3;
-    return ((kb * 16 + ob) << 4) + (((k & 3) ^ f) << 2) + (o & 3);
-}
-
-__device__ __forceinline__ float rw_comp(const float4 v, int c) {
-    return c == 0 ? v.x : (c == 1 ? v.y : (c == 2 ? v.z : v.w));
-}
-
-// acc[i][c] = sum_k At[k][atom i] B[k][4 cb + c] over k = 0..63, where B = W
-// (forward: W stored [in][out]) or B = W^T (backward).  The multiply-adds run
-// on packed FP32x2 (fma.rn.f32x2, each half rounded as fmaf): atom pairs
-// (i, i + 1) against a duplicated weight, so one instruction does two.
-template <bool BWD>
-__device__ __forceinline__ void rw_product(const float *At, const float *Wm, int rb, int cb, float (&acc)[8][4]) {
-    float2 acc2[4][4];   // acc2[j][c] = (acc[2 j][c], acc[2 j + 1][c])
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) acc2[j][c] = make_float2(0.f, 0.f);
-#pragma unroll 1
-    for (int g = 0; g < RW_N / 4; ++g) {
-        // forward: block (g, cb), row k & 3 for k = 4 g .. 4 g + 3;
-        // backward: block (cb, g), column k & 3
-        const float *bk = Wm + (BWD ? 16 * (16 * cb + g) : 16 * (16 * g + cb));
-        const int f = BWD ? ((cb ^ (g >> 1)) & 3) : ((g ^ (cb >> 1)) & 3);
-        float4 w[4];   // logical rows 0..3 of the block
-#pragma unroll
-        for (int r = 0; r < 4; ++r) w[r] = *reinterpret_cast<const float4 *>(bk + 4 * (r ^ f));
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            const float *a = At + (4 * g + r) * RW_LDT + 4 * rb;
-            const float4 a0 = *reinterpret_cast<const float4 *>(a);
-            const float4 a1 = *reinterpret_cast<const float4 *>(a + 64);
-            const float2 ap[4] = {make_float2(a0.x, a0.y), make_float2(a0.z, a0.w), make_float2(a1.x, a1.y),
-                                  make_float2(a1.z, a1.w)};
-            float wv[4];
-            if (!BWD) {
-                wv[0] = w[r].x; wv[1] = w[r].y; wv[2] = w[r].z; wv[3] = w[r].w;
-            } else {
-#pragma unroll
-                for (int q = 0; q < 4; ++q) wv[q] = rw_comp(w[q], r);
-            }
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const float2 w2 = make_float2(wv[c], wv[c]);
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc2[j][c] = __ffma2_rn(ap[j], w2, acc2[j][c]);
-            }
-        }
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            acc[2 * j][c] = acc2[j][c].x;
-            acc[2 * j + 1][c] = acc2[j][c].y;
-        }
-}
-
-// the 8 atoms of a thread's result block as two float4 of a transposed row
-__device__ __forceinline__ void rw_store_col(float *Ct, int col, int rb, const float (&v)[8]) {
-    float *c = Ct + col * RW_LDT + 4 * rb;
-    *reinterpret_cast<float4 *>(c) = make_float4(v[0], v[1], v[2], v[3]);
-    *reinterpret_cast<float4 *>(c + 64) = make_float4(v[4], v[5], v[6], v[7]);
-}
-
-// weights of species s into shared memory: W_l blocked (rw_widx), biases,
-// output weights and bias
-__device__ __forceinline__ void rw_load_species(const DevModel &m, int s, float *sW, float *sBias, float *sWout,
-                                                float *sBout) {
-    const int L = m.L;
-    for (int l = 0; l < L; ++l) {
-        const float *W = m.wf[s] + m.off_f[l];   // [64 in][64 out], then the bias [64]
-        for (int idx = threadIdx.x; idx < RW_N * (RW_N / 4); idx += RW_THREADS) {
-            const int k = idx >> 4, o = 4 * (idx & 15);
-            *reinterpret_cast<float4 *>(sW + l * RW_WF + rw_widx(k, o)) =
-                __ldg(reinterpret_cast<const float4 *>(W + k * RW_N + o));
-        }
-        if (threadIdx.x < RW_N) sBias[l * RW_N + threadIdx.x] = __ldg(W + RW_WF + threadIdx.x);
-    }
-    const float *wo = m.wf[s] + m.off_f[L];   // output layer: [64][1], then its bias
-    if (threadIdx.x < RW_N) sWout[threadIdx.x] = __ldg(wo + threadIdx.x);
-    if (threadIdx.x == 0) sBout[0] = __ldg(wo + RW_N);
-}
-
-// half h (threadIdx.x >> 7) of the G row at perm position p0 + (threadIdx.x
-// & 127) (zeros beyond n) -> the staging buffer (row-major, stride RW_LDG),
-// by cp.async; not waited for
-__device__ __forceinline__ void rw_stage_g(const float *__restrict__ G, int64_t p0, int64_t n, float *X) {
-    const int row = threadIdx.x & (RW_TR - 1), h = threadIdx.x >> 7;
-    const int64_t p = p0 + row;
-    const bool ok = p < n;
-    const float *src = ok ? G + (size_t)p * RW_N + 32 * h : G;
-    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(X + row * RW_LDG + 32 * h);
-    const int bytes = ok ? 16 : 0;   // 0: the 16 bytes are zero-filled
-#pragma unroll
-    for (int c4 = 0; c4 < 8; ++c4)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst + 16 * c4),
-                     "l"(src + (ok ? 4 * c4 : 0)), "r"(bytes));
-    cp_async_commit();
-}
-
-__global__ void __launch_bounds__(RW_THREADS, 2) k_mlp_res(DevModel m, const int32_t *__restrict__ perm,
-                                                        const int32_t *__restrict__ types, int64_t n,
-                                                        const float *__restrict__ G, float *__restrict__ dG,
-                                                        float *__restrict__ e_atom, double *__restrict__ part_e) {
-    extern __shared__ __align__(16) float sm[];
-    float *sW = sm;                                  // L blocked 64 x 64 matrices
-    float *buf0 = sW + RW_MAXL * RW_WF;              // the two activation buffers
-    float *sBias = buf0 + 2 * RW_BUF;                // [L][64]
-    float *sWout = sBias + RW_MAXL * RW_N;           // [64]
-    float *sBout = sWout + RW_N;                     // [1] (+ 3 pad)
-    float *sEp = sBout + 4;                          // [RW_CG][RW_TR]
-    // per tile parity: atoms, species, energies and the warps' species
-    // ranges (a tile's are written during the previous tile's last product)
-    __shared__ int s_atom2[2][RW_TR], s_type2[2][RW_TR];
-    __shared__ float s_e2[2][RW_TR];
-    __shared__ int s_lohi2[2][RW_THREADS / 32][2];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int rb = (lane & 7) + 8 * (warp & 1), cb = (lane >> 3) + 4 * (warp >> 1);
-    const int L = m.L, act = m.act;
-    const float spb = m.sp_b;
-    const int64_t ntile = (n + RW_TR - 1) / RW_TR;
-    const int64_t t_beg = ntile * blockIdx.x / gridDim.x, t_end = ntile * (blockIdx.x + 1) / gridDim.x;
-    int loaded = -1;   // species whose weights are in sW
-    int xb = 0;        // buffer holding the tile's staged G rows
-    float acc[8][4];
-    // atoms and species of tile t at parity par (threads >= RW_TR only take
-    // part in the warp reductions)
-    auto publish = [&](int par, int a, int ty) {
-        if (tid < RW_TR) {
-            s_atom2[par][tid] = a;
-            s_type2[par][tid] = ty;
-            s_e2[par][tid] = 0.f;
-        }
-        const int lo = __reduce_min_sync(0xffffffffu, ty >= 0 ? ty : TMD_MAX_SPECIES);
-        const int hi = __reduce_max_sync(0xffffffffu, ty);
-        if (lane == 0) { s_lohi2[par][warp][0] = lo; s_lohi2[par][warp][1] = hi; }
-    };
-    if (t_beg < t_end) {
-        rw_stage_g(G, t_beg * RW_TR, n, buf0);
-        const int64_t p = t_beg * RW_TR + tid;
-        const int a = (tid < RW_TR && p < n) ? perm[p] : -1;
-        publish(0, a, a >= 0 ? types[a] : -1);
-        __syncthreads();
-    }
-    for (int64_t tile = t_beg; tile < t_end; ++tile) {
-        const int64_t p0 = tile * RW_TR;
-        float *X = buf0 + xb * RW_BUF, *Y = buf0 + (xb ^ 1) * RW_BUF;
-        const int *s_atom = s_atom2[xb], *s_type = s_type2[xb];
-        float *s_e = s_e2[xb];
-        const bool more = tile + 1 < t_end;
-        int next_a = -1, next_ty = -1;   // the next tile's atom and species of this thread's row
-        asm volatile("cp.async.wait_all;\n" ::);   // this thread's staged G row (read by it alone)
-        int s_lo = TMD_MAX_SPECIES, s_hi = -1;
-#pragma unroll
-        for (int w = 0; w < RW_THREADS / 32; ++w) {
-            s_lo = min(s_lo, s_lohi2[xb][w][0]);
-            s_hi = max(s_hi, s_lohi2[xb][w][1]);
-        }
-        for (int s = s_lo; s <= s_hi; ++s) {
-            if (s != s_lo) {   // a second species in this tile: its G rows again (X was overwritten)
-                __syncthreads();
-                rw_stage_g(G, p0, n, X);
-                asm volatile("cp.async.wait_all;\n" ::);
-                __syncthreads();
-            }
-            if (s != loaded) {
-                rw_load_species(m, s, sW, sBias, sWout, sBout);
-                loaded = s;
-            }
-            if (s == s_hi && more && tid < RW_TR) {   // read ahead: the next tile's atom (used before G')
-                const int64_t p = p0 + RW_TR + tid;
-                next_a = p < n ? perm[p] : -1;
-            }
-            {   // half of G row (tid & 127) (X, row-major) -> Y transposed (conflict-free both ways)
-                const int row = tid & (RW_TR - 1), h = tid >> 7;
-                const float *xr = X + row * RW_LDG + 32 * h;
-#pragma unroll
-                for (int c4 = 0; c4 < 8; ++c4) {
-                    const float4 v = *reinterpret_cast<const float4 *>(xr + 4 * c4);
-                    const int k = 32 * h + 4 * c4;
-                    Y[k * RW_LDT + row] = v.x;
-                    Y[(k + 1) * RW_LDT + row] = v.y;
-                    Y[(k + 2) * RW_LDT + row] = v.z;
-                    Y[(k + 3) * RW_LDT + row] = v.w;
-                }
-            }
-            __syncthreads();
-            // forward layers: G (Y) -> a_1 (X); the last one also forms E_a
-            // and dz_L = w act'(a_L): L = 1 writes dz_1 into X, L = 2 writes
-            // dz_2 into Y (G is dead)
-            for (int l = 0; l < L; ++l) {
-                const float *Ain = (l == 0) ? Y : X;
-                float *Cout = (l == 0) ? X : Y;
-                rw_product<false>(Ain, sW + l * RW_WF, rb, cb, acc);
-                const float4 bv = *reinterpret_cast<const float4 *>(sBias + l * RW_N + 4 * cb);
-                const float bias[4] = {bv.x, bv.y, bv.z, bv.w};
-                if (l < L - 1) {
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        float v[8];
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) v[i] = act_f(act, acc[i][c] + bias[c], spb);
-                        rw_store_col(Cout, 4 * cb + c, rb, v);
-                    }
-                    __syncthreads();
-                } else {
-                    const float4 wv = *reinterpret_cast<const float4 *>(sWout + 4 * cb);
-                    const float wout[4] = {wv.x, wv.y, wv.z, wv.w};
-                    float ep[8];
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) ep[i] = 0.f;
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        float v[8];
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            const float a = act_f(act, acc[i][c] + bias[c], spb);
-                            ep[i] = fmaf(a, wout[c], ep[i]);
-                            v[i] = wout[c] * act_da(act, a, spb);
-                        }
-                        rw_store_col(Cout, 4 * cb + c, rb, v);
-                    }
-                    // E partials over this thread's 4 columns -> the 4 column
-                    // groups of the warp (lanes 8 apart) -> the 4 warp pairs
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        ep[i] += __shfl_xor_sync(0xffffffffu, ep[i], 8);
-                        ep[i] += __shfl_xor_sync(0xffffffffu, ep[i], 16);
-                    }
-                    if ((lane >> 3) == 0) {
-                        float *e = sEp + (warp >> 1) * RW_TR + 4 * rb;
-                        *reinterpret_cast<float4 *>(e) = make_float4(ep[0], ep[1], ep[2], ep[3]);
-                        *reinterpret_cast<float4 *>(e + 64) = make_float4(ep[4], ep[5], ep[6], ep[7]);
-                    }
-                    __syncthreads();
-                    if (tid < RW_TR && s_type[tid] == s) {
-                        const float e = ((sEp[tid] + sEp[RW_TR + tid]) + (sEp[2 * RW_TR + tid] + sEp[3 * RW_TR + tid])) +
-                                        sBout[0];
-                        s_e[tid] = e;
-                        if (e_atom) e_atom[s_atom[tid]] = e;
-                    }
-                }
-            }
-            // L = 2: dz_1 = (dz_2 W_1^T) act'(a_1), written over a_1 (each
-            // thread reads and writes only its own block)
-            if (L == 2) {
-                rw_product<true>(Y, sW + RW_WF, rb, cb, acc);
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    const float *cp = X + (4 * cb + c) * RW_LDT + 4 * rb;
-                    const float4 a0 = *reinterpret_cast<const float4 *>(cp);
-                    const float4 a1 = *reinterpret_cast<const float4 *>(cp + 64);
-                    const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-                    float v[8];
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) v[i] = acc[i][c] * act_da(act, av[i], spb);
-                    rw_store_col(X, 4 * cb + c, rb, v);
-                }
-                __syncthreads();
-            }
-            // Y is free from here on: the next tile's G rows go there while
-            // the last product runs
-            if (s == s_hi && more) {
-                rw_stage_g(G, p0 + RW_TR, n, Y);
-                if (next_a >= 0) next_ty = types[next_a];
-            }
-            // G' = dz_1 W_0^T -> dG rows of species s (perm position)
-            rw_product<true>(X, sW, rb, cb, acc);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int row = (i < 4) ? 4 * rb + i : 64 + 4 * rb + (i - 4);
-                if (s_type[row] == s)
-                    *reinterpret_cast<float4 *>(dG + (size_t)(p0 + row) * RW_N + 4 * cb) =
-                        make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
-            }
-        }
-        if (more) publish(xb ^ 1, next_a, next_ty);
-        __syncthreads();   // every thread is done with X and s_e; the next tile's atoms are visible
-        if (warp == 0) {   // tile energy in FP64, fixed order
-            double t = 0.0;
-            for (int r = lane; r < RW_TR; r += 32) t += (double)s_e[r];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-            if (lane == 0) part_e[tile] = t;
-        }
-        xb ^= 1;
-    }
-    asm volatile("cp.async.wait_all;\n" ::);
-}
-
-// ---------------------------------------------------------------------------
 // network on BF16 tensor cores (FP32 accumulation): the same forward / input-
 // gradient chain as k_mlp for a 64-atom tile.  Eight warps: warp w owns rows
 // 16 (w % 4) .. + 16 and one half of each weight chunk's output columns, and
@@ -1205,22 +868,17 @@ size_t mlp_smem_bytes(const DevModel &dm) { return mlp_smem_tr(dm, mlp_tr(dm)); 
 
 size_t mlp_smem_tr_public(const DevModel &dm, int tr) { return mlp_smem_tr(dm, tr); }
 
-// the resident-weight FP32 network applies: descriptor length and hidden
-// widths all 64, one or two hidden layers, 16-byte aligned weight rows
-static bool mlp_res_ok(const DevModel &dm) {
-    if (dm.precision != TMD_PREC_FP32 || dm.L < 1 || dm.L > RW_MAXL || dm.dims[dm.L + 1] != 1) return false;
+// descriptor length and hidden widths all 64, one or two hidden layers: the
+// networks for which tile_rows 128 is a choice
+static bool mlp_all64(const DevModel &dm) {
+    if (dm.precision != TMD_PREC_FP32 || dm.L < 1 || dm.L > 2) return false;
     for (int l = 0; l <= dm.L; ++l)
-        if (dm.dims[l] != RW_N || dm.off_f[l] % 4 != 0) return false;
-    for (int s = 0; s < dm.S; ++s)
-        if (reinterpret_cast<uintptr_t>(dm.wf[s]) % 16 != 0) return false;
+        if (dm.dims[l] != 64) return false;
     return true;
 }
 
-// tile_rows 0 (built-in choice) or 128 selects it where it applies
-static bool mlp_use_res(const DevModel &dm) { return (dm.tile_rows == 0 || dm.tile_rows == RW_TR) && mlp_res_ok(dm); }
-
 bool mlp_rows_ok(const DevModel &dm, int tr) {
-    if (tr == RW_TR) return mlp_res_ok(dm);
+    if (tr == 128) return mlp_all64(dm);
     return (tr == 32 || tr == 64) && mlp_smem_tr(dm, tr) <= 227 * 1024;
 }
 
@@ -1268,7 +926,6 @@ static tmd_status set_mlp_smem(const DevModel &dm, bool bf16) {
         }
         return TMD_OK;
     }
-    if (mlp_use_res(dm)) return TMD_OK;   // k_mlp_res sets its own
     const int tr = mlp_tr(dm);
     const size_t smem = mlp_smem_bytes(dm);
     size_t &done = smem_set[tr == 64 ? 1 : 0];
@@ -1292,6 +949,15 @@ static tmd_status launch_network(const DevModel &dm, const int32_t *perm, const 
         set_error("the tcgen05 network kernel does not support these network shapes");
         return TMD_ERR_UNIMPLEMENTED;
     }
+    // FP32: the tensor cores wherever the widths are multiples of 16 up to 128
+    // and a tile fits on chip; k_mlp has the rest.  At every size: one 32-atom
+    // tile 15.5 us against 15.6 in k_mlp, 1,048,576 atoms x 64-64 423 us
+    // against 850, 147,456 atoms x 128-128-128 254 us against 922 (k_mlp).
+    // Two labels, as tile_rows has two kinds of tile: "k_mlp_res" where 0 or
+    // 128 stands for 128-atom tiles, else "k_mlp".
+    if (mlp_tf32_ok(dm))
+        return mlp_tf32_launch(mlp_all64(dm) && (dm.tile_rows == 0 || dm.tile_rows == 128) ? "k_mlp_res" : "k_mlp", dm,
+                               perm, types, n, G, dG, e_atom, part_e, ntile_out, s);
     if ((st = set_mlp_smem(dm, dm.precision == TMD_PREC_BF16)) != TMD_OK) return st;
     if (dm.precision == TMD_PREC_BF16) {
         const int ntile = (int)((n + BT - 1) / BT);
@@ -1299,22 +965,6 @@ static tmd_status launch_network(const DevModel &dm, const int32_t *perm, const 
         TMD_LAUNCH("k_mlp_bf16", s, k_mlp_bf16<<<ntile, BF_THREADS, mlp_bf16_smem_bytes(dm), s>>>(
                                         dm, perm, types, n, G, dG, e_atom, part_e, bcfg.bnc, bcfg.compact ? 1 : 0));
         *ntile_out = ntile;
-    } else if (mlp_use_res(dm)) {
-        static int per_sm = 0, nsm = 0;   // resident blocks of k_mlp_res per SM
-        if (!per_sm) {
-            const int smem = (int)(RW_SMEM_FLOATS * sizeof(float));
-            TMD_CUDA(cudaFuncSetAttribute(k_mlp_res, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-            int dev = 0;
-            TMD_CUDA(cudaGetDevice(&dev));
-            TMD_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-            TMD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_mlp_res, RW_THREADS, smem));
-            per_sm = std::max(per_sm, 1);
-        }
-        const int64_t ntile = (n + RW_TR - 1) / RW_TR;
-        const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(ntile, (int64_t)per_sm * nsm));
-        TMD_LAUNCH("k_mlp_res", s, k_mlp_res<<<grid, RW_THREADS, RW_SMEM_FLOATS * sizeof(float), s>>>(
-                                       dm, perm, types, n, G, dG, e_atom, part_e));
-        *ntile_out = (int)ntile;
     } else {
         const int tr = mlp_tr(dm);
         const int ntile = (int)((n + tr - 1) / tr);
