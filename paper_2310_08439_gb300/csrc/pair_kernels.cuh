@@ -23,11 +23,9 @@
 // the pair cache (filled by k_screen in screen.cu, read by both passes) or,
 // without a cache, from screening the table in the pass itself, compacted
 // through a per-warp shared-memory queue; either way every lane works on an
-// in-cutoff pair.  Each lane computes H and M for one
-// neighbour and stages them in shared memory; the warp then accumulates the
-// per-atom P[b][k][d] outer products with each lane owning a (K/8 x 4) block
-// of P in registers.  In k_force each lane owns one cached pair and reads the
-// atom's P' from shared memory with broadcast loads.
+// in-cutoff pair.  k_desc: the pairs' geometry is staged in shared memory and
+// the sums run on the tensor cores.  k_force: a lane owns one or two pairs and
+// reads the atom's P' from shared memory with broadcast loads.
 //
 // Templates over the radial channel count K and the species count S; each
 // pair_k<K>.cu translation unit instantiates one K (compiled in parallel).
@@ -289,12 +287,11 @@ __device__ __forceinline__ void pair_geom(const float4 jh, const float4 jl, cons
 // Used when there is no pair cache (k_screen in screen.cu fills the cache
 // with the same pairs, in the same order, by the same arithmetic).
 //
-// f(q, q2, nb) takes the first nb pairs of the queue (nb = 32 NL but for the
+// f(q, q2, nb) takes the first nb pairs of the queue (nb = NB but for the
 // atom's last batch).
-template <int NL, typename F>
+template <int NB, typename F>
 __device__ __forceinline__ void queue_pairs(const DevNlist &nl, int a, int64_t beg, int64_t end, float rc2h, float rc2l,
                                             float4 *q, float2 *q2, int lane, F &&f) {
-    constexpr int NB = 32 * NL;
     int qn = 0;
     const unsigned lt = (1u << lane) - 1u;
     const float4 ih = nl.ph[a], il = nl.pl[a];
@@ -338,31 +335,6 @@ __device__ __forceinline__ void queue_pairs(const DevNlist &nl, int a, int64_t b
         }
         __syncwarp();
         qn -= nb;
-    }
-}
-
-// the same, one pair per lane: f(pair, r^2, valid, nb)
-template <typename F>
-__device__ __forceinline__ void for_pairs(const DevNlist &nl, int a, int64_t beg, int64_t end, float rc2h, float rc2l,
-                                          float4 *q, float2 *q2, int lane, F &&f) {
-    queue_pairs<1>(nl, a, beg, end, rc2h, rc2l, q, q2, lane,
-                   [&](const float4 *p, const float2 *p2, int nb) { f(p[lane], p2[lane], lane < nb, nb); });
-}
-
-// The in-cutoff pairs of atom a from the pair cache written by k_screen, in
-// batches of up to 32 (one per lane).
-template <typename F>
-__device__ __forceinline__ void cached_pairs(const DevNlist &nl, int a, int np, int lane, F &&f) {
-    const int64_t pb = nl.beg[a];
-    for (int base = 0; base < np; base += 32) {
-        const int nb = min(32, np - base);
-        float4 e = make_float4(0.f, 0.f, 0.f, 0.f);
-        float2 e2 = make_float2(1.f, 0.f);
-        if (lane < nb) {
-            e = nl.pq[pb + base + lane];
-            e2 = nl.pq2[pb + base + lane];
-        }
-        f(e, e2, lane < nb, nb);
     }
 }
 
@@ -727,7 +699,7 @@ __global__ void __launch_bounds__(PW * 32, desc_min_blocks(S * K)) k_desc(DevMod
             }
             if (ps.np == 0) ps.advance(nl, 0, lane);
         } else {
-            queue_pairs<2>(nl, a, nl.beg[a], nl.end[a], m.rc2h, m.rc2l, s_q[warp], s_q2[warp], lane,
+            queue_pairs<64>(nl, a, nl.beg[a], nl.end[a], m.rc2h, m.rc2l, s_q[warp], s_q2[warp], lane,
                            [&](const float4 *p, const float2 *p2, int nb) {
                                pair_fn(load_two(p, p2, 2 * lane, nb), nb);
                            });
@@ -887,6 +859,67 @@ __device__ __forceinline__ void pair_grad(const DevModel &m, const float4 e, con
     pair_grad_tail(V2, W2, ux, uy, uz, ir, gxs, gys, gzs);
 }
 
+// V_c = sum_k A'_kc H_k and W_c = sum_k A'_kc H'_k of two in-cutoff pairs
+// of one atom with neighbours of one species (Eqs. dP_abkd, U_abck, F1_abcx,
+// F2_abcx), as packed pairs (c, c + 1): every multiply-add of the channel loop
+// is one FP32x2 instruction (each half rounded as fmaf).  Pb = the atom's A' for
+// the neighbours' species, rad = the channels of the (centre, neighbour) species
+// pair in the packed layout of stage_rad2.
+template <int K, bool TAB>
+__device__ __forceinline__ void pair_sums2(const DevModel &m, const float (&rh)[2], const float (&rl)[2], const float *Pb,
+                                            const float4 *rad, const float *tab, float2 (&V)[2][NHAR / 2],
+                                           float2 (&W)[2][NHAR / 2]) {
+    TabCell tc[2];
+    float2 fc[2], dfc[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+#pragma unroll
+        for (int d = 0; d < NHAR / 2; ++d) V[i][d] = W[i][d] = make_float2(0.f, 0.f);
+        if (TAB) {
+            tc[i] = tab_cell(tab, K, m.rtab_scale, rh[i], rl[i]);
+        } else {
+            float c, d;
+            cutoff_fn(rh[i], m.inv_rc, c, d);
+            fc[i] = bc2(c);
+            dfc[i] = bc2(d);
+        }
+    }
+    constexpr int KU = K > 32 ? 16 : K;   // channels per unrolled block
+#pragma unroll 1
+    for (int kb = 0; kb < K; kb += KU)
+#pragma unroll
+    for (int ku = 0; ku < KU; ku += 2) {
+        const int k = kb + ku;
+        // H and H' of channels k, k + 1 formed inside the loop (no per-pair arrays)
+        float2 H[2], dH[2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            if (TAB) {
+                tab_eval(tc[i], k, m.rtab_scale, H[i].x, dH[i].x);
+                tab_eval(tc[i], k + 1, m.rtab_scale, H[i].y, dH[i].y);
+            } else {
+                const Radial2 o = radial2<true>(rad, k, bc2(rh[i]), bc2(rl[i]), fc[i], dfc[i]);
+                H[i] = o.H;
+                dH[i] = o.dH;
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+#pragma unroll
+            for (int q4 = 0; q4 < NHAR / 4; ++q4) {
+                const float4 pd = *reinterpret_cast<const float4 *>(Pb + (k + c) * NHAR + 4 * q4);
+                const float2 plo = make_float2(pd.x, pd.y), phi = make_float2(pd.z, pd.w);
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const float2 h2 = bc2(c ? H[i].y : H[i].x), d2 = bc2(c ? dH[i].y : dH[i].x);
+                    V[i][2 * q4] = __ffma2_rn(plo, h2, V[i][2 * q4]);
+                    V[i][2 * q4 + 1] = __ffma2_rn(phi, h2, V[i][2 * q4 + 1]);
+                    W[i][2 * q4] = __ffma2_rn(plo, d2, W[i][2 * q4]);
+                    W[i][2 * q4 + 1] = __ffma2_rn(phi, d2, W[i][2 * q4 + 1]);
+                }
+            }
+    }
+}
 
 // A'_bkc = dE/dA_bkc (Eq. dP_abkd) of the atom at perm position p (A and G'
 // are indexed by perm position) into a shared slot, each lane its (K/8 x 4)
@@ -940,6 +973,9 @@ __device__ __forceinline__ void virial_flush(float (&wacc)[9], double *acc, int 
 // contiguous run of atoms (perm order) and fills every batch of 32 lanes with
 // the rest of the current atom's pairs followed by the first pairs of the
 // next atom (two P' slots per warp, two self-force accumulators).
+// For one species: there it is the faster one (1,048,576 atoms, K = 16, 54
+// pairs: 2.06 ms, k_force 2.10; 39,366 atoms, K = 128: 0.63, k_force 0.70; only
+// K = 32 is 4 % the other way).  Two pairs per lane in this form: 2.37 ms.
 template <int K, int S, bool TAB>
 __global__ void __launch_bounds__(PW * 32, 4) k_force_merged(DevModel m, DevNlist nl, const int32_t *__restrict__ types,
                                                           const float *__restrict__ Pin, const float *__restrict__ dG,
@@ -1267,112 +1303,187 @@ __global__ void __launch_bounds__(PW * 32, 4) k_force_tc(DevModel m, DevNlist nl
     }
 }
 
-// PAW (batched): each atom's virial is summed over its own pairs and written
-// to w_atom [atoms][9] for per-system reductions; otherwise lanes keep
-// compensated running sums and each block writes one FP64 partial.
+// Force pass: A' = dE/dA of every atom, g_ij = dE/dD_ij of its pairs, the
+// ScatterSum of g_ij and the virial.  One warp per atom.  Batches of up to BF
+// pairs, two neighbouring places per lane: pairs of one species, so that a lane
+// reads each A' value once for both (more than one species: the batch is put in
+// shared memory in groups of the neighbour species, padded to even length); up
+// to 32 remaining pairs go one per lane.
+//
+// What bounds it: the A' values of the channel loop.  16 floats a channel and
+// lane take the data path of shared memory 4 cycles for each 16 bytes a lane,
+// for one pair per lane more than their multiply-adds take the FP32 pipes
+// (without these loads the pass runs in 1.29 ms instead of 2.1 at 1,048,576
+// atoms, K = 16).  A batch passes through shared memory also with one species:
+// pairs read from global memory stay in registers over the channel loop, which
+// then spills (2.99 ms against 2.10).  Measured, one pair per lane -> two:
+// 16,384 atoms, 2 species, K = 16, 78 pairs: 87 -> 66 us; 225,008 atoms in 128
+// systems, 3 species, 54 pairs: 0.76 -> 0.67 ms; 93,802 atoms in 24 systems, 2
+// species: 0.40 -> 0.33 ms; table screened in the pass, 8,160 atoms: 46 -> 41 us.
+//
+// CACHED: the pairs are those of the pair cache, else the table is screened
+// here.  PAW (batched): each atom's virial is summed over its own pairs and
+// written to w_atom [atoms][9] for per-system reductions; otherwise each block
+// writes one FP64 partial.
 template <int K, int S, bool PAW, bool CACHED, bool TAB>
-__global__ void __launch_bounds__(PW * 32, 4) k_force(DevModel m, DevNlist nl, const double *__restrict__ pos,
-                                                   const int32_t *__restrict__ types, const float *__restrict__ Pin,
-                                                   const float *__restrict__ dG,
+__global__ void __launch_bounds__(PW * 32, 4) k_force(DevModel m, DevNlist nl, const int32_t *__restrict__ types,
+                                                   const float *__restrict__ Pin, const float *__restrict__ dG,
                                                    unsigned long long *__restrict__ Fq,
                                                    double *__restrict__ part_w, float *__restrict__ w_atom) {
-    constexpr int PSTR = K * NHAR + 4;   // per-species stride of P' (bank offset between species)
+    constexpr int PSTR = K * NHAR + 4;   // per-species stride of A' (bank offset between species)
+    constexpr int BF = S == 1 ? 64 : (64 - S) & ~1;
+    constexpr bool QUEUE = !CACHED;
     __shared__ float4 s_rad[S * S * K];
-    __shared__ float4 s_q[PW][64];
-    __shared__ float2 s_q2[PW][64];
+    __shared__ float4 s_q[QUEUE ? PW : 1][QUEUE ? 96 : 1];
+    __shared__ float2 s_q2[QUEUE ? PW : 1][QUEUE ? 96 : 1];
+    constexpr bool STAGE = S > 1 || CACHED;
+    __shared__ float4 s_g[STAGE ? PW : 1][STAGE ? 64 : 1];   // a batch in species groups
+    __shared__ float2 s_g2[STAGE ? PW : 1][STAGE ? 64 : 1];
     __shared__ __align__(16) float s_Pd[PW][S * PSTR];
     __shared__ double s_w[PW][9];
     stage_rad2(s_rad, m.radial, S * S * K);
-    __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (lane < 9) s_w[warp][lane] = 0.0;
+    __syncthreads();
     const int kg = lane >> 2, g = lane & 3;
+    const unsigned lt = (1u << lane) - 1u;
     float Wg[4];
 #pragma unroll
     for (int dd = 0; dd < 4; ++dd) Wg[dd] = c_W[4 * g + dd];
-    float wsum[9], wcmp[9];
+    float wacc[9];   // virial: this lane's pairs of the atom (PAW) or of up to VFLUSH atoms
 #pragma unroll
-    for (int t = 0; t < 9; ++t) { wsum[t] = 0.f; wcmp[t] = 0.f; }
-    float *sPd = s_Pd[warp];
-    const int64_t total = (int64_t)gridDim.x * PW;
-    for (int64_t p = (int64_t)blockIdx.x * PW + warp; p < nl.n; p += total) {
-        const int a = nl.perm[p];
-        const int ti = types[a];
+    for (int t = 0; t < 9; ++t) wacc[t] = 0.f;
+    int since = 0;
+    float *const sPd = s_Pd[warp];
+    const int nw = (int)gridDim.x * PW;
+    int p = (int)blockIdx.x * PW + warp;
+    const int n = (int)nl.n;
+    int a = p < n ? nl.perm[p] : -1;
+    while (a >= 0) {
+        const int an = p + nw < n ? nl.perm[p + nw] : -1;
+        const int ti = S > 1 ? types[a] : 0;
+        const int64_t pb = nl.beg[a];
+        const int np = CACHED ? nl.npair[a] : 0;
         pprime_setup<K, S>(Pin, dG, p, sPd, kg, g, Wg);
         __syncwarp();
         long long fx = 0, fy = 0, fz = 0;
-        float wa[9];  // this lane's pairs of this atom
+        auto scatter = [&](float gx, float gy, float gz, const float4 e) {
+            // ScatterSum in 2^-32 fixed point: integer adds are exact and
+            // order independent, so forces are bitwise reproducible.
+            const long long qx = to_fixed(gx), qy = to_fixed(gy), qz = to_fixed(gz);
+            fx += qx; fy += qy; fz += qz;
+            unsigned long long *const Fj = Fq + 3 * (int64_t)(__float_as_uint(e.w) & 0x0FFFFFFFu);
+            atomicAdd(Fj, (unsigned long long)(-qx));
+            atomicAdd(Fj + 1, (unsigned long long)(-qy));
+            atomicAdd(Fj + 2, (unsigned long long)(-qz));
+            const float D[3] = {e.x, e.y, e.z};
+            const float gv[3] = {gx, gy, gz};
 #pragma unroll
-        for (int t = 0; t < 9; ++t) wa[t] = 0.f;
-        auto pair_fn = [&](const float4 e, const float2 e2, bool valid, int) {
-                      if (!valid) return;
-                      const uint32_t jb = __float_as_uint(e.w);
-                      const int b = (int)(jb >> 28);
-                      const int j = (int)(jb & 0x0FFFFFFFu);
-                      float gxs, gys, gzs;
-                      pair_grad<K, TAB>(m, e, e2, sPd + b * PSTR, &s_rad[(ti * S + b) * K],
-                                        TAB ? m.rtab + (size_t)(ti * S + b) * m.rtab_n * 4 * K : nullptr, gxs, gys, gzs);
-                      // ScatterSum in 2^-32 fixed point: integer adds are exact and
-                      // order independent, so forces are bitwise reproducible.
-                      const long long qx = to_fixed(gxs);
-                      const long long qy = to_fixed(gys);
-                      const long long qz = to_fixed(gzs);
-                      fx += qx; fy += qy; fz += qz;
-                      atomicAdd(&Fq[3 * (int64_t)j], (unsigned long long)(-qx));
-                      atomicAdd(&Fq[3 * (int64_t)j + 1], (unsigned long long)(-qy));
-                      atomicAdd(&Fq[3 * (int64_t)j + 2], (unsigned long long)(-qz));
-                      const float D[3] = {e.x, e.y, e.z};
-                      const float gv[3] = {gxs, gys, gzs};
+            for (int al = 0; al < 3; ++al)
 #pragma unroll
-                      for (int al = 0; al < 3; ++al)
+                for (int be = 0; be < 3; ++be) wacc[al * 3 + be] = fmaf(-D[al], gv[be], wacc[al * 3 + be]);
+        };
+        // the nb pairs at q, q2: in shared memory or in the cache
+        auto batch = [&](const float4 *q, const float2 *q2, int nb) {
+            if (nb <= 32) {   // one pair per lane
+                if (lane < nb) {
+                    const float4 e = q[lane];
+                    const int b = S > 1 ? (int)(__float_as_uint(e.w) >> 28) : 0;
+                    float gx, gy, gz;
+                    pair_grad<K, TAB>(m, e, q2[lane], sPd + b * PSTR, &s_rad[(ti * S + b) * K],
+                                      TAB ? m.rtab + (size_t)(ti * S + b) * m.rtab_n * 4 * K : nullptr, gx, gy, gz);
+                    scatter(gx, gy, gz, e);
+                }
+                return;
+            }
+            int b = 0, n0 = nb;   // this lane's species group, the end of its pairs
+            if constexpr (S == 1 && STAGE) {
+                s_g[warp][lane] = q[lane];
+                s_g2[warp][lane] = q2[lane];
+                if (lane + 32 < nb) {
+                    s_g[warp][lane + 32] = q[lane + 32];
+                    s_g2[warp][lane + 32] = q2[lane + 32];
+                }
+                q = s_g[warp];
+                q2 = s_g2[warp];
+                __syncwarp();
+            } else if constexpr (S > 1) {
+                const bool two = lane + 32 < nb;
+                const float4 e0 = q[lane], e1 = q[two ? lane + 32 : lane];
+                const float2 f0 = q2[lane], f1 = q2[two ? lane + 32 : lane];
+                const int b0 = (int)(__float_as_uint(e0.w) >> 28), b1 = two ? (int)(__float_as_uint(e1.w) >> 28) : S;
+                int start = 0;
+                n0 = 0;
 #pragma unroll
-                          for (int be = 0; be < 3; ++be) wa[al * 3 + be] = fmaf(-D[al], gv[be], wa[al * 3 + be]);
-                  };
-        if constexpr (CACHED)
-            cached_pairs(nl, a, nl.npair[a], lane, pair_fn);
-        else
-            for_pairs(nl, a, nl.beg[a], nl.end[a], m.rc2h, m.rc2l, s_q[warp], s_q2[warp], lane, pair_fn);
+                for (int s = 0; s < S; ++s) {
+                    const unsigned m0 = __ballot_sync(0xffffffffu, b0 == s), m1 = __ballot_sync(0xffffffffu, b1 == s);
+                    const int c0 = start + __popc(m0 & lt), c1 = start + __popc(m0) + __popc(m1 & lt);
+                    if (b0 == s) { s_g[warp][c0] = e0; s_g2[warp][c0] = f0; }
+                    if (b1 == s) { s_g[warp][c1] = e1; s_g2[warp][c1] = f1; }
+                    const int cnt = __popc(m0) + __popc(m1);
+                    if (2 * lane >= start && 2 * lane < start + cnt) { b = s; n0 = start + cnt; }
+                    start += (cnt + 1) & ~1;
+                }
+                q = s_g[warp];
+                q2 = s_g2[warp];
+                __syncwarp();
+            }
+            const int i0 = 2 * lane;
+            if (i0 < n0) {
+                const bool two = i0 + 1 < n0;
+                const float2 ra = q2[i0], rb = q2[two ? i0 + 1 : i0];
+                float2 rh, rl, ir;
+                split_sqrt2(make_float2(ra.x, rb.x), make_float2(ra.y, rb.y), rh, rl, ir);
+                float2 V[2][NHAR / 2], W[2][NHAR / 2];
+                const float rhx[2] = {rh.x, rh.y}, rlx[2] = {rl.x, rl.y};
+                pair_sums2<K, TAB>(m, rhx, rlx, sPd + b * PSTR, &s_rad[(ti * S + b) * K],
+                                     TAB ? m.rtab + (size_t)(ti * S + b) * m.rtab_n * 4 * K : nullptr, V, W);
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+                    if (i == 0 || two) {
+                        const float4 e = q[i0 + i];
+                        const float r1 = i ? ir.y : ir.x;
+                        float gx, gy, gz;
+                        pair_grad_tail(V[i], W[i], e.x * r1, e.y * r1, e.z * r1, r1, gx, gy, gz);
+                        scatter(gx, gy, gz, e);
+                    }
+            }
+            if (STAGE) __syncwarp();   // the groups are rewritten by the next batch
+        };
+        if constexpr (CACHED) {
+            for (int base = 0; base < np; base += BF) batch(nl.pq + pb + base, nl.pq2 + pb + base, min(BF, np - base));
+        } else {
+            queue_pairs<BF>(nl, a, pb, nl.end[a], m.rc2h, m.rc2l, s_q[warp], s_q2[warp], lane, batch);
+        }
         fx = warp_sum_fixed(fx);
         fy = warp_sum_fixed(fy);
         fz = warp_sum_fixed(fz);
-        if (lane == 0) {
-            atomicAdd(&Fq[3 * (int64_t)a], (unsigned long long)fx);
-            atomicAdd(&Fq[3 * (int64_t)a + 1], (unsigned long long)fy);
-            atomicAdd(&Fq[3 * (int64_t)a + 2], (unsigned long long)fz);
-        }
+        if (lane < 3) atomicAdd(&Fq[3 * (int64_t)a + lane], (unsigned long long)(lane == 0 ? fx : (lane == 1 ? fy : fz)));
         if constexpr (PAW) {
 #pragma unroll
             for (int t = 0; t < 9; ++t) {
-                float v = wa[t];
+                float v = wacc[t];
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
                 if (lane == 0) w_atom[(size_t)a * 9 + t] = v;
+                wacc[t] = 0.f;
             }
-        } else {
-#pragma unroll
-            for (int t = 0; t < 9; ++t) kahan_add(wsum[t], wcmp[t], wa[t]);
+        } else if (++since == VFLUSH) {
+            virial_flush(wacc, s_w[warp], lane);
+            since = 0;
         }
-        __syncwarp();
+        __syncwarp();   // A' is rewritten by the next atom
+        p += nw;
+        a = an;
     }
-    // virial: per-lane compensated sums (value = sum - comp) -> warp total as
-    // an FP32 double-float (error-free additions) -> FP64 block total
-#pragma unroll
-    for (int t = 0; t < 9; ++t) {
-        float hi = wsum[t], lo = -wcmp[t];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const float oh = __shfl_xor_sync(0xffffffffu, hi, o), ol = __shfl_xor_sync(0xffffffffu, lo, o);
-            float sh, se;
-            two_sum(hi, oh, sh, se);
-            lo = (lo + ol) + se;
-            two_sum(sh, lo, hi, lo);
+    if (!PAW) {
+        virial_flush(wacc, s_w[warp], lane);
+        __syncthreads();
+        if (threadIdx.x < 9) {
+            double v = 0.0;
+            for (int w = 0; w < PW; ++w) v += s_w[w][threadIdx.x];
+            part_w[(size_t)blockIdx.x * 9 + threadIdx.x] = v;
         }
-        if (lane == 0) s_w[warp][t] = (double)hi + (double)lo;
-    }
-    __syncthreads();
-    if (!PAW && threadIdx.x < 9) {
-        double v = 0.0;
-        for (int w = 0; w < PW; ++w) v += s_w[w][threadIdx.x];
-        part_w[(size_t)blockIdx.x * 9 + threadIdx.x] = v;
     }
 }
 
@@ -1405,6 +1516,13 @@ void launch_desc(const DevModel &dm, const DevNlist &dn, const double *pos, cons
     TMD_LAUNCH("k_desc", s, k_desc<K, S, TAB, CACHED><<<nb, PW * 32, 0, s>>>(dm, dn, pos, types, nl->G, nl->P));
 }
 
+template <int K, int S, bool PAW, bool CACHED, bool TAB>
+void launch_force(const DevModel &dm, const DevNlist &dn, const double *pos, const int32_t *types, tmd_nlist *nl,
+                  double *part_w, int nblk, cudaStream_t s, float *w_atom) {
+    TMD_LAUNCH("k_force", s, k_force<K, S, PAW, CACHED, TAB><<<nblk, PW * 32, 0, s>>>(dm, dn, types, nl->P, nl->dG,
+                                                                                   nl->Fq, part_w, w_atom));
+}
+
 template <int K, int S>
 tmd_status launch_pair_kernels(const DevModel &dm, const DevNlist &dn, const double *pos, const int32_t *types,
                                tmd_nlist *nl, double *part_w, int nblk, cudaStream_t s, bool forward,
@@ -1419,11 +1537,9 @@ tmd_status launch_pair_kernels(const DevModel &dm, const DevNlist &dn, const dou
     else if (forward)
         launch_desc<K, S, false, false>(dm, dn, pos, types, nl, nblk, s);
     else if (w_atom && dm.rtab)   // batched evaluations always run with the pair cache
-        TMD_LAUNCH("k_force", s, k_force<K, S, true, true, true><<<nblk, PW * 32, 0, s>>>(dm, dn, pos, types, nl->P,
-                                                                                        nl->dG, nl->Fq, part_w, w_atom));
+        launch_force<K, S, true, true, true>(dm, dn, pos, types, nl, part_w, nblk, s, w_atom);
     else if (w_atom)
-        TMD_LAUNCH("k_force", s, k_force<K, S, true, true, false><<<nblk, PW * 32, 0, s>>>(dm, dn, pos, types, nl->P,
-                                                                                         nl->dG, nl->Fq, part_w, w_atom));
+        launch_force<K, S, true, true, false>(dm, dn, pos, types, nl, part_w, nblk, s, w_atom);
     // the tensor-core pass reads the pair cache; an evaluation without one
     // (the allocation-free call) runs the SIMT pass whatever the setting
     else if (force_kernel() == TMD_FORCE_TENSOR && dn.pq && !(!dm.rtab && S == 1 && K <= 32)) {
@@ -1432,18 +1548,23 @@ tmd_status launch_pair_kernels(const DevModel &dm, const DevNlist &dn, const dou
     } else if (force_kernel() == TMD_FORCE_TENSOR && dn.pq) {
         if constexpr (S == 1 && K <= 32)
             TMD_LAUNCH("k_force", s, k_force_tc<K><<<nblk, PW * 32, 0, s>>>(dm, dn, nl->P, nl->dG, nl->Fq, part_w));
-    } else if (dn.pq && dm.rtab)
-        TMD_LAUNCH("k_force", s, k_force_merged<K, S, true><<<nblk, PW * 32, 0, s>>>(dm, dn, types, nl->P, nl->dG,
-                                                                                   nl->Fq, part_w));
-    else if (dn.pq)
-        TMD_LAUNCH("k_force", s, k_force_merged<K, S, false><<<nblk, PW * 32, 0, s>>>(dm, dn, types, nl->P, nl->dG,
-                                                                                    nl->Fq, part_w));
+    } else if (dn.pq && dm.rtab) {
+        if constexpr (S == 1)
+            TMD_LAUNCH("k_force", s, k_force_merged<K, S, true><<<nblk, PW * 32, 0, s>>>(dm, dn, types, nl->P, nl->dG,
+                                                                                       nl->Fq, part_w));
+        else
+            launch_force<K, S, false, true, true>(dm, dn, pos, types, nl, part_w, nblk, s, nullptr);
+    } else if (dn.pq) {
+        if constexpr (S == 1)
+            TMD_LAUNCH("k_force", s, k_force_merged<K, S, false><<<nblk, PW * 32, 0, s>>>(dm, dn, types, nl->P, nl->dG,
+                                                                                        nl->Fq, part_w));
+        else
+            launch_force<K, S, false, true, false>(dm, dn, pos, types, nl, part_w, nblk, s, nullptr);
+    }
     else if (dm.rtab)
-        TMD_LAUNCH("k_force", s, k_force<K, S, false, false, true><<<nblk, PW * 32, 0, s>>>(dm, dn, pos, types, nl->P,
-                                                                                          nl->dG, nl->Fq, part_w, nullptr));
+        launch_force<K, S, false, false, true>(dm, dn, pos, types, nl, part_w, nblk, s, nullptr);
     else
-        TMD_LAUNCH("k_force", s, k_force<K, S, false, false, false><<<nblk, PW * 32, 0, s>>>(dm, dn, pos, types, nl->P,
-                                                                                           nl->dG, nl->Fq, part_w, nullptr));
+        launch_force<K, S, false, false, false>(dm, dn, pos, types, nl, part_w, nblk, s, nullptr);
     TMD_CUDA(cudaGetLastError());
     return TMD_OK;
 }
