@@ -15,7 +15,16 @@
 // row per thread; the two warps of a TMEM lane quarter take alternate
 // 16-column blocks), apply bias and activation, keep act' in TMEM for the
 // backward chain (tcgen05.st) and write the BF16 operand of the next product.
-// One elected thread issues the MMAs and the copies.
+// One warp issues the MMAs and another the copies, with one elected lane at the
+// instructions (elect_one).
+//
+// Bound by the chain of a tile: staging, product, epilogue, each waiting on the
+// one before, with one block on an SM when the tensor memory is full (K = 128:
+// 512 columns) and two to four otherwise.  Measured: 39,366 atoms x
+// 512-128-128-128-128 180 us with both issued by thread 0 and the chunks of G
+// after the first loaded where they are staged; 151 with elected lanes, 139 with
+// every chunk loaded one ahead, 131 with the copies in a warp of their own.
+// 131,072 atoms x 64-64-64: 47 -> 41 us.
 //
 // Operand layout (no swizzle, K-major): 8 x 8 BF16 core matrices of 128
 // contiguous bytes; along K the next core matrix is 128 B away (LBO), the
@@ -114,6 +123,15 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, uint32_t
                  "l"(src), "r"(bytes), "r"(bar)
                  : "memory");
 }
+// one lane of a converged warp, always the same: tells the compiler that one
+// thread runs what follows, whose operands then go to uniform registers at once
+// (after `if (tid == 0)` it loops over the threads that might be there: 200
+// cycles an MMA, 700 a copy)
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}" : "=r"(p));
+    return p != 0;
+}
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -200,15 +218,15 @@ constexpr int MAX_NST = 4;   // weight-chunk stages at most
 constexpr int MAX_CHUNKS = 64;   // weight chunks of one species block at most
 
 __global__ void __launch_bounds__(UTHREADS, 2)
-    k_mlp_umma(DevModel m, UmmaNet u, const int32_t *__restrict__ perm, const int32_t *__restrict__ types, int64_t n,
-               const float *__restrict__ G, float *__restrict__ dG, float *__restrict__ e_atom,
-               double *__restrict__ part_e, int ntile) {
+    k_mlp_umma(const __grid_constant__ DevModel m, const __grid_constant__ UmmaNet u, const int32_t *__restrict__ perm,
+               const int32_t *__restrict__ types, int64_t n, const float *__restrict__ G, float *__restrict__ dG,
+               float *__restrict__ e_atom, double *__restrict__ part_e, int ntile) {
     extern __shared__ __align__(1024) unsigned char smraw[];
     // barriers: full[MAX_NST], empty[MAX_NST] (weight stages), aempty[2] (G stages), done
     __shared__ __align__(8) uint64_t s_bar[2 * MAX_NST + 3];
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort;
-    __shared__ int s_atom[UM], s_type[UM], s_range[2];
+    __shared__ int s_type[UM], s_range[2];
     __shared__ float s_e[2][UM], s_ep[2][UM];   // s_e: E_a of the rows, by tile parity
     // per product pr: (K, N, N of a pass, npass | nkc << 8 | layer << 16) and
     // (bias offset, TMEM column of the act' written (forward) or read
@@ -216,7 +234,8 @@ __global__ void __launch_bounds__(UTHREADS, 2)
     // block: (element offset in ub[s], bytes)
     __shared__ int4 s_pa[2 * MAX_LAYERS], s_pb[2 * MAX_LAYERS];
     __shared__ int2 s_ck[MAX_CHUNKS];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // (uniform for the compiler)
     const int rq = warp & 3, ch = warp >> 2;   // TMEM lane quarter, column-block parity
     const int row = rq * 32 + lane;            // this thread's tile row
     const int L = m.L, Dd = m.Dd, NST = u.nst;
@@ -271,7 +290,7 @@ __global__ void __launch_bounds__(UTHREADS, 2)
         }
     }
     volatile int *abort = &s_abort;
-    uint32_t pending = 0;   // thread 0: stages with a copy not yet seen complete
+    uint32_t copies = 0;   // copies issued (CWARP)
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
                      "r"(u.tcols)
@@ -286,34 +305,38 @@ __global__ void __launch_bounds__(UTHREADS, 2)
     uint32_t q = 0;    // weight chunks consumed
     int qs = 0;        // its stage, q % NST
     uint32_t qph = 0;  // the parity of its use, (q / NST) & 1
-    uint32_t qi = 0;   // weight chunks whose copy was issued (thread 0)
+    uint32_t qi = 0;   // weight chunks whose copy was issued (CWARP)
     int qis = 0;       // its stage, qi % NST
     uint32_t qiu = 0;  // its use, qi / NST
     uint32_t ua = 0;   // G chunks consumed (stage ua & 1, use ua >> 1)
     uint32_t pd = 0;   // products (passes) completed
-    // thread 0: issue the copies of this block's chunks up to global index lim
+    // CWARP (beside the MMAs): issue the copies of this block's chunks up to global index lim
+    constexpr int CWARP = UTHREADS / 32 - 2;
     auto issue_upto = [&](uint32_t lim, uint32_t qbase, int s) {
         if (u.resident && qi >= (uint32_t)NST) {   // the stages already hold every chunk
             qi = max(qi, lim);
             return;
         }
-        while (qi < lim && !*abort) {
+        while (qi < lim) {
             const int st = qis;
-            if (qiu >= 1) mbar_wait(bar_empty(st), (qiu - 1) & 1, abort);   // the MMAs that read it are done
-            if (*abort) break;
+            bool ok = !*abort;
+            if (qiu >= 1) ok = mbar_wait(bar_empty(st), (qiu - 1) & 1, abort);   // the MMAs that read it are done
+            if (!__all_sync(0xffffffffu, ok)) break;
             const int2 ck = s_ck[qi - qbase];
-            mbar_expect_tx(bar_full(st), (uint32_t)ck.y);
-            bulk_g2s(smem_u32(B0 + st * bstride), m.ub[s] + ck.x, (uint32_t)ck.y, bar_full(st));
-            pending |= 1u << st;
+            if (elect_one()) {
+                mbar_expect_tx(bar_full(st), (uint32_t)ck.y);
+                bulk_g2s(smem_u32(B0 + st * bstride), m.ub[s] + ck.x, (uint32_t)ck.y, bar_full(st));
+            }
+            ++copies;
             ++qi;
             if (++qis == NST) { qis = 0; ++qiu; }
         }
     };
-    // Software pipeline over tiles: this thread's atom of the next tile, and
-    // its share of that tile's first G chunk, are loaded into registers while
-    // the current tile runs (a quarter warp per row: lane l covers row
-    // 4 it + l / 8 of its lane quarter, columns 32 ch + 4 (l % 8) .. + 3 of
-    // the chunk).
+    // Software pipeline: this thread's share of the G chunk that is staged next
+    // (the tile's next chunk, or the first one of the next species or tile) is
+    // loaded into registers while the MMAs of the one before run (a quarter warp
+    // per row: lane l covers row 4 it + l / 8 of its lane quarter, columns
+    // 32 ch + 4 (l % 8) .. + 3 of the chunk).
     auto row_atom = [&](int t) -> int {
         const int64_t p = (int64_t)t * UM + row;
         return (t < ntile && p < n) ? perm[p] : -1;
@@ -321,12 +344,12 @@ __global__ void __launch_bounds__(UTHREADS, 2)
     float4 gpre[8];
     uint32_t gok = 0;   // bit it: gpre[it] holds a row of an atom (else it reads as zeros)
     // G and G' rows are indexed by perm position: row r of tile t is t UM + r
-    auto load_g0 = [&](int atom_of_my_row, int t) {
+    auto load_g = [&](int atom_of_my_row, int t, int c) {
         gok = 0;
 #pragma unroll
         for (int it = 0; it < 8; ++it) {
             const int a = __shfl_sync(0xffffffffu, atom_of_my_row, 4 * it + (lane >> 3));
-            const int col = 32 * ch + 4 * (lane & 7);
+            const int col = c * UKC + 32 * ch + 4 * (lane & 7);
             // the null row of a missing atom reads as zeros
             const bool ok = a >= 0 && col < Dd;
             const size_t p = (size_t)t * UM + rq * 32 + 4 * it + (lane >> 3);
@@ -356,16 +379,14 @@ __global__ void __launch_bounds__(UTHREADS, 2)
     int kt = 0, prev_tile = -1;                // tiles done by this block, the last of them
     int nx_atom = row_atom(blockIdx.x);
     int nx_type = nx_atom >= 0 ? types[nx_atom] : -1;
-    load_g0(nx_atom, blockIdx.x);
+    load_g(nx_atom, blockIdx.x, 0);
     for (int tile = blockIdx.x; tile < ntile; tile += gridDim.x) {
         const int eb = kt & 1;
         if (ch == 0) {
-            s_atom[row] = nx_atom;
             s_type[row] = nx_type;
             s_e[eb][row] = 0.f;
         }
         const int my_atom = nx_atom, my_type = nx_type;
-        bool g0_ready = true;   // gpre holds this tile's first chunk
         // the tile after this one: atom ids now, species and G rows once gpre is consumed
         nx_atom = row_atom(tile + gridDim.x);
         __syncthreads();
@@ -384,7 +405,7 @@ __global__ void __launch_bounds__(UTHREADS, 2)
         const int s_lo = s_range[0], s_hi = s_range[1];
         for (int s = s_lo; s <= s_hi; ++s) {
             const uint32_t qbase = q, qend = q + (uint32_t)u.block_chunks;
-            if (tid == 0) issue_upto(min(qend, q + NST), qbase, s);
+            if (warp == CWARP) issue_upto(min(qend, q + NST), qbase, s);
             for (int pr = 0; pr < 2 * L; ++pr) {
                 const bool fwd = pr < L, last = pr == 2 * L - 1;
                 const int4 pa = s_pa[pr], pb = s_pb[pr];
@@ -398,19 +419,6 @@ __global__ void __launch_bounds__(UTHREADS, 2)
                         const uint32_t ause = ua >> (na - 1);
                         uint16_t *Ast = A0 + ast * CHUNK_EL;
                         if (pr == 0) {   // G chunk c -> BF16 operand (a quarter warp per row, own rows)
-                            if (!(c == 0 && g0_ready)) {
-                                const int r0 = rq * 32 + (lane >> 3);
-#pragma unroll
-                                for (int it = 0; it < 8; ++it) {
-                                    const int a = s_atom[r0 + 4 * it];
-                                    const int col = c * UKC + 32 * ch + 4 * (lane & 7);
-                                    gpre[it] = make_float4(0.f, 0.f, 0.f, 0.f);
-                                    if (a >= 0 && col < Dd)
-                                        gpre[it] = __ldg(reinterpret_cast<const float4 *>(
-                                            G + ((size_t)tile * UM + r0 + 4 * it) * Dd + col));
-                                }
-                                gok = 0xffu;
-                            }
                             if (ause >= 1) mbar_wait(bar_aempty(ast), (ause - 1) & 1, abort);
 #pragma unroll
                             for (int it = 0; it < 8; ++it) {
@@ -424,40 +432,48 @@ __global__ void __launch_bounds__(UTHREADS, 2)
                             fence_proxy_async();
                             __syncthreads();
                         }
-                        if (tid == 0 && !*abort) {
-                            if (!(u.resident && q >= (uint32_t)NST) && mbar_wait(bar_full(st), qph, abort))
-                                pending &= ~(1u << st);
+                        if (warp == 0 && __all_sync(0xffffffffu, !*abort)) {
+                            if (!(u.resident && q >= (uint32_t)NST)) mbar_wait(bar_full(st), qph, abort);
+                            __syncwarp();
                             tc_fence_after();
                             const int kl = min(UKC, K - c * UKC);
                             // the descriptors of the next K16 step are 256 bytes on (16 in the address field)
                             const uint64_t da = sdesc(smem_u32(pr == 0 ? Ast : Xin + (size_t)c * CHUNK_EL));
                             const uint64_t db = sdesc(smem_u32(B0 + st * bstride));
                             const uint32_t id = idesc_bf16(Np);
-                            for (int j = 0; j < kl / 16; ++j)
-                                umma_bf16(tmem, da + 16 * j, db + 16 * j, id, (c | j) != 0);
-                            // resident weights: no copy ever waits for a stage to drain
-                            if (!u.resident) umma_commit(bar_empty(st));
-                            if (pr == 0) umma_commit(bar_aempty(ast));
-                            // keep the stages filled: the copy for chunk q + NST - 1 reuses the
-                            // stage of chunk q - 1, whose MMAs were issued one chunk earlier
-                            issue_upto(min(qend, q + NST), qbase, s);
+                            if (elect_one()) {
+                                if (kl == UKC) {
+#pragma unroll
+                                    for (int j = 0; j < UKC / 16; ++j)
+                                        umma_bf16(tmem, da + 16 * j, db + 16 * j, id, (c | j) != 0);
+                                } else {
+                                    for (int j = 0; j < kl / 16; ++j)
+                                        umma_bf16(tmem, da + 16 * j, db + 16 * j, id, (c | j) != 0);
+                                }
+                                // resident weights: no copy ever waits for a stage to drain
+                                if (!u.resident) umma_commit(bar_empty(st));
+                                if (pr == 0) umma_commit(bar_aempty(ast));
+                            }
+                            __syncwarp();
                         }
-                        // the rest of warp 0 waits here rather than polling an
-                        // mbarrier beside the issuing lane
-                        if (warp == 0) __syncwarp();
+                        // keep the stages filled: the copy for chunk q + NST - 1 reuses the
+                        // stage of chunk q - 1, whose MMAs were issued one chunk earlier
+                        if (warp == CWARP) issue_upto(min(qend, q + NST), qbase, s);
                         if (pr == 0) {
-                            // gpre is free: (re)start on the next tile's first chunk
-                            // (after the MMA issue, which then waits on none of these loads)
-                            if (g0_ready) nx_type = nx_atom >= 0 ? types[nx_atom] : -1;
-                            g0_ready = false;
-                            load_g0(nx_atom, tile + gridDim.x);
+                            // gpre is free: on to the next chunk (after the MMA
+                            // issue, which then waits on none of these loads)
+                            const bool tile_end = c == nkc - 1 && s == s_hi;
+                            if (tile_end) nx_type = nx_atom >= 0 ? types[nx_atom] : -1;
+                            load_g(tile_end ? nx_atom : my_atom, tile + (tile_end ? gridDim.x : 0), c < nkc - 1 ? c + 1 : 0);
                             ++ua;
                         }
                         ++q;
                         if (++qs == NST) { qs = 0; qph ^= 1u; }
                     }
-                    if (tid == 0) umma_commit(bar_done);
-                    if (warp == 0) __syncwarp();
+                    if (warp == 0) {
+                        if (elect_one()) umma_commit(bar_done);
+                        __syncwarp();
+                    }
                     if (pr == 0 && P == 0 && s == s_lo && warp == EWARP && prev_tile >= 0)
                         tile_energy(s_e[eb ^ 1], prev_tile);
                     mbar_wait(bar_done, pd & 1, abort);
@@ -558,11 +574,15 @@ __global__ void __launch_bounds__(UTHREADS, 2)
     }
     __syncthreads();
     if (warp == EWARP && prev_tile >= 0) tile_energy(s_e[(kt - 1) & 1], prev_tile);
-    if (tid == 0 && *abort) {   // bounded drain of this block's copies and MMAs in flight
-        for (uint32_t k = (qi > (uint32_t)NST ? qi - NST : 0); k < qi; ++k)
-            if (pending & (1u << (k % NST))) mbar_drain(bar_full(k % NST), (k / NST) & 1);
-        umma_commit(bar_done);
-        mbar_drain(bar_done, pd & 1);
+    if (*abort) {   // bounded drain of this block's copies and MMAs in flight
+        if (warp == CWARP)
+            for (uint32_t k = copies > (uint32_t)NST ? copies - NST : 0; k < copies; ++k)
+                mbar_drain(bar_full(k % NST), (k / NST) & 1);
+        if (warp == 0) {
+            if (elect_one()) umma_commit(bar_done);
+            __syncwarp();
+            mbar_drain(bar_done, pd & 1);
+        }
     }
     tc_fence_before();
     __syncthreads();
