@@ -230,8 +230,9 @@ int64_t tmd_graph_replays(void);
  *                      pipes: 32 or 64; 128 (networks whose descriptor length
  *                      and hidden widths are all 64, one or two hidden layers)
  *                      and 0 = built-in choice.  Networks that run on the
- *                      tensor cores (hidden widths multiples of 16 up to 128,
- *                      activations of a tile within an SM's shared memory)
+ *                      tensor cores (descriptor length up to 192, hidden
+ *                      widths multiples of 16 up to 128, activations of a tile
+ *                      within an SM's shared memory)
  *                      have 128-atom tiles with each of them;
  *  pair_blocks_per_sm  blocks per SM of the persistent descriptor / force
  *                      grids (0 = built-in 16);

@@ -45,22 +45,11 @@ constexpr float PI_F = 3.14159265358979323846f;
 // weights w_c of the squared sums A_c, in the order of harmonics16
 __constant__ float c_W[NHAR] = {1.f, 1.f, 1.f, 1.f, 2.f, 2.f, 2.f, 0.5f, 1.5f, 0.1f, 0.15f, 0.15f, 1.5f, 6.f, 0.25f, 0.25f};
 
-// 1 | x y z | xy yz xz x^2-y^2 | z^2-1/3, z(5z^2-3) x(5z^2-1) y(5z^2-1) | z(x^2-y^2) xyz x(x^2-3y^2) y(3x^2-y^2)
-// of a unit vector (degrees 0; 1; 2; 3)
-__device__ __forceinline__ void harmonics16(float x, float y, float z, float *Y) {
-    const float xx = x * x, yy = y * y, zz = z * z, d = xx - yy, q = fmaf(5.f, zz, -1.f);
-    Y[0] = 1.f;
-    Y[1] = x; Y[2] = y; Y[3] = z;
-    Y[4] = x * y; Y[5] = y * z; Y[6] = x * z; Y[7] = d;
-    Y[8] = zz - (1.f / 3.f);
-    Y[9] = z * fmaf(5.f, zz, -3.f); Y[10] = x * q; Y[11] = y * q;
-    Y[12] = z * d; Y[13] = Y[4] * z; Y[14] = x * fmaf(-3.f, yy, xx); Y[15] = y * fmaf(3.f, xx, -yy);
-}
-
 __device__ __forceinline__ float2 bc2(float x) { return make_float2(x, x); }
 
-// harmonics16 of two vectors (packed FP32x2)
-__device__ __forceinline__ void harmonics16x2(float2 x, float2 y, float2 z, float2 *Y) {
+// 1 | x y z | xy yz xz x^2-y^2 | z^2-1/3, z(5z^2-3) x(5z^2-1) y(5z^2-1) | z(x^2-y^2) xyz x(x^2-3y^2) y(3x^2-y^2)
+// of two unit vectors (degrees 0; 1; 2; 3; packed FP32x2)
+__device__ __forceinline__ void harmonics16(float2 x, float2 y, float2 z, float2 *Y) {
     const float2 xx = __fmul2_rn(x, x), yy = __fmul2_rn(y, y), zz = __fmul2_rn(z, z);
     const float2 d = __ffma2_rn(yy, bc2(-1.f), xx), q = __ffma2_rn(zz, bc2(5.f), bc2(-1.f));
     Y[0] = bc2(1.f);
@@ -177,20 +166,6 @@ __device__ __forceinline__ void tab_eval(const TabCell &tc, int k, float scale, 
     const float4 q = __ldg(tc.c + k);
     H = fmaf(tc.t, fmaf(tc.t, fmaf(tc.t, q.w, q.z), q.y), q.x);
     dH = scale * fmaf(tc.t, fmaf(tc.t3, q.w, 2.f * q.z), q.y);
-}
-
-// channels k0 .. k0 + KC - 1 of a table of K channels
-template <int KC, bool DERIV>
-__device__ __forceinline__ void radial_tab(const float *tab, int K, int k0, float scale, float r_hi, float r_lo,
-                                           float *H, float *dH) {
-    const TabCell tc = tab_cell(tab, K, scale, r_hi, r_lo);
-#pragma unroll
-    for (int k = 0; k < KC; ++k) {
-        float h, d;
-        tab_eval(tc, k0 + k, scale, h, d);
-        H[k] = h;
-        if (DERIV) dH[k] = d;
-    }
 }
 
 // r = |D| as an unevaluated sum r_hi + r_lo from r^2 = r2_hi + r2_lo, and 1/r.
@@ -612,7 +587,7 @@ __global__ void __launch_bounds__(PW * 32, desc_min_blocks(S * K)) k_desc(DevMod
                 put(2, make_float2(v0 ? fc.x : 0.f, v1 ? fc.y : 0.f));
             }
             float2 Y[NHAR];
-            harmonics16x2(__fmul2_rn(make_float2(w.e0.x, w.e1.x), ir), __fmul2_rn(make_float2(w.e0.y, w.e1.y), ir),
+            harmonics16(__fmul2_rn(make_float2(w.e0.x, w.e1.x), ir), __fmul2_rn(make_float2(w.e0.y, w.e1.y), ir),
                           __fmul2_rn(make_float2(w.e0.z, w.e1.z), ir), Y);
 #pragma unroll
             for (int c = 1; c < NHAR; ++c) put(3 + 8 * ((c >> 1) & 1) + 2 * (c >> 2) + (c & 1), Y[c]);

@@ -960,8 +960,9 @@ static tmd_status launch_network(const DevModel &dm, const int32_t *perm, const 
         set_error("the tcgen05 network kernel does not support these network shapes");
         return TMD_ERR_UNIMPLEMENTED;
     }
-    // FP32: the tensor cores wherever the widths are multiples of 16 up to 128
-    // and a tile fits on chip; k_mlp has the rest.  At every size: one 32-atom
+    // FP32: the tensor cores wherever the widths are multiples of 16 up to 128,
+    // the descriptor has at most 192 columns (for its accuracy, TF_DD) and a tile
+    // fits on chip; k_mlp has the rest.  At every size: one 32-atom
     // tile 15.5 us against 15.6 in k_mlp, 1,048,576 atoms x 64-64 423 us
     // against 850, 147,456 atoms x 128-128-128 254 us against 922 (k_mlp).
     // Two labels, as tile_rows has two kinds of tile: "k_mlp_res" where 0 or
