@@ -36,16 +36,16 @@ UNIT = "atom-steps/s"
 CONV = 1.0 / 103.6427
 
 # algorithmic flops per in-cutoff pair (FMA = 2 flops), from the operation
-# counts of the tensor chain: forward P = sum H M (K x 20 FMA) + radial basis
-# (~8 per channel) + geometry/moments (~50); backward U and V (2 x K x 20 FMA),
+# counts of the tensor chain: forward P = sum H M (K x 16 FMA) + radial basis
+# (~8 per channel) + geometry/moments (~50); backward U and V (2 x K x 16 FMA),
 # H' (K FMA), radial basis with derivative (~10 per channel), M' contraction
 # and projection (~120), virial (~45).
 def fwd_flops_per_pair(K):
-    return 2 * 20 * K + 8 * K + 50
+    return 2 * 16 * K + 8 * K + 50
 
 
 def bwd_flops_per_pair(K):
-    return 2 * (2 * 20 * K + K) + 10 * K + 165
+    return 2 * (2 * 16 * K + K) + 10 * K + 165
 
 
 def mlp_flops_per_atom(dims):
