@@ -1268,7 +1268,7 @@ tmd_status noalloc_capacity(const tmd_model *model, int64_t n, size_t *need) {
     b += al(sizeof(float) * n * dm.S * dm.K * NMOM);           // P (with room for NMOM components: the documented limit)
     b += 2 * al(sizeof(float) * n * dm.Dd);                    // G, G'
     b += al(sizeof(unsigned long long) * 3 * n);               // force accumulator
-    b += al(sizeof(double) * (ntile + 9 * nblk + 16));         // block partials
+    b += al(sizeof(double) * (ntile + 9 * nblk + 16 + 640));   // block partials (640: as the limit was documented)
     b += al(sizeof(int32_t) * 4);                              // check flag
     *need = b;
     return b <= NOALLOC_BYTES ? TMD_OK : TMD_ERR_CAPACITY;
