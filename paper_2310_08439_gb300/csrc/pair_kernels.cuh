@@ -459,6 +459,10 @@ __device__ __forceinline__ Split2 split2(const float2 x) {
 // lost from the magnitude of each such sum (twice half a unit in its last place
 // on average): without it G is 1.8e-7 too small on average, with it 1e-8 (rms
 // error of G 2.0e-7 and 1.4e-7; the FP32 sums before: 1.3e-7 and 1.6e-7).
+// Part of that is not the sums' but the Gaussians' (ex2.approx); H from a table
+// has no such part, and the sums run without the factor: over 24 random cases the
+// virial's error is 4.4e-6 of its norm (with the factor 6.1e-6, FP32 sums 3.6e-6
+// to 4.5e-6: near zero pressure it amplifies what all atoms have in common).
 //
 // A lane stages two pairs (2 l, 2 l + 1 of a batch of 64) on packed FP32x2
 // arithmetic, so that most atoms need one batch.
@@ -490,7 +494,7 @@ __global__ void __launch_bounds__(PW * 32, desc_min_blocks(S * K)) k_desc(DevMod
     constexpr int RS = S <= 2 ? 72 : 104;
     constexpr int Dd = S * K * 4;
     constexpr bool HOIST = MT <= 2;       // channel parameters in registers (per species group)
-    const float2 untrunc = bc2(1.00000012f);   // 1 + 2^-23
+    const float2 untrunc = bc2(TAB ? 1.f : 1.00000012f);   // 1 + 2^-23
     constexpr bool RSH = S * S * K <= 512;   // the channel parameters fit beside the staging
     __shared__ float4 s_rad[RSH ? S * S * K : 1];   // (-mu_hi, -mu_lo, -eta log2 e, 0)
     __shared__ float4 s_q[CACHED ? 1 : PW][CACHED ? 1 : 96];
