@@ -519,7 +519,10 @@ __global__ void __launch_bounds__(PW * 32, desc_min_blocks(S * K)) k_desc(DevMod
     const unsigned lt = (1u << lane) - 1u;
     float *const st = s_st[warp];
     // unused slots hold f_c = 0 and finite values; component 0 is 1
-    for (int i = lane; i < (3 + NHAR) * RS; i += 32) st[i] = (i / RS == 3) ? 1.f : 0.f;
+    auto clear_staging = [&]() {
+        for (int i = lane; i < (3 + NHAR) * RS; i += 32) st[i] = (i / RS == 3) ? 1.f : 0.f;
+    };
+    clear_staging();
     __syncthreads();
     float Wt[4];
 #pragma unroll
@@ -577,6 +580,11 @@ __global__ void __launch_bounds__(PW * 32, desc_min_blocks(S * K)) k_desc(DevMod
             };
             float2 r_hi, r_lo, ir;
             split_sqrt2(make_float2(w.q0.x, w.q1.x), make_float2(w.q0.y, w.q1.y), r_hi, r_lo, ir);
+            // Two atoms at one place have no direction and r is not a number.
+            // What such a pair stages must not be there when its slots pad a
+            // group of a later atom (0 x NaN is NaN): the staging is cleared
+            // after this batch.  (One species: every slot is written each time.)
+            const bool broken = S > 1 && __any_sync(0xffffffffu, !(r_hi.x + r_hi.y < INFINITY));
             if constexpr (TAB) {
                 const float2 x = __fmul2_rn(r_hi, bc2(m.rtab_scale)), gf = make_float2(floorf(x.x), floorf(x.y));
                 put(0, __ffma2_rn(r_lo, bc2(m.rtab_scale), __ffma2_rn(gf, bc2(-1.f), x)));
@@ -669,6 +677,10 @@ __global__ void __launch_bounds__(PW * 32, desc_min_blocks(S * K)) k_desc(DevMod
                 start += (cnt[s] + 7) & ~7;
             }
             __syncwarp();
+            if (broken) {
+                clear_staging();
+                __syncwarp();
+            }
         };
         if constexpr (CACHED) {
             for (int base = 0; base < ps.np; base += 64) {
