@@ -151,10 +151,16 @@ struct TabCell {
     float t, t3;       // t and 3 t
 };
 
-__device__ __forceinline__ TabCell tab_cell(const float *tab, int K, float scale, float r_hi, float r_lo) {
+// interval number from its floating value (exact for 0 <= gf < 2^22); inside
+// the table also where r is not a number (two atoms at one place)
+__device__ __forceinline__ int tab_interval(float gf, int n) {
+    return (int)min((unsigned)(__float_as_int(gf + 12582912.0f) - 0x4B400000), (unsigned)(n - 1));
+}
+
+__device__ __forceinline__ TabCell tab_cell(const float *tab, int K, int n, float scale, float r_hi, float r_lo) {
     const float x = r_hi * scale;
     const float gf = floorf(x);
-    const int g = __float_as_int(gf + 12582912.0f) - 0x4B400000;   // exact: 0 <= gf < 2^22
+    const int g = tab_interval(gf, n);
     TabCell c;
     c.c = reinterpret_cast<const float4 *>(tab) + (size_t)g * K;
     c.t = (x - gf) + r_lo * scale;
@@ -589,8 +595,8 @@ __global__ void __launch_bounds__(PW * 32, desc_min_blocks(S * K)) k_desc(DevMod
                 const float2 x = __fmul2_rn(r_hi, bc2(m.rtab_scale)), gf = make_float2(floorf(x.x), floorf(x.y));
                 put(0, __ffma2_rn(r_lo, bc2(m.rtab_scale), __ffma2_rn(gf, bc2(-1.f), x)));
                 // as tab_cell; a place without a pair reads interval 0
-                put(1, make_float2(__int_as_float(v0 ? __float_as_int(gf.x + 12582912.0f) - 0x4B400000 : 0),
-                                   __int_as_float(v1 ? __float_as_int(gf.y + 12582912.0f) - 0x4B400000 : 0)));
+                put(1, make_float2(__int_as_float(v0 ? tab_interval(gf.x, m.rtab_n) : 0),
+                                   __int_as_float(v1 ? tab_interval(gf.y, m.rtab_n) : 0)));
                 put(2, make_float2(v0 ? 1.f : 0.f, v1 ? 1.f : 0.f));
             } else {
                 const float2 fc = cutoff2(r_hi, m.inv_rc);
@@ -812,7 +818,7 @@ __device__ __forceinline__ void pair_grad(const DevModel &m, const float4 e, con
     float fc = 0.f, dfc = 0.f;
     TabCell tc;
     if (TAB)
-        tc = tab_cell(tab, K, m.rtab_scale, r_hi, r_lo);
+        tc = tab_cell(tab, K, m.rtab_n, m.rtab_scale, r_hi, r_lo);
     else
         cutoff_fn(r_hi, m.inv_rc, fc, dfc);
     const float2 rh2 = make_float2(r_hi, r_hi), rl2 = make_float2(r_lo, r_lo);
@@ -867,7 +873,7 @@ __device__ __forceinline__ void pair_sums2(const DevModel &m, const float (&rh)[
 #pragma unroll
         for (int d = 0; d < NHAR / 2; ++d) V[i][d] = W[i][d] = make_float2(0.f, 0.f);
         if (TAB) {
-            tc[i] = tab_cell(tab, K, m.rtab_scale, rh[i], rl[i]);
+            tc[i] = tab_cell(tab, K, m.rtab_n, m.rtab_scale, rh[i], rl[i]);
         } else {
             float c, d;
             cutoff_fn(rh[i], m.inv_rc, c, d);

@@ -31,9 +31,12 @@ def _systems(n_species, broken):
     return out
 
 
-@pytest.mark.parametrize("n_species,K", [(2, 16), (3, 8), (5, 16)])
-def test_other_systems_of_a_batch_stay_as_they_are(tmdlib, n_species, K):
+@pytest.mark.parametrize("n_species,K,table", [(2, 16, 0), (3, 8, 0), (5, 16, 0), (1, 16, 64), (2, 16, 64), (3, 8, 256)])
+def test_other_systems_of_a_batch_stay_as_they_are(tmdlib, n_species, K, table):
+    """With a table the coincident pair's interval stays inside it."""
     m = tmdlib.Model(I.random_model(n_species, K, RC, [32, 32], seed=K + n_species))
+    if table:
+        m.set_radial_table(table)
     res = []
     for broken in (False, True):
         systems = _systems(n_species, broken)
