@@ -16,6 +16,8 @@
 //   G_0 = |A_0|                     G_1 = sum_{1..3} A_c^2
 //   G_2 = A_0^2 / 3 + sum_{4..8} w_c A_c^2
 //   G_3 = 3/5 G_1 + sum_{9..15} w_c A_c^2
+// (1/3, 3/5 and, in dE/dA, 2/3 as hi + lo: an error of such a constant is the
+// same in every atom and adds up in the virial.)
 // The sums are the same numbers with 16 instead of 20 multiply-adds per
 // channel, pair and pass, and every term is a square with a positive weight.
 //
@@ -44,6 +46,9 @@ constexpr float PI_F = 3.14159265358979323846f;
 
 // weights w_c of the squared sums A_c, in the order of harmonics16
 __constant__ float c_W[NHAR] = {1.f, 1.f, 1.f, 1.f, 2.f, 2.f, 2.f, 0.5f, 1.5f, 0.1f, 0.15f, 0.15f, 1.5f, 6.f, 0.25f, 0.25f};
+
+// a x + b for a constant a of which FP32 holds a_hi and a_lo is the rest
+#define FMA_HILO(a, x, b) fmaf((float)(a), x, fmaf((float)((a) - (double)(float)(a)), x, b))
 
 __device__ __forceinline__ float2 bc2(float x) { return make_float2(x, x); }
 
@@ -401,7 +406,7 @@ __device__ __forceinline__ float desc_value(const float (&A)[4], const float (&W
     const float a00 = __shfl_sync(0xffffffffu, s0, quad);     // A_0^2
     const float one = __shfl_sync(0xffffffffu, s13, quad);    // G_1
     const float up = __shfl_up_sync(0xffffffffu, g == 1 ? s0 + s13 : s13, 1);
-    const float val2 = fmaf(1.f / 3.f, a00, up + s0), val3 = fmaf(0.6f, one, up + (s0 + s13));
+    const float val2 = FMA_HILO(1.0 / 3.0, a00, up + s0), val3 = FMA_HILO(0.6, one, up + (s0 + s13));
     return g == 0 ? fabsf(A[0]) : (g == 1 ? one : (g == 2 ? val2 : val3));
 }
 
@@ -939,9 +944,9 @@ __device__ __forceinline__ void pair_sums2(const DevModel &m, const float (&rh)[
 // the place of G'_1 (c = 1..3).
 __device__ __forceinline__ float4 aprime(const float4 A, const float4 gm, const float (&Wg)[4], int g) {
     const float h0 = g == 1 || g == 2 ? gm.z : gm.w;                      // c = 4g
-    const float h = g == 0 ? fmaf(0.6f, gm.w, gm.y) : (g == 1 ? gm.z : gm.w);
+    const float h = g == 0 ? FMA_HILO(0.6, gm.w, gm.y) : (g == 1 ? gm.z : gm.w);
     float4 o = make_float4(2.f * Wg[0] * A.x * h0, 2.f * Wg[1] * A.y * h, 2.f * Wg[2] * A.z * h, 2.f * Wg[3] * A.w * h);
-    if (g == 0) o.x = fmaf(2.f / 3.f * gm.z, A.x, (A.x > 0.f) ? gm.x : ((A.x < 0.f) ? -gm.x : 0.f));
+    if (g == 0) o.x = fmaf(FMA_HILO(2.0 / 3.0, gm.z, 0.f), A.x, (A.x > 0.f) ? gm.x : ((A.x < 0.f) ? -gm.x : 0.f));
     return o;
 }
 

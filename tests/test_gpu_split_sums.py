@@ -35,21 +35,37 @@ def _descriptors(tmd, m, s):
     return G.double().cpu().numpy(), dG.double().cpu().numpy()
 
 
-@pytest.mark.parametrize("S,K,lattice", [(1, 16, "fcc"), (1, 32, "bcc"), (2, 16, "fcc"), (3, 8, "bcc")])
-def test_descriptor_sums_have_no_common_error(tmdlib, S, K, lattice, capsys):
+CASES = [(1, 16, "fcc"), (1, 32, "bcc"), (2, 16, "fcc"), (3, 8, "bcc")]
+
+
+def _mean_errors(tmd, S, K, lattice):
     s = _system(S, 10 * S + K, *(((6, 6, 6), 3.7) if lattice == "fcc" else ((8, 8, 8), 2.95)), lattice)
     p = I.random_model(S, K, RC, [16], seed=1)
-    m = tmdlib.Model(p)
+    m = tmd.Model(p)
     m.set_radial_table(256)
     o = O.evaluate(O.OracleModel(p, radial_table=256), s.pos, s.types, s.box, s.pbc, want_G=True)["G"]
-    G = _descriptors(tmdlib, m, s)[0]
+    G = _descriptors(tmd, m, s)[0]
     G, o = G.reshape(len(G), S * K, 4), o.reshape(len(G), S * K, 4)
     rms = np.sqrt((o ** 2).mean(axis=0))
     mean = []
     for rank in range(4):
         big = o[:, :, rank] > 0.1 * rms[None, :, rank].max()
         mean.append(float(((G[:, :, rank] - o[:, :, rank])[big] / o[:, :, rank][big]).mean()))
+    return np.array(mean)
+
+
+@pytest.mark.parametrize("S,K,lattice", CASES)
+def test_descriptor_sums_have_no_common_error(tmdlib, S, K, lattice, capsys):
+    mean = _mean_errors(tmdlib, S, K, lattice)
     with capsys.disabled():
         print(f"\n[S={S} K={K} {lattice}] mean relative error of G_0 .. G_3: " + " ".join(f"{x:.2e}" for x in mean))
     assert abs(mean[0]) <= 2.0 ** -25
-    assert max(abs(x) for x in mean[1:]) <= 2.0 ** -24
+    assert np.abs(mean[1:]).max() <= 2.0 ** -24
+
+
+def test_constants_of_the_ranks(tmdlib):
+    """1/3 and 3/5, with which the lower degrees enter G_2 and G_3, are off by
+    3e-8 and 4e-8 as FP32 numbers.  Over the four cases the mean error stays
+    below a quarter of a unit in the last place, half of either."""
+    mean = np.mean([_mean_errors(tmdlib, *c) for c in CASES], axis=0)
+    assert np.abs(mean[2:]).max() <= 2.0 ** -26
