@@ -437,9 +437,10 @@ __device__ __forceinline__ void mma_tf32_first(float (&c)[4], const uint32_t (&a
 
 // Two values as operands of a split product: x_h = x rounded to TF32 (11
 // significant bits, ties away) and x_l = x - x_h (exact, 12 bits or fewer), of
-// which the tensor cores read the TF32 part, dropping at most the last bit of
-// x.  Integer operations: the conversion cvt.rna.tf32 issues at the rate of
-// the special functions and made it the bound of the descriptor pass.
+// which the tensor cores read the TF32 part: half a unit of that is added, so
+// that the last bit of x is rounded where it does not fit, not dropped.  Integer
+// operations: the conversion cvt.rna.tf32 issues at the rate of the special
+// functions and made it the bound of the descriptor pass.
 struct Split2 {
     uint32_t h0, h1, l0, l1;
 };
@@ -449,8 +450,8 @@ __device__ __forceinline__ Split2 split2(const float2 x) {
     o.h0 = (__float_as_uint(x.x) + 0x1000u) & 0xffffe000u;
     o.h1 = (__float_as_uint(x.y) + 0x1000u) & 0xffffe000u;
     const float2 r = __ffma2_rn(make_float2(__uint_as_float(o.h0), __uint_as_float(o.h1)), make_float2(-1.f, -1.f), x);
-    o.l0 = __float_as_uint(r.x);
-    o.l1 = __float_as_uint(r.y);
+    o.l0 = __float_as_uint(r.x) + 0x1000u;
+    o.l1 = __float_as_uint(r.y) + 0x1000u;
     return o;
 }
 
@@ -462,40 +463,48 @@ __device__ __forceinline__ Split2 split2(const float2 x) {
 // the lane that holds the pair, and staged in shared memory, one row per
 // quantity and one column per pair.
 //
-// FP32 accuracy from split operands: x = x_h + x_l + O(2^-23 x), both parts
-// TF32, and x y = x_l y_h + x_h y_l + x_h y_h (the products are exact in FP32).
-// The tensor cores cut the sum to 24 bits where an FP32 add would round it: the
-// sums of 8 pairs therefore start from zero, small terms first, and are added to
-// the totals in FP32.  What the cut takes from each of them is known on average,
-// half a unit in the last place of a number whose leading digits are as those of
-// numbers are: 2^-24 (1/2) / ln 2 of it, and is put back once, at the end
+// FP32 accuracy from split operands: x = x_h + x_l + O(2^-24 x), both parts
+// TF32, and x y = x_l y_l + x_l y_h + x_h y_l + x_h y_h (the products are exact in
+// FP32).  The tensor cores cut the sum to 24 bits where an FP32 add would round
+// it: the sums of 8 pairs therefore start from zero, small terms first, and are
+// added to the totals in FP32.  What the cut takes from each of them is known on
+// average, half a unit in the last place of a number whose leading digits are as
+// those of numbers are: 2^-24 (1/2) / ln 2 of it, and is put back once, at the end
 // (UNCUT).  Component 0, the sum of H over the pairs, to which all terms add with
 // one sign, is not left to them: every lane adds the H that it forms, in FP32.
-// Error of G against FP64 over 38 models and lattices of 8 to 128 channels: 0.88
-// to 0.96 times that of FP32 multiply-adds in sequence (rms, of the norm).
+// Errors against FP64 over 543 evaluations of the workloads and of random models,
+// lattices and sizes, as multiples of those with FP32 multiply-adds in sequence
+// and k_mlp (rms, K up to 64): G 0.95 to 0.99, forces 0.85 to 1.00.  Without x_l y_l
+// and the rounding of x_l the forces of a 32-atom fcc and an 8,160-atom bcc cell are
+// 1.04 and 1.05 (now 0.99 and 1.00).
+// K = 128 (FINE false): three products and no separate sum, whose registers and
+// additions would cost 0.07 of 0.32 ms (39,366 atoms): G 1.03, forces 0.94.
 //
 // A lane stages two pairs (2 l, 2 l + 1 of a batch of 64) on packed FP32x2
 // arithmetic, so that most atoms need one batch.
 //
-// What bounds it: instruction issue (61 % of the slots; 760 warp instructions
-// per atom at 53 pairs and K = 16; FMA pipe 41 %, ALU 35 %, tensor 27 %).  The
-// pass before it (packed FP32 multiply-adds on a (K/8 x 4) block per lane)
-// staged H as well, read 6 shared float4 per 16 multiply-add instructions and
-// waited on shared memory.  1,048,576 atoms, K = 16: 1.60 -> 1.02 ms; 148,176
-// atoms, K = 32: 0.356 -> 0.285; 39,366 atoms, K = 128: 0.487 -> 0.338 ms.
+// What bounds it: instruction issue (with three products and the sum of H on the
+// tensor cores 61 % of the slots, 760 warp instructions per atom at 53 pairs and K
+// = 16, FMA pipe 41 %, ALU 35 %, tensor 27 %).  The pass before it (packed FP32
+// multiply-adds on a (K/8 x 4) block per lane) staged H as well, read 6 shared
+// float4 per 16 multiply-add instructions and waited on shared memory.  1,048,576
+// atoms, K = 16: 1.60 -> 1.20 ms; 148,176 atoms, K = 32: 0.356 -> 0.330; 39,366
+// atoms, K = 128: 0.487 -> 0.322 ms.  (Three products, no separate sum of H: 1.03,
+// 0.286, 0.338 ms, with the errors above.)
 //
 // CACHED: the atom's in-cutoff pairs come from the pair cache filled by
-// k_screen; otherwise the pass screens the table itself (for_pairs).
-// Blocks per SM asked for (registers): measured 7 of 5 .. 10 at K = 16, S = 1
-// (1.02 ms for 1M atoms; 5 blocks 1.20, 9 blocks 1.17), 5 at K = 32 (0.285 ms
-// for 148,176 atoms; without a bound 0.290, 6 blocks 0.308) and at K = 16, S = 3
-// (0.369 against 0.399 and 0.480); the totals of larger S K leave no choice.
-constexpr int desc_min_blocks(int sk) { return sk <= 16 ? 7 : (sk <= 48 ? 5 : 1); }
+// k_screen; otherwise the pass screens the table itself (queue_pairs).
+// Blocks per SM asked for (registers): measured 7 of 5 .. 8 at K = 16, S = 1
+// (1.20 ms for 1M atoms, 6 and 8 the same, 5 1.21; for few atoms 7 is ahead: 37,044
+// atoms 106 us, 6 blocks 115), 4 at K = 32, S = 1 (0.330 ms for 148,176 atoms; 5
+// spill, 0.357, 3 0.383) and 5 at K = 16, S = 2 and 3 (S = 3: 0.432 ms for the batch
+// of 128 systems, 4 blocks 0.445); the totals of larger S K leave no choice.
+constexpr int desc_min_blocks(int s, int k) { return s * k <= 16 ? 7 : (s == 1 && k == 32 ? 4 : (s * k <= 48 ? 5 : 1)); }
 
 constexpr float UNCUT = 4.3e-8f;
 
 template <int K, int S, bool TAB, bool CACHED>
-__global__ void __launch_bounds__(PW * 32, desc_min_blocks(S * K)) k_desc(DevModel m, DevNlist nl, const double *__restrict__ pos,
+__global__ void __launch_bounds__(PW * 32, desc_min_blocks(S, K)) k_desc(DevModel m, DevNlist nl, const double *__restrict__ pos,
                                                   const int32_t *__restrict__ types, float *__restrict__ G,
                                                   float *__restrict__ Pout) {
     constexpr int MT = (K + 15) / 16;     // tiles of 16 channels
@@ -505,6 +514,7 @@ __global__ void __launch_bounds__(PW * 32, desc_min_blocks(S * K)) k_desc(DevMod
     // conflict-free
     constexpr int RS = S <= 2 ? 72 : 104;
     constexpr int Dd = S * K * 4;
+    constexpr bool FINE = K <= 64;        // the product x_l y_l and a separate sum of H
     constexpr bool HOIST = MT <= 2;       // channel parameters in registers (per species group)
     constexpr bool RSH = S * S * K <= 512;   // the channel parameters fit beside the staging
     __shared__ float4 s_rad[RSH ? S * S * K : 1];   // (-mu_hi, -mu_lo, -eta log2 e, 0)
@@ -677,7 +687,7 @@ __global__ void __launch_bounds__(PW * 32, desc_min_blocks(S * K)) k_desc(DevMod
                                 const float2 ex = __fmul2_rn(__fmul2_rn(qe, d), d);
                                 H = __fmul2_rn(make_float2(ex2_ftz(ex.x), ex2_ftz(ex.y)), fc);
                             }
-                            sum0[s][mt][h] += H.x + H.y;
+                            if constexpr (FINE) sum0[s][mt][h] += H.x + H.y;
                             x[h] = split2(H);
                         }
 #pragma unroll
@@ -685,7 +695,12 @@ __global__ void __launch_bounds__(PW * 32, desc_min_blocks(S * K)) k_desc(DevMod
                             float c[4];
                             const uint32_t xl[4] = {x[0].l0, x[1].l0, x[0].l1, x[1].l1};
                             const uint32_t xh[4] = {x[0].h0, x[1].h0, x[0].h1, x[1].h1};
-                            mma_tf32_first(c, xl, y[i].h0, y[i].h1);
+                            if constexpr (FINE) {
+                                mma_tf32_first(c, xl, y[i].l0, y[i].l1);
+                                mma_tf32(c, xl, y[i].h0, y[i].h1);
+                            } else {
+                                mma_tf32_first(c, xl, y[i].h0, y[i].h1);
+                            }
                             mma_tf32(c, xh, y[i].l0, y[i].l1);
                             mma_tf32(c, xh, y[i].h0, y[i].h1);
                             acc[s][mt][i] = __fadd2_rn(make_float2(c[0], c[1]), acc[s][mt][i]);
@@ -728,10 +743,12 @@ __global__ void __launch_bounds__(PW * 32, desc_min_blocks(S * K)) k_desc(DevMod
                                   acc[s][mt][2 * h + 1].y};
 #pragma unroll
                     for (int i = 0; i < 4; ++i) A[i] = fmaf(A[i], UNCUT, A[i]);
-                    float a0 = sum0[s][mt][h];
-                    a0 += __shfl_xor_sync(0xffffffffu, a0, 1);
-                    a0 += __shfl_xor_sync(0xffffffffu, a0, 2);
-                    if (t == 0) A[0] = a0;
+                    if constexpr (FINE) {
+                        float a0 = sum0[s][mt][h];
+                        a0 += __shfl_xor_sync(0xffffffffu, a0, 1);
+                        a0 += __shfl_xor_sync(0xffffffffu, a0, 2);
+                        if (t == 0) A[0] = a0;
+                    }
                     *reinterpret_cast<float4 *>(Pa + row * NHAR + 4 * t) = make_float4(A[0], A[1], A[2], A[3]);
                     Ga[row * 4 + t] = desc_value(A, Wt, t);
                 }
