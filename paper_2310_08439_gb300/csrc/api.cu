@@ -528,7 +528,7 @@ tmd_status tmd_model_create(const tmd_model_desc *d, tmd_model **out) {
     m->rc_exact = d->rc;
     {
         tmd_status su = tmd::mlp_umma_build(m, d->weights);
-        if (su == TMD_OK) su = tmd::mlp_tf32_build(m, d->weights);
+        if (su == TMD_OK) su = tmd::mlp_split_build(m, d->weights);
         if (su != TMD_OK) { tmd_model_destroy(m); return su; }
     }
     if (tmd::mlp_smem_tr_public(m->dm, 32) > 227 * 1024) {
@@ -549,7 +549,7 @@ tmd_status tmd_model_destroy(tmd_model *m) {
     if (m->dev_block) cudaFree(m->dev_block);
     if (m->dev_rtab) cudaFree(m->dev_rtab);
     if (m->dev_umma) cudaFree(m->dev_umma);
-    if (m->dev_tf32) cudaFree(m->dev_tf32);
+    if (m->dev_split) cudaFree(m->dev_split);
     delete m;
     return TMD_OK;
 }

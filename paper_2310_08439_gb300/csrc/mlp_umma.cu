@@ -33,6 +33,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <vector>
 
@@ -716,7 +717,14 @@ uint16_t bf16_bits(double x) {
     return (uint16_t)((v + 0x7fffu + ((v >> 16) & 1u)) >> 16);   // round to nearest even
 }
 
-#include "mlp_tf32.cuh"
+double bf16_value(uint16_t b) {
+    const uint32_t v = (uint32_t)b << 16;
+    float f;
+    std::memcpy(&f, &v, 4);
+    return f;
+}
+
+#include "mlp_split.cuh"
 
 }  // namespace
 
@@ -818,52 +826,60 @@ tmd_status mlp_umma_build(tmd_model *m, const double *const *weights) {
     return TMD_OK;
 }
 
-bool mlp_tf32_ok(const DevModel &dm) {
-    Tf32Net u;
-    return dm.precision == TMD_PREC_FP32 && tf32_plan(dm, u);
+bool mlp_split_ok(const DevModel &dm) {
+    SplitNet u;
+    return dm.precision == TMD_PREC_FP32 && split_plan(dm, u);
 }
 
-tmd_status mlp_tf32_launch(const char *name, const DevModel &dm, const int32_t *perm, const int32_t *types, int64_t n,
+tmd_status mlp_split_launch(const char *name, const DevModel &dm, const int32_t *perm, const int32_t *types, int64_t n,
                            const float *G, float *dG, float *e_atom, double *part_e, int *ntile_out, cudaStream_t s) {
-    Tf32Net u;
-    if (!tf32_plan(dm, u)) {
-        set_error("network shapes outside the split-TF32 kernel");
+    SplitNet u;
+    if (!split_plan(dm, u)) {
+        set_error("network shapes outside the split-operand kernel");
         return TMD_ERR_UNIMPLEMENTED;
     }
     static const cudaError_t set =
-        cudaFuncSetAttribute(k_mlp_tf32, cudaFuncAttributeMaxDynamicSharedMemorySize, TF_SMEM_MAX);
+        cudaFuncSetAttribute(k_mlp_split, cudaFuncAttributeMaxDynamicSharedMemorySize, SN_SMEM_MAX);
     TMD_CUDA(set);
     const int ntile = (int)((n + UM - 1) / UM);
     int dev = 0, nsm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     const int grid = std::max(1, std::min(ntile, std::max(1, nsm) * u.blocks_per_sm));
-    TMD_LAUNCH(name, s, k_mlp_tf32<<<grid, UTHREADS, u.smem, s>>>(dm, u, perm, types, n, G, dG, e_atom, part_e, ntile));
+    TMD_LAUNCH(name, s, k_mlp_split<<<grid, UTHREADS, u.smem, s>>>(dm, u, perm, types, n, G, dG, e_atom, part_e, ntile));
     TMD_CUDA(cudaGetLastError());
     *ntile_out = ntile;
     return TMD_OK;
 }
 
-// FP32 weights split into two TF32 planes in the operand layout of k_mlp_tf32
+// FP32 weights split into three BF16 planes in the operand layout of k_mlp_split
 // (product order as mlp_umma_build; leaves dm.tb null when the widths have no
 // such form)
-tmd_status mlp_tf32_build(tmd_model *m, const double *const *weights) {
+tmd_status mlp_split_build(tmd_model *m, const double *const *weights) {
     DevModel &dm = m->dm;
     const int L = dm.L, S = dm.S;
-    if (m->dev_tf32) {
-        cudaFree(m->dev_tf32);
-        m->dev_tf32 = nullptr;
+    if (m->dev_split) {
+        cudaFree(m->dev_split);
+        m->dev_split = nullptr;
     }
     for (int s = 0; s < TMD_MAX_SPECIES; ++s) dm.tb[s] = nullptr;
-    TfShape sh;
-    if (!tf32_shape(dm, sh)) return TMD_OK;
-    size_t off = 0;
+    SplitShape sh;
+    if (!split_shape(dm, sh)) return TMD_OK;
+    size_t off = 0, toff[2 * MAX_LAYERS];   // in BF16 values
     for (int pr = 0; pr < 2 * L; ++pr) {
-        dm.toff[pr] = (int)off;
-        off += (size_t)sh.npass[pr] * sh.nk[pr] * sh.np[pr] * TKC * 2;
+        toff[pr] = off;
+        off += (size_t)sh.npass[pr] * sh.nk[pr] * sh.np[pr] * SN_KC * SN_PL;
     }
-    const size_t per = (off + 255) & ~size_t(255);   // 1 KiB aligned species blocks
-    std::vector<float> h(per * S, 0.f);
+    const size_t per = (off + 511) & ~size_t(511);   // 1 KiB aligned species blocks
+    std::vector<uint16_t> h(per * S, 0);
+    // scales (powers of two) of the descriptor columns: those of their weights
+    std::vector<float> scale((size_t)S * dm.Dd, 1.f);
+    for (int s = 0; s < S; ++s)
+        for (int k = 0; k < dm.Dd; ++k) {
+            double mx = 0.0;
+            for (int nn = 0; nn < dm.dims[1]; ++nn) mx = std::max(mx, std::fabs(weights[s][(size_t)nn * dm.Dd + k]));
+            if (mx > 0.0) scale[(size_t)s * dm.Dd + k] = (float)std::ldexp(1.0, std::min(60, std::max(-60, std::ilogb(mx))));
+        }
     for (int s = 0; s < S; ++s) {
         const double *w = weights[s];
         size_t lo[MAX_LAYERS], o = 0;
@@ -876,18 +892,29 @@ tmd_status mlp_tf32_build(tmd_model *m, const double *const *weights) {
             const int l = fwd ? pr : 2 * L - 1 - pr;
             const int in = dm.dims[l];
             const int K = fwd ? dm.dims[l] : dm.dims[l + 1], N = fwd ? dm.dims[l + 1] : dm.dims[l];
-            float *b = h.data() + per * s + dm.toff[pr];
+            uint16_t *b = h.data() + per * s + toff[pr];
             const int np = sh.np[pr];
             for (int nn = 0; nn < N; ++nn)
-                for (int k = 0; k < K; ++k) {
-                    const double v = fwd ? w[lo[l] + (size_t)nn * in + k] : w[lo[l] + (size_t)k * in + nn];
-                    const int P = nn / np, r = nn % np, c = k / TKC, kk = k % TKC;
-                    const size_t plane = (size_t)np * TKC;
-                    const size_t idx = ((size_t)P * sh.nk[pr] + c) * plane * 2 + (size_t)(r >> 3) * (8 * TKC) +
-                                       (size_t)(kk >> 2) * 32 + (r & 7) * 4 + (kk & 3);
-                    const float hi = tf32_value(v);
-                    b[idx] = hi;
-                    b[idx + plane] = tf32_value(v - (double)hi);
+                for (int k0 = 0; k0 < K; k0 += 16) {   // the K of one MMA
+                    double v[16], mx = 0.0;
+                    for (int i = 0; i < 16; ++i) {
+                        const int k = k0 + i;
+                        v[i] = fwd ? w[lo[l] + (size_t)nn * in + k] : w[lo[l] + (size_t)k * in + nn];
+                        if (pr == 0) v[i] /= scale[(size_t)s * dm.Dd + k];
+                        mx = std::max(mx, std::fabs(v[i]));
+                    }
+                    const double unit = mx > 0.0 ? std::ldexp(1.0, std::ilogb(mx) - 7) : 1.0;
+                    for (int i = 0; i < 16; ++i) {
+                        const int P = nn / np, r = nn % np, c = (k0 + i) / SN_KC, kk = (k0 + i) % SN_KC;
+                        const size_t plane = (size_t)np * SN_KC;
+                        const size_t idx = ((size_t)P * sh.nk[pr] + c) * plane * SN_PL + (size_t)(r >> 3) * (8 * SN_KC) +
+                                           (size_t)(kk >> 3) * 64 + (r & 7) * 8 + (kk & 7);
+                        double x = v[i];
+                        for (int q = 0; q < SN_PL; ++q) {
+                            b[idx + q * plane] = bf16_bits(q == 0 ? std::nearbyint(x / unit) * unit : x);
+                            x -= bf16_value(b[idx + q * plane]);
+                        }
+                    }
                 }
         }
     }
@@ -897,21 +924,17 @@ tmd_status mlp_tf32_build(tmd_model *m, const double *const *weights) {
         const int K = pr < L ? dm.dims[pr] : dm.dims[2 * L - pr], kg = pr == 0 ? sh.ka : K, np = sh.np[pr];
         for (int P = 0; P < sh.npass[pr]; ++P)
             for (int k0 = 0; k0 < K; k0 += kg) {
-                const int nk = (std::min(kg, K - k0) + TKC - 1) / TKC, half = (nk + 1) >> 1;
-                for (int hh = 0; hh < 2; ++hh)
-                    for (int plane = 1; plane >= 0; --plane)
-                        for (int c = hh ? half : 0; c < (hh ? nk : half); ++c)
-                            ck.push_back(make_int2(
-                                dm.toff[pr] + ((P * sh.nk[pr] + k0 / TKC + c) * 2 + plane) * np * TKC, np * TKC * 4));
+                for (int k = k0; k < std::min(K, k0 + kg); k += SN_KC)
+                    for (int q = SN_PL - 1; q >= 0; --q)
+                        ck.push_back(make_int2((int)toff[pr] + ((P * sh.nk[pr] + k / SN_KC) * SN_PL + q) * np * SN_KC, np * SN_KC * 2));
             }
     }
-    int at[MAX_LAYERS + 1];
-    const int cstride = tf32_consts(dm, at);
-    const size_t c0 = h.size();
-    h.resize(c0 + ((size_t)cstride * S + 1) / 2 * 2, 0.f);
+    int at[MAX_LAYERS + 2];
+    const int cstride = split_consts(dm, at);
+    std::vector<float> cst(((size_t)cstride * S + 1) / 2 * 2, 0.f);
     for (int s = 0; s < S; ++s) {
         const double *w = weights[s];
-        float *c = h.data() + c0 + (size_t)s * cstride;
+        float *c = cst.data() + (size_t)s * cstride;
         for (int l = 0; l <= L; ++l) {   // layer L: the output (weights, then its bias)
             const size_t nw = (size_t)dm.dims[l] * dm.dims[l + 1];
             for (int j = 0; j < dm.dims[l + 1]; ++j) c[l < L ? at[l] + j : at[L + 1]] = (float)w[nw + j];
@@ -919,21 +942,24 @@ tmd_status mlp_tf32_build(tmd_model *m, const double *const *weights) {
                 for (int j = 0; j < dm.dims[L]; ++j) c[at[L] + j] = (float)w[j];
             w += nw + dm.dims[l + 1];
         }
+        std::copy_n(scale.data() + (size_t)s * dm.Dd, dm.Dd, c + at[L + 2]);
     }
     void *dev = nullptr;
-    cudaError_t e = cudaMalloc(&dev, sizeof(float) * h.size() + sizeof(int2) * ck.size());
+    const size_t b_w = sizeof(uint16_t) * h.size(), b_c = sizeof(float) * cst.size();   // (multiples of 8)
+    cudaError_t e = cudaMalloc(&dev, b_w + b_c + sizeof(int2) * ck.size());
     if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc split weights");
-    e = cudaMemcpy(dev, h.data(), sizeof(float) * h.size(), cudaMemcpyHostToDevice);
-    int2 *const ck_dev = reinterpret_cast<int2 *>(static_cast<float *>(dev) + h.size());
-    if (e == cudaSuccess) e = cudaMemcpy(ck_dev, ck.data(), sizeof(int2) * ck.size(), cudaMemcpyHostToDevice);
+    unsigned char *const at_w = static_cast<unsigned char *>(dev);
+    e = cudaMemcpy(at_w, h.data(), b_w, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(at_w + b_w, cst.data(), b_c, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(at_w + b_w + b_c, ck.data(), sizeof(int2) * ck.size(), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         cudaFree(dev);
         return cuda_fail(e, "cudaMemcpy split weights");
     }
-    m->dev_tf32 = dev;
-    dm.tck = ck_dev;
-    dm.tconst = static_cast<const float *>(dev) + c0;
-    for (int s = 0; s < S; ++s) dm.tb[s] = static_cast<const float *>(dev) + per * s;
+    m->dev_split = dev;
+    dm.tck = reinterpret_cast<const int2 *>(at_w + b_w + b_c);
+    dm.tconst = reinterpret_cast<const float *>(at_w + b_w);
+    for (int s = 0; s < S; ++s) dm.tb[s] = reinterpret_cast<const uint16_t *>(dev) + per * s;
     return TMD_OK;
 }
 

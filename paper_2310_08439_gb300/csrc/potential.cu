@@ -961,14 +961,14 @@ static tmd_status launch_network(const DevModel &dm, const int32_t *perm, const 
         return TMD_ERR_UNIMPLEMENTED;
     }
     // FP32: the tensor cores wherever the widths are multiples of 16 up to 128,
-    // the descriptor has at most 192 columns (for its accuracy, TF_DD) and a tile
-    // fits on chip; k_mlp has the rest.  At every size: one 32-atom
-    // tile 15.5 us against 15.6 in k_mlp, 1,048,576 atoms x 64-64 423 us
-    // against 850, 147,456 atoms x 128-128-128 254 us against 922 (k_mlp).
+    // the descriptor has at most 192 columns (SN_DD) and a tile fits on chip;
+    // k_mlp has the rest.  At every size: one 32-atom tile 16.3 us against 15.6 in
+    // k_mlp, 1,048,576 atoms x 64-64 420 us against 850, 147,456 atoms x
+    // 128-128-128 247 us against 922 (k_mlp).
     // Two labels, as tile_rows has two kinds of tile: "k_mlp_res" where 0 or
     // 128 stands for 128-atom tiles, else "k_mlp".
-    if (mlp_tf32_ok(dm))
-        return mlp_tf32_launch(mlp_all64(dm) && (dm.tile_rows == 0 || dm.tile_rows == 128) ? "k_mlp_res" : "k_mlp", dm,
+    if (mlp_split_ok(dm))
+        return mlp_split_launch(mlp_all64(dm) && (dm.tile_rows == 0 || dm.tile_rows == 128) ? "k_mlp_res" : "k_mlp", dm,
                                perm, types, n, G, dG, e_atom, part_e, ntile_out, s);
     if ((st = set_mlp_smem(dm, dm.precision == TMD_PREC_BF16)) != TMD_OK) return st;
     if (dm.precision == TMD_PREC_BF16) {

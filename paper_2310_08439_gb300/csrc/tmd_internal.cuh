@@ -55,12 +55,11 @@ struct DevModel {
     // elements, as [N pass][64-wide K chunk][N/8][8 core matrices][8 x 8]
     const uint16_t *ub[TMD_MAX_SPECIES];
     int uoff[2 * MAX_LAYERS];
-    // FP32 weights as two TF32 planes in the tcgen05 operand layout (nullptr:
-    // not built): product p at toff[p] floats, as [N pass][32-wide K chunk]
-    // [plane][N/8][8 core matrices][8 x 4]
-    const float *tb[TMD_MAX_SPECIES];
-    int toff[2 * MAX_LAYERS];
-    const float *tconst;   // biases, output weights and output bias of the species
+    // FP32 weights as three BF16 planes in the tcgen05 operand layout (nullptr:
+    // not built): per product [N pass][64-wide K chunk][plane][N/8][8 core
+    // matrices][8 x 8]
+    const uint16_t *tb[TMD_MAX_SPECIES];
+    const float *tconst;   // biases, output weights, output bias and column scales of the species
     const int2 *tck;   // per copy of a species, in order: offset in tb[s], bytes
 };
 
@@ -76,9 +75,9 @@ size_t mlp_bf16_smem_bytes(const DevModel &dm);
 bool mlp_umma_supported(const DevModel &dm);
 tmd_status mlp_umma_launch(const DevModel &dm, const int32_t *perm, const int32_t *types, int64_t n, const float *G,
                            float *dG, float *e_atom, double *part_e, int *ntile_out, cudaStream_t s);
-// tcgen05 form of the FP32 network on split TF32 operands (mlp_tf32.cuh)
-bool mlp_tf32_ok(const DevModel &dm);
-tmd_status mlp_tf32_launch(const char *name, const DevModel &dm, const int32_t *perm, const int32_t *types, int64_t n,
+// tcgen05 form of the FP32 network on split operands (mlp_split.cuh)
+bool mlp_split_ok(const DevModel &dm);
+tmd_status mlp_split_launch(const char *name, const DevModel &dm, const int32_t *perm, const int32_t *types, int64_t n,
                            const float *G, float *dG, float *e_atom, double *part_e, int *ntile_out, cudaStream_t s);
 // network kernel of the BF16 form: 0 = tcgen05 when the shapes allow it, else
 // mma.sync; 1 = tcgen05 only; 2 = mma.sync only
@@ -142,7 +141,7 @@ struct tmd_model {
     int precision = TMD_PREC_FP32;
     float *dev_rtab = nullptr;  // tabulated radial basis (tmd_model_set_radial_table)
     void *dev_umma = nullptr;   // BF16 weights in the tcgen05 operand layout
-    void *dev_tf32 = nullptr;   // FP32 weights as two TF32 planes in the tcgen05 operand layout
+    void *dev_split = nullptr;   // FP32 weights as three BF16 planes in the tcgen05 operand layout
     std::vector<double> mu, eta; // radial parameters [S][S][K] (host copy, for tables)
     double rc_exact = 0.0;
 };
@@ -346,7 +345,7 @@ tmd_status launch_screen(const DevModel &dm, const DevNlist &dn, cudaStream_t s)
 // dm.ub null when the widths have no BF16 form); status bits of the
 // tensor-core kernels, read and cleared (synchronises)
 tmd_status mlp_umma_build(tmd_model *m, const double *const *weights);
-tmd_status mlp_tf32_build(tmd_model *m, const double *const *weights);
+tmd_status mlp_split_build(tmd_model *m, const double *const *weights);
 tmd_status umma_status(int32_t *bits);
 tmd_status wait_probe(int32_t *gave_up);
 extern int g_network_kernel;

@@ -69,3 +69,50 @@ def test_constants_of_the_ranks(tmdlib):
     below a quarter of a unit in the last place, half of either."""
     mean = np.mean([_mean_errors(tmdlib, *c) for c in CASES], axis=0)
     assert np.abs(mean[2:]).max() <= 2.0 ** -26
+
+
+def _gradient64(p, G, types):
+    """dE_a/dG_a of the network at these descriptors, in FP64."""
+    dG = np.zeros_like(G)
+    for t in range(p.n_species):
+        layers = p.unpack(t)
+        rows = types == t
+        a, d = G[rows], []
+        for W, b in layers[:-1]:
+            z = a @ W.T + b
+            if p.activation == "tanh":
+                a = np.tanh(z)
+                d.append(1.0 - a * a)
+            else:
+                q = np.sqrt(z * z + p.squareplus_b)
+                a = 0.5 * (z + q)
+                d.append(a / q)
+        g = np.repeat(layers[-1][0], rows.sum(), axis=0)
+        for (W, _), da in zip(layers[:-1][::-1], d[::-1]):
+            g = (g * da) @ W
+        dG[rows] = g
+    return dG
+
+
+@pytest.mark.parametrize("floor", [0.1, 1e-4])   # 1e-4: columns of very different weights
+@pytest.mark.parametrize("S,K,widths,act", [(1, 16, [64], "tanh"), (1, 16, [64, 64], "tanh"),
+                                            (2, 8, [64, 64], "squareplus"), (3, 16, [128, 128], "tanh"),
+                                            (1, 32, [128, 128, 128], "squareplus"), (1, 8, [16, 48], "tanh")])
+def test_network_sums_are_as_exact_as_their_rounding(tmdlib, S, K, widths, act, floor, capsys):
+    """dE/dG of the network against FP64 at the descriptors that it was given.
+    A hidden layer rounds about 12 numbers one after the other (the sums and the
+    bias, the activation and its derivative, the way back); each is off by at most
+    half a unit, 2^-24 / sqrt(12) rms, and what is off early goes through the rest
+    twice: 2 sqrt(12 L) 2^-24 / sqrt(12) = 2^-23 sqrt(L) for L layers.  The products
+    themselves must add nothing to that."""
+    s = _system(S, 3 * S + K)
+    def model(scale):
+        return I.random_model(S, K, RC, widths, seed=K + len(widths), activation=act, feature_scale=scale, scale_floor=floor)
+    G0 = O.evaluate(O.OracleModel(model(None)), s.pos, s.types, s.box, s.pbc, want_G=True)["G"]
+    p = model([np.sqrt((G0[s.types == t] ** 2).mean(axis=0)) for t in range(S)])
+    G, dG = _descriptors(tmdlib, tmdlib.Model(p), s)
+    ref = _gradient64(p, G, s.types)
+    err = float(np.linalg.norm(dG - ref) / np.linalg.norm(ref))
+    with capsys.disabled():
+        print(f"\n[S={S} K={K} {widths} {act} floor {floor}] dE/dG error {err:.2e}")
+    assert err <= 2.0 ** -23 * np.sqrt(len(widths))
