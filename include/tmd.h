@@ -99,11 +99,19 @@ const char *tmd_version(void);
  *             c = ((b*K) + k)*4 + m, b = neighbour species.
  *  activation TMD_ACT_TANH or TMD_ACT_SQUAREPLUS (b = squareplus_b); the
  *             output layer is linear.
- *  precision  TMD_PREC_FP32: every layer in FP32.  TMD_PREC_BF16: network
- *             layers on BF16 tensor cores with FP32 accumulation (input,
- *             activations and weights rounded to BF16; hidden widths must be
- *             multiples of 16, else TMD_ERR_UNIMPLEMENTED); radial basis,
- *             moments and contractions stay FP32 in both modes.
+ *  precision  TMD_PREC_FP32: every layer in FP32: inputs, weights and
+ *             activations are held to 24 bits and summed in FP32.  Where the
+ *             tensor cores form the products (hidden widths multiples of 16 up
+ *             to 128) an operand goes in as three BF16 parts that together
+ *             hold its 24 bits, and dE/dG is 0.4 to 0.7 times as far from FP64
+ *             as with FP32 multiply-adds.  TMD_PREC_BF16: network layers on
+ *             BF16 tensor cores with FP32 accumulation (input, activations and
+ *             weights rounded to BF16; hidden widths must be multiples of 16,
+ *             else TMD_ERR_UNIMPLEMENTED).  In both modes radial basis, moments
+ *             and contractions are FP32; the sums over pairs of the descriptor
+ *             run on the tensor cores with operands in two TF32 parts (23 to 24
+ *             bits) and are added in FP32: G is 0.95 to 1.03 times as far from
+ *             FP64 as with FP32 multiply-adds.
  */
 typedef struct {
     int32_t n_species;
@@ -230,9 +238,8 @@ int64_t tmd_graph_replays(void);
  *                      pipes: 32 or 64; 128 (networks whose descriptor length
  *                      and hidden widths are all 64, one or two hidden layers)
  *                      and 0 = built-in choice.  Networks that run on the
- *                      tensor cores (descriptor length up to 192, hidden
- *                      widths multiples of 16 up to 128, activations of a tile
- *                      within an SM's shared memory)
+ *                      tensor cores (hidden widths multiples of 16 up to 128,
+ *                      activations of a tile within an SM's shared memory)
  *                      have 128-atom tiles with each of them;
  *  pair_blocks_per_sm  blocks per SM of the persistent descriptor / force
  *                      grids (0 = built-in 16);

@@ -97,7 +97,10 @@ def _gradient64(p, G, types):
 @pytest.mark.parametrize("floor", [0.1, 1e-4])   # 1e-4: columns of very different weights
 @pytest.mark.parametrize("S,K,widths,act", [(1, 16, [64], "tanh"), (1, 16, [64, 64], "tanh"),
                                             (2, 8, [64, 64], "squareplus"), (3, 16, [128, 128], "tanh"),
-                                            (1, 32, [128, 128, 128], "squareplus"), (1, 8, [16, 48], "tanh")])
+                                            (1, 32, [128, 128, 128], "squareplus"), (1, 8, [16, 48], "tanh"),
+                                            # 160 (in 5 passes of G'), 256, 320 and 640 columns
+                                            (5, 8, [64, 64], "tanh"), (1, 64, [128, 128], "squareplus"),
+                                            (5, 16, [112], "tanh"), (5, 32, [64, 32], "tanh")])
 def test_network_sums_are_as_exact_as_their_rounding(tmdlib, S, K, widths, act, floor, capsys):
     """dE/dG of the network against FP64 at the descriptors that it was given.
     A hidden layer rounds about 12 numbers one after the other (the sums and the
