@@ -213,11 +213,23 @@ tmd_status tmd_set_network_kernel(int32_t kind);
  * INVALID_ARG. */
 tmd_status tmd_set_force_kernel(int32_t kind);
 
-/* Status bits recorded by device kernels that have no neighbour table to
- * report through (today: a bounded wait of the tcgen05 network kernel that
- * gave up), read and cleared.  Returns TMD_ERR_TIMEOUT when such a wait ran
- * out since the last call (the results of the calls in between are invalid),
- * else TMD_OK; *bits receives the raw bits.  Synchronises the device. */
+/* Status bits recorded by device kernels (today: a bounded wait of a tcgen05
+ * network kernel that gave up), read and cleared.  Returns TMD_ERR_TIMEOUT when
+ * such a wait ran out since the last call, else TMD_OK; *bits receives the raw
+ * bits.  Synchronises the device.
+ *
+ * The tcgen05 network kernels (BF16 and FP32, see precision) wait for their own
+ * copies and products for at most 0.2 s at a time.  A kernel that gives up (a
+ * GPU taken away for longer in the middle of it) ends in order, and the whole
+ * evaluation is invalid, never partly so in silence:
+ *  - tmd_compute, _owned, _noalloc and tmd_descriptors, which only enqueue work:
+ *    energy, virial, all forces, and e_atom and dE/dG of the atoms concerned
+ *    are NaN;
+ *  - tmd_evaluate_host, tmd_batch_compute, tmd_batch_step, tmd_step with thermo,
+ *    tmd_step_host and tmd_system_get_state return TMD_ERR_TIMEOUT; tmd_step
+ *    without thermo in the next call that waits for the system.  A run of steps
+ *    (skin > 0, see tmd_step) is undone and stepped again instead; otherwise the
+ *    system's or systems' state is to be set again. */
 tmd_status tmd_device_status(int32_t *bits);
 
 /* Self-test of the bounded waits of the tensor-core kernels: one warp
@@ -228,6 +240,12 @@ tmd_status tmd_device_status(int32_t *bits);
  * usable.  *gave_up (host) = 1 when the wait gave up as designed.  Errors:
  * INVALID_ARG, CUDA.  Synchronises the device. */
 tmd_status tmd_selftest_bounded_wait(int32_t *gave_up);
+
+/* Self-test of what follows such a wait: the next network launched on tensor
+ * cores by this process (outside a stream capture) is treated as one that gave
+ * up in its last 128 atoms, though it did not: its outputs become NaN and the
+ * time-out is recorded as above.  No wait runs out. */
+tmd_status tmd_selftest_network_timeout(void);
 int64_t tmd_graph_replays(void);
 
 /*

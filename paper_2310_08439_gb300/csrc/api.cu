@@ -119,6 +119,17 @@ constexpr double ACC_CONV = 1.0 / 103.6427;
 constexpr double FQ_UNIT = 1.0 / 4294967296.0;   // the force accumulator's unit, 2^-32 eV/A
 constexpr double KB_EV = 8.617333262e-5;
 
+// TMD_ERR_TIMEOUT when the time-out word of a system or batch, read back to *w,
+// is set: what it holds is not the result of a whole evaluation
+tmd_status timed_out(const void *w, const char *what) {
+    int32_t v = 0;
+    std::memcpy(&v, w, sizeof(v));
+    if (!v) return TMD_OK;
+    set_error("a bounded wait of the network kernel gave up; %s", what);
+    return TMD_ERR_TIMEOUT;
+}
+constexpr const char * SYSTEM_INVALID = "the state of the system is invalid: set it again";
+
 // Half kick and drift.  Positions are not wrapped here: the neighbour table's
 // image shifts refer to the positions at the last build, so atoms move
 // continuously until the next rebuild, which wraps them first.
@@ -188,13 +199,14 @@ __global__ void k_wrap(double *__restrict__ pos, int64_t n, double L0, double L1
 // accumulator (int64, 2^-32 eV/A) to the FP32 forces it also writes: the
 // same values as the conversion and the kick launched one after the other
 __global__ void k_vv_second_fq(double *__restrict__ vel, const long long *__restrict__ Fq, float *__restrict__ F,
-                               const double *__restrict__ inv_mass, int64_t n, double dt) {
+                               const double *__restrict__ inv_mass, int64_t n, double dt,
+                               const int32_t *__restrict__ err) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const double h = 0.5 * dt * inv_mass[i] * ACC_CONV;
 #pragma unroll
     for (int x = 0; x < 3; ++x) {
-        const float f = (float)((double)Fq[3 * i + x] * FQ_UNIT);
+        const float f = *err ? NAN : (float)((double)Fq[3 * i + x] * FQ_UNIT);   // (as k_forces_out)
         F[3 * i + x] = f;
         vel[3 * i + x] += h * (double)f;
     }
@@ -730,6 +742,11 @@ tmd_status tmd_set_graphs(int32_t on) {
     return TMD_OK;
 }
 
+tmd_status tmd_selftest_network_timeout(void) {
+    tmd::arm_network_timeout();
+    return TMD_OK;
+}
+
 int64_t tmd_graph_replays(void) { return g_replays; }
 
 tmd_status tmd_model_set_tuning(tmd_model *m, const tmd_tuning *t) {
@@ -946,6 +963,11 @@ tmd_status tmd_evaluate_host(const tmd_model *model, tmd_nlist *nl, const double
     if (forces_host && n > 0)
         TMD_CUDA(cudaMemcpyAsync(forces_host, nl->io_forces, sizeof(float) * 3 * n, cudaMemcpyDeviceToHost, s));
     TMD_CUDA(cudaStreamSynchronize(s));
+    if (n > 0 && !(energy_host && std::isfinite(*energy_host))) {   // (an invalid evaluation has an energy of NaN)
+        int32_t w = 0;
+        TMD_CUDA(cudaMemcpy(&w, nl->err, sizeof(w), cudaMemcpyDeviceToHost));
+        return timed_out(&w, "the results are invalid");
+    }
     return TMD_OK;
 }
 
@@ -976,6 +998,7 @@ tmd_status tmd_system_create(int64_t n, const double box[3], const int32_t pbc[3
     if (e == cudaSuccess) e = cudaMemset(sys->vel, 0, sizeof(double) * 3 * n);
     if (e == cudaSuccess) e = cudaMemset(sys->forces, 0, sizeof(float) * 3 * n);
     if (e == cudaSuccess) e = cudaMemset(sys->red, 0, sizeof(double) * 32);
+    if (e == cudaSuccess) sys->nl.err_ext = reinterpret_cast<int32_t *>(sys->red + 21);
     if (e != cudaSuccess) {
         tmd_system_destroy(sys);
         cudaGetLastError();
@@ -988,7 +1011,7 @@ tmd_status tmd_system_create(int64_t n, const double box[3], const int32_t pbc[3
 
 tmd_status tmd_system_destroy(tmd_system *sys) {
     if (!sys) return TMD_OK;
-    void *sp_[] = {sys->snap_pos, sys->snap_vel, sys->snap_forces, sys->run_flags};
+    void *sp_[] = {sys->snap_pos, sys->snap_vel, sys->snap_forces};
     for (void *q : sp_)
         if (q) cudaFree(q);
     if (sys->h_run) cudaFreeHost(sys->h_run);
@@ -1022,6 +1045,7 @@ tmd_status tmd_system_set_state(tmd_system *sys, const double *pos, const double
         TMD_CUDA(cudaGetLastError());
     }
     if (!on_device) TMD_CUDA(cudaStreamSynchronize(s));  // host arrays may be pageable and reused
+    TMD_CUDA(cudaMemsetAsync(sys->red + 21, 0, sizeof(int32_t), s));   // a new state is a valid one
     sys->step = 0;
     sys->rebuilds = 0;
     sys->need_rebuild = 1;
@@ -1038,8 +1062,9 @@ tmd_status tmd_system_get_state(const tmd_system *sys, double *pos, double *vel,
     if (pos) TMD_CUDA(cudaMemcpyAsync(pos, sys->pos, sizeof(double) * 3 * n, k, s));
     if (vel) TMD_CUDA(cudaMemcpyAsync(vel, sys->vel, sizeof(double) * 3 * n, k, s));
     if (forces) TMD_CUDA(cudaMemcpyAsync(forces, sys->forces, sizeof(float) * 3 * n, k, s));
+    TMD_CUDA(cudaMemcpyAsync(sys->h_red + 21, sys->red + 21, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     TMD_CUDA(cudaStreamSynchronize(s));
-    return TMD_OK;
+    return timed_out(sys->h_red + 21, SYSTEM_INVALID);
 }
 
 // The system's split-position arrays when they have room for its atoms (the
@@ -1092,8 +1117,9 @@ static tmd_status step_eager(const tmd_model *model, tmd_system *sys, double dt_
     sys->step++;
     bool rebuild = sys->need_rebuild || (rebuild_every > 0 && (sys->step % rebuild_every) == 0);
     if (!rebuild) {
-        TMD_CUDA(cudaMemcpyAsync(sys->h_red + 20, flag, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+        TMD_CUDA(cudaMemcpyAsync(sys->h_red + 20, flag, 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
         TMD_CUDA(cudaStreamSynchronize(s));
+        if ((st = timed_out(sys->h_red + 21, SYSTEM_INVALID)) != TMD_OK) return st;   // (of the steps before)
         int32_t f = 0;
         std::memcpy(&f, sys->h_red + 20, sizeof(int32_t));
         rebuild = (f & 1) != 0;
@@ -1117,7 +1143,7 @@ static tmd_status step_eager(const tmd_model *model, tmd_system *sys, double dt_
         if (st2 != TMD_OK) return st2;
         TMD_LAUNCH("k_vv_second", s, k_vv_second_fq<<<nb, 256, 0, s>>>(
                                          sys->vel, reinterpret_cast<const long long *>(sys->nl.Fq), sys->forces,
-                                         sys->inv_mass, n, dt_fs));
+                                         sys->inv_mass, n, dt_fs, sys->nl.err_ext));
         TMD_CUDA(cudaGetLastError());
         return TMD_OK;
     });
@@ -1130,8 +1156,8 @@ constexpr int RUN_MAX = 16;   // steps per launch sequence when no cadence sets 
 // whose rebuild runs on the device (build_tables device_only), and every
 // other step records its skin check in its own flag.  The flags, the table's
 // entry counter and its status are read once at the end.  A run in which an
-// atom moved more than skin / 2 before a rebuild was due, or whose table
-// overflowed, is undone and stepped again on the host-decided path, so the
+// atom moved more than skin / 2 before a rebuild was due, whose table
+// overflowed or whose network gave up waiting, is undone and stepped again on the host-decided path, so the
 // trajectory is always the one that path gives.
 static tmd_status step_run(const tmd_model *model, tmd_system *sys, double dt_fs, int k, bool rebuild_first,
                            cudaStream_t s, bool *redo) {
@@ -1144,8 +1170,7 @@ static tmd_status step_run(const tmd_model *model, tmd_system *sys, double dt_fs
         cudaError_t e = cudaMalloc(&sys->snap_pos, sizeof(double) * 3 * n);
         if (e == cudaSuccess) e = cudaMalloc(&sys->snap_vel, sizeof(double) * 3 * n);
         if (e == cudaSuccess) e = cudaMalloc(&sys->snap_forces, sizeof(float) * 3 * n);
-        if (e == cudaSuccess) e = cudaMalloc(&sys->run_flags, sizeof(int32_t) * RUN_MAX);
-        if (e == cudaSuccess) e = cudaMallocHost(&sys->h_run, sizeof(int64_t) * (RUN_MAX + 4));
+        if (e == cudaSuccess) e = cudaMallocHost(&sys->h_run, sizeof(int64_t) * 13);
         if (e != cudaSuccess) {
             cudaGetLastError();
             set_error("run state: %s", cudaGetErrorString(e));
@@ -1154,6 +1179,7 @@ static tmd_status step_run(const tmd_model *model, tmd_system *sys, double dt_fs
     }
     if ((st = reserve_compute(model->dm, &sys->nl, n, n)) != TMD_OK) return st;
     tmd_nlist *nl = &sys->nl;
+    int32_t *const run_flags = reinterpret_cast<int32_t *>(sys->red + 24);
     SysParams q;
     int64_t ncell = 0;
     if (rebuild_first &&
@@ -1176,11 +1202,11 @@ static tmd_status step_run(const tmd_model *model, tmd_system *sys, double dt_fs
         TMD_CUDA(cudaMemcpyAsync(sys->snap_pos, sys->pos, sizeof(double) * 3 * n, cudaMemcpyDeviceToDevice, s));
         TMD_CUDA(cudaMemcpyAsync(sys->snap_vel, sys->vel, sizeof(double) * 3 * n, cudaMemcpyDeviceToDevice, s));
         TMD_CUDA(cudaMemcpyAsync(sys->snap_forces, sys->forces, sizeof(float) * 3 * n, cudaMemcpyDeviceToDevice, s));
-        TMD_CUDA(cudaMemsetAsync(sys->run_flags, 0, sizeof(int32_t) * RUN_MAX, s));
+        TMD_CUDA(cudaMemsetAsync(run_flags, 0, sizeof(int32_t) * RUN_MAX, s));
         for (int j = 0; j < k; ++j) {
             TMD_LAUNCH("k_vv_first", s, k_vv_first<<<nb, 256, 0, s>>>(sys->pos, sys->vel, sys->forces, sys->inv_mass,
                                                                       n, dt_fs, sys->pos_ref, lim * lim,
-                                                                      sys->run_flags + j, ph, pl));
+                                                                      run_flags + j, ph, pl));
             if (j == 0 && rebuild_first) {
                 TMD_LAUNCH("k_wrap", s, k_wrap<<<nb, 256, 0, s>>>(sys->pos, n, sys->box[0], sys->box[1], sys->box[2],
                                                                   sys->pbc[0], sys->pbc[1], sys->pbc[2], ph, pl));
@@ -1194,18 +1220,20 @@ static tmd_status step_run(const tmd_model *model, tmd_system *sys, double dt_fs
             if (c != TMD_OK) return c;
             TMD_LAUNCH("k_vv_second", s, k_vv_second_fq<<<nb, 256, 0, s>>>(
                                              sys->vel, reinterpret_cast<const long long *>(nl->Fq), sys->forces,
-                                             sys->inv_mass, n, dt_fs));
+                                             sys->inv_mass, n, dt_fs, nl->err_ext));
             TMD_CUDA(cudaGetLastError());
         }
         return TMD_OK;
     });
     if (st != TMD_OK) return st;
-    TMD_CUDA(cudaMemcpyAsync(sys->h_run, sys->run_flags, sizeof(int32_t) * RUN_MAX, cudaMemcpyDeviceToHost, s));
-    TMD_CUDA(cudaMemcpyAsync(sys->h_run + RUN_MAX / 2, nl->counter, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    TMD_CUDA(cudaMemcpyAsync(sys->h_run + RUN_MAX / 2 + 1, nl->status, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    static_assert(RUN_MAX == 16, "red[24..31] holds the flags of a run");
+    TMD_CUDA(cudaMemcpyAsync(sys->h_run, sys->red + 21, sizeof(double) * 11, cudaMemcpyDeviceToHost, s));
+    TMD_CUDA(cudaMemcpyAsync(sys->h_run + 11, nl->counter, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+    TMD_CUDA(cudaMemcpyAsync(sys->h_run + 12, nl->status, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     TMD_CUDA(cudaStreamSynchronize(s));
     int32_t flags[RUN_MAX];
-    std::memcpy(flags, sys->h_run, sizeof(flags));
+    std::memcpy(flags, sys->h_run + 3, sizeof(flags));
+    const bool invalid = (int32_t)sys->h_run[0] != 0;   // (the time-out word)
     bool moved = false, near = false;
     for (int j = rebuild_first ? 1 : 0; j < k; ++j) {
         moved = moved || (flags[j] & 1) != 0;
@@ -1214,10 +1242,18 @@ static tmd_status step_run(const tmd_model *model, tmd_system *sys, double dt_fs
     bool bad_table = false;
     if (rebuild_first) {
         int32_t status = 0;
-        std::memcpy(&status, sys->h_run + RUN_MAX / 2 + 1, sizeof(int32_t));
-        bad_table = sys->h_run[RUN_MAX / 2] > std::min(nl->cap_nnz, nl->cap_shift) || status != 0;
+        std::memcpy(&status, sys->h_run + 12, sizeof(int32_t));
+        bad_table = sys->h_run[11] > std::min(nl->cap_nnz, nl->cap_shift) || status != 0;
     }
-    if (moved || bad_table) {   // undo: back to the state at the start of the run
+    if (moved || bad_table || invalid) {   // undo: back to the state at the start of the run
+        if (invalid) {
+            // (all forces at the start are NaN if it was a step before the run that gave up)
+            float f0 = 0.f;
+            TMD_CUDA(cudaMemcpyAsync(&f0, sys->snap_forces, sizeof(float), cudaMemcpyDeviceToHost, s));
+            TMD_CUDA(cudaStreamSynchronize(s));
+            if (std::isnan(f0)) return timed_out(sys->h_run, SYSTEM_INVALID);
+            TMD_CUDA(cudaMemsetAsync(sys->red + 21, 0, sizeof(int32_t), s));
+        }
         TMD_CUDA(cudaMemcpyAsync(sys->pos, sys->snap_pos, sizeof(double) * 3 * n, cudaMemcpyDeviceToDevice, s));
         TMD_CUDA(cudaMemcpyAsync(sys->vel, sys->snap_vel, sizeof(double) * 3 * n, cudaMemcpyDeviceToDevice, s));
         TMD_CUDA(cudaMemcpyAsync(sys->forces, sys->snap_forces, sizeof(float) * 3 * n, cudaMemcpyDeviceToDevice, s));
@@ -1290,8 +1326,9 @@ tmd_status tmd_step(const tmd_model *model, tmd_system *sys, double dt_fs, int32
         TMD_LAUNCH("k_kinetic", s, k_kinetic<<<kb, 256, 0, s>>>(sys->vel, sys->mass, n, sys->part));
         TMD_LAUNCH("k_kinetic_total", s, k_kinetic_total<<<1, 192, 0, s>>>(sys->part, kb, sys->red + 10));
         TMD_CUDA(cudaGetLastError());
-        TMD_CUDA(cudaMemcpyAsync(sys->h_red, sys->red, sizeof(double) * 16, cudaMemcpyDeviceToHost, s));
+        TMD_CUDA(cudaMemcpyAsync(sys->h_red, sys->red, sizeof(double) * 22, cudaMemcpyDeviceToHost, s));
         TMD_CUDA(cudaStreamSynchronize(s));
+        if ((st = timed_out(sys->h_red + 21, SYSTEM_INVALID)) != TMD_OK) return st;
         const double *r = sys->h_red;
         const double conv = 1.0 / ACC_CONV;  // amu A^2/fs^2 -> eV
         const double mvv[9] = {r[10], r[13], r[14], r[13], r[11], r[15], r[14], r[15], r[12]};
@@ -1328,6 +1365,7 @@ tmd_status tmd_step_host(const tmd_model *model, tmd_system *sys, double *pos_ho
     const int64_t n = sys->n;
     TMD_CUDA(cudaMemcpyAsync(sys->pos, pos_host, sizeof(double) * 3 * n, cudaMemcpyHostToDevice, s));
     TMD_CUDA(cudaMemcpyAsync(sys->vel, vel_host, sizeof(double) * 3 * n, cudaMemcpyHostToDevice, s));
+    TMD_CUDA(cudaMemsetAsync(sys->red + 21, 0, sizeof(int32_t), s));   // a new state is a valid one
     if (forces_host) {
         TMD_CUDA(cudaMemcpyAsync(sys->forces, forces_host, sizeof(float) * 3 * n, cudaMemcpyHostToDevice, s));
         sys->have_forces = 1;
@@ -1343,8 +1381,9 @@ tmd_status tmd_step_host(const tmd_model *model, tmd_system *sys, double *pos_ho
     TMD_CUDA(cudaMemcpyAsync(pos_host, sys->pos, sizeof(double) * 3 * n, cudaMemcpyDeviceToHost, s));
     TMD_CUDA(cudaMemcpyAsync(vel_host, sys->vel, sizeof(double) * 3 * n, cudaMemcpyDeviceToHost, s));
     if (forces_host) TMD_CUDA(cudaMemcpyAsync(forces_host, sys->forces, sizeof(float) * 3 * n, cudaMemcpyDeviceToHost, s));
+    TMD_CUDA(cudaMemcpyAsync(sys->h_red + 21, sys->red + 21, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     TMD_CUDA(cudaStreamSynchronize(s));
-    return TMD_OK;
+    return timed_out(sys->h_red + 21, SYSTEM_INVALID);
 }
 
 
@@ -1367,7 +1406,8 @@ struct tmd_batch {
     int64_t *d_off = nullptr;
     uint8_t *active = nullptr;       // [S] device flags
     int32_t *act_list = nullptr;     // [S] device list of active systems
-    double *sys_out = nullptr;       // [S][16] device per-system sums
+    double *sys_hdr = nullptr;       // [2] device: the time-out word (pool.err_ext), read back with the sums
+    double *sys_out = nullptr;       // [S][16] device per-system sums (sys_hdr + 2)
     double *h_out = nullptr;         // pinned mirror
     int32_t *h_act = nullptr;        // pinned staging of the active list
     uint8_t *h_flags = nullptr;      // pinned staging of the flags
@@ -1643,10 +1683,22 @@ tmd_status batch_eval(const tmd_model *model, tmd_batch *b, int32_t n_act, cudaS
     return batch_compute_only(model, b, n_act, s);
 }
 
+// the sums of the active systems and the time-out word; when that is set, the
+// active systems are without forces (and, after steps, without a valid state)
+tmd_status batch_read(tmd_batch *b, int32_t n_act, cudaStream_t s) {
+    TMD_CUDA(cudaMemcpyAsync(b->h_out, b->sys_hdr, sizeof(double) * (2 + 16 * (size_t)n_act), cudaMemcpyDeviceToHost, s));
+    TMD_CUDA(cudaStreamSynchronize(s));
+    const tmd_status st = timed_out(b->h_out, "the listed systems have no forces and, after steps, no valid state");
+    if (st == TMD_OK) return TMD_OK;
+    TMD_CUDA(cudaMemsetAsync(b->sys_hdr, 0, sizeof(int32_t), s));
+    for (int k = 0; k < n_act; ++k) b->has_forces[b->h_act[k]] = 0;
+    return st;
+}
+
 void batch_results(tmd_batch *b, int32_t n_act, double *energy, double *virial, tmd_thermo *thermo) {
     const double conv = 103.6427;  // amu A^2/fs^2 -> eV
     for (int k = 0; k < n_act; ++k) {
-        const double *r = b->h_out + 16 * k;
+        const double *r = b->h_out + 2 + 16 * k;
         const int sys = b->h_act[k];
         if (energy) energy[k] = r[0];
         if (virial)
@@ -1714,7 +1766,12 @@ tmd_status tmd_batch_create(int32_t n_systems, const int64_t *n_atoms, const dou
     if (e == cudaSuccess) e = cudaMalloc(&b->d_off, sizeof(int64_t) * (n_systems + 1));
     if (e == cudaSuccess) e = cudaMalloc(&b->active, n_systems);
     if (e == cudaSuccess) e = cudaMalloc(&b->act_list, sizeof(int32_t) * n_systems);
-    if (e == cudaSuccess) e = cudaMalloc(&b->sys_out, sizeof(double) * 16 * n_systems);
+    if (e == cudaSuccess) e = cudaMalloc(&b->sys_hdr, sizeof(double) * (2 + 16 * (size_t)n_systems));
+    if (e == cudaSuccess) {
+        b->sys_out = b->sys_hdr + 2;
+        b->pool.err_ext = reinterpret_cast<int32_t *>(b->sys_hdr);
+        e = cudaMemset(b->sys_hdr, 0, sizeof(double) * 2);
+    }
     if (e == cudaSuccess) e = cudaMalloc(&b->pos_ref, sizeof(double) * 3 * n);
     if (e == cudaSuccess) e = cudaMalloc(&b->rank, sizeof(int32_t) * n);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_moved, sizeof(int32_t) * n_systems);
@@ -1723,7 +1780,7 @@ tmd_status tmd_batch_create(int32_t n_systems, const int64_t *n_atoms, const dou
     if (e == cudaSuccess) e = cudaMalloc(&b->d_overflow, sizeof(int32_t));
     if (e == cudaSuccess) e = cudaMalloc(&b->d_pbase, sizeof(int64_t) * TMD_MAX_SPECIES * n_systems);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_rflags, n_systems);
-    if (e == cudaSuccess) e = cudaMallocHost(&b->h_out, sizeof(double) * 16 * n_systems);
+    if (e == cudaSuccess) e = cudaMallocHost(&b->h_out, sizeof(double) * (2 + 16 * (size_t)n_systems));
     if (e == cudaSuccess) e = cudaMallocHost(&b->h_act, sizeof(int32_t) * n_systems);
     if (e == cudaSuccess) e = cudaMallocHost(&b->h_flags, n_systems);
     if (e == cudaSuccess) e = cudaMallocHost(&b->h_moved, sizeof(int32_t) * n_systems);
@@ -1754,7 +1811,7 @@ tmd_status tmd_batch_create(int32_t n_systems, const int64_t *n_atoms, const dou
 tmd_status tmd_batch_destroy(tmd_batch *b) {
     if (!b) return TMD_OK;
     void *p[] = {b->pos, b->vel, b->mass, b->inv_mass, b->types, b->sys_of, b->forces, b->e_atom, b->w_atom,
-                 b->d_off, b->active, b->act_list, b->sys_out, b->pos_ref, b->rank, b->d_moved, b->d_region,
+                 b->d_off, b->active, b->act_list, b->sys_hdr, b->pos_ref, b->rank, b->d_moved, b->d_region,
                  b->d_fill, b->d_overflow, b->d_pbase, b->d_rflags};
     for (void *q : p)
         if (q) cudaFree(q);
@@ -1852,8 +1909,7 @@ tmd_status tmd_batch_compute(const tmd_model *model, tmd_batch *b, const int32_t
     tmd_status st;
     if ((st = batch_activate(b, systems, n_act, s, &na)) != TMD_OK) return st;
     if ((st = batch_eval(model, b, n_act, s)) != TMD_OK) return st;
-    TMD_CUDA(cudaMemcpyAsync(b->h_out, b->sys_out, sizeof(double) * 16 * n_act, cudaMemcpyDeviceToHost, s));
-    TMD_CUDA(cudaStreamSynchronize(s));
+    if ((st = batch_read(b, n_act, s)) != TMD_OK) return st;
     for (int k = 0; k < n_act; ++k) b->has_forces[systems[k]] = 1;
     batch_results(b, n_act, energy, virial, nullptr);
     return TMD_OK;
@@ -1930,8 +1986,7 @@ tmd_status tmd_batch_step(const tmd_model *model, tmd_batch *b, const int32_t *s
         TMD_LAUNCH("k_sys_reduce", s, tmd::sys_reduce_launch(b->act_list, n_act, b->d_off, b->e_atom, b->w_atom, b->vel,
                                                              b->mass, b->sys_out, s));
     }
-    TMD_CUDA(cudaMemcpyAsync(b->h_out, b->sys_out, sizeof(double) * 16 * n_act, cudaMemcpyDeviceToHost, s));
-    TMD_CUDA(cudaStreamSynchronize(s));
+    if ((st = batch_read(b, n_act, s)) != TMD_OK) return st;
     batch_results(b, n_act, nullptr, nullptr, thermo);
     return TMD_OK;
 }

@@ -33,6 +33,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstring>
 #include <vector>
@@ -99,8 +100,8 @@ constexpr uint64_t WAIT_NS = 200000000ull;   // 0.2 s per wait
 // gives up (0.2 s, or the iteration cap) it records DEV_ERR_TIMEOUT and sets
 // the block's abort flag, after which every later wait returns at once: the
 // kernel runs on to its end, waits (bounded) for its copies and MMAs in
-// flight, frees its tensor memory and the host reports the status; the
-// results of that call are not valid.
+// flight, frees its tensor memory and marks its results as invalid
+// (net_invalid), which every entry point that waits for results reports.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int *abort) {
     if (*abort) return false;
     if (mbar_try_wait(bar, parity)) return true;
@@ -123,6 +124,20 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, uint32_t
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
                  "l"(src), "r"(bytes), "r"(bar)
                  : "memory");
+}
+// The outputs of the tiles tile0, tile0 + step, ... of a network that gave up:
+// NaN, and the evaluation's error word set (all threads of a block).
+__device__ __forceinline__ void net_invalid(const int32_t *perm, int64_t n, int Dd, float *dG, float *e_atom,
+                                            double *part_e, int tile0, int step, int ntile, int32_t *err) {
+    for (int tile = tile0; tile < ntile; tile += step) {
+        const int64_t p0 = (int64_t)tile * UM;
+        const int rows = (int)min((int64_t)UM, n - p0);
+        for (int i = threadIdx.x; i < rows * Dd; i += blockDim.x) dG[(size_t)p0 * Dd + i] = NAN;
+        if (e_atom)
+            for (int r = threadIdx.x; r < rows; r += blockDim.x) e_atom[perm[p0 + r]] = NAN;
+        if (threadIdx.x == 0) part_e[tile] = NAN;
+    }
+    if (threadIdx.x == 0) atomicOr(err, DEV_ERR_TIMEOUT);
 }
 // one lane of a converged warp, always the same: tells the compiler that one
 // thread runs what follows, whose operands then go to uniform registers at once
@@ -221,7 +236,7 @@ constexpr int MAX_CHUNKS = 64;   // weight chunks of one species block at most
 __global__ void __launch_bounds__(UTHREADS, 2)
     k_mlp_umma(const __grid_constant__ DevModel m, const __grid_constant__ UmmaNet u, const int32_t *__restrict__ perm,
                const int32_t *__restrict__ types, int64_t n, const float *__restrict__ G, float *__restrict__ dG,
-               float *__restrict__ e_atom, double *__restrict__ part_e, int ntile) {
+               float *__restrict__ e_atom, double *__restrict__ part_e, int ntile, int32_t *__restrict__ err) {
     extern __shared__ __align__(1024) unsigned char smraw[];
     // barriers: full[MAX_NST], empty[MAX_NST] (weight stages), aempty[2] (G stages), done
     __shared__ __align__(8) uint64_t s_bar[2 * MAX_NST + 3];
@@ -584,6 +599,8 @@ __global__ void __launch_bounds__(UTHREADS, 2)
             __syncwarp();
             mbar_drain(bar_done, pd & 1);
         }
+        __syncthreads();
+        net_invalid(perm, n, Dd, dG, e_atom, part_e, blockIdx.x, gridDim.x, ntile, err);
     }
     tc_fence_before();
     __syncthreads();
@@ -617,6 +634,14 @@ __global__ void __launch_bounds__(32, 1) k_wait_probe(int32_t *__restrict__ gave
     __syncthreads();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(32) : "memory");
     if (threadIdx.x == 0) *gave_up = s_abort;
+}
+
+// net_invalid by itself (the self-test of what follows a time-out)
+__global__ void __launch_bounds__(256) k_net_invalid(const int32_t *__restrict__ perm, int64_t n, int Dd,
+                                                     float *__restrict__ dG, float *__restrict__ e_atom,
+                                                     double *__restrict__ part_e, int ntile, int32_t *__restrict__ err) {
+    net_invalid(perm, n, Dd, dG, e_atom, part_e, blockIdx.x, gridDim.x, ntile, err);
+    if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&g_umma_status, DEV_ERR_TIMEOUT);
 }
 
 // launch plan for a model, or false when the shapes do not fit
@@ -726,7 +751,28 @@ double bf16_value(uint16_t b) {
 
 #include "mlp_split.cuh"
 
+std::atomic<int> g_net_timeout{0};   // tmd_selftest_network_timeout
+
+// armed: the network just enqueued on s is treated as one that gave up in its
+// last tile (not within a capture: the graph would keep it)
+tmd_status giveup_if_armed(const DevModel &dm, const int32_t *perm, int64_t n, float *dG, float *e_atom, double *part_e,
+                           int ntile, int32_t *err, cudaStream_t s) {
+    if (!g_net_timeout.load()) return TMD_OK;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        (void)cudaGetLastError();
+        return TMD_OK;
+    }
+    if (!g_net_timeout.exchange(0)) return TMD_OK;
+    const int64_t p0 = (int64_t)(ntile - 1) * UM;
+    k_net_invalid<<<1, 256, 0, s>>>(perm + p0, n - p0, dm.Dd, dG + (size_t)p0 * dm.Dd, e_atom, part_e + (ntile - 1), 1, err);
+    TMD_CUDA(cudaGetLastError());
+    return TMD_OK;
+}
+
 }  // namespace
+
+void arm_network_timeout() { g_net_timeout.store(1); }
 
 int g_network_kernel = 0;
 int network_kernel() { return g_network_kernel; }
@@ -737,7 +783,7 @@ bool mlp_umma_supported(const DevModel &dm) {
 }
 
 tmd_status mlp_umma_launch(const DevModel &dm, const int32_t *perm, const int32_t *types, int64_t n, const float *G,
-                           float *dG, float *e_atom, double *part_e, int *ntile_out, cudaStream_t s) {
+                           float *dG, float *e_atom, double *part_e, int *ntile_out, int32_t *err, cudaStream_t s) {
     UmmaNet u;
     if (!plan(dm, u)) {
         set_error("network shapes outside the tcgen05 kernel");
@@ -755,10 +801,10 @@ tmd_status mlp_umma_launch(const DevModel &dm, const int32_t *perm, const int32_
     const int grid = std::max(1, std::min(ntile, std::max(1, nsm) * u.blocks_per_sm));
     if (ntile > 0)
         TMD_LAUNCH("k_mlp_umma", s, k_mlp_umma<<<grid, UTHREADS, u.smem, s>>>(dm, u, perm, types, n, G, dG, e_atom,
-                                                                              part_e, ntile));
+                                                                              part_e, ntile, err));
     TMD_CUDA(cudaGetLastError());
     *ntile_out = ntile;
-    return TMD_OK;
+    return giveup_if_armed(dm, perm, n, dG, e_atom, part_e, ntile, err, s);
 }
 
 // BF16 weights in the operand layout of k_mlp_umma (product order: forward
@@ -832,7 +878,8 @@ bool mlp_split_ok(const DevModel &dm) {
 }
 
 tmd_status mlp_split_launch(const char *name, const DevModel &dm, const int32_t *perm, const int32_t *types, int64_t n,
-                           const float *G, float *dG, float *e_atom, double *part_e, int *ntile_out, cudaStream_t s) {
+                           const float *G, float *dG, float *e_atom, double *part_e, int *ntile_out, int32_t *err,
+                           cudaStream_t s) {
     SplitNet u;
     if (!split_plan(dm, u)) {
         set_error("network shapes outside the split-operand kernel");
@@ -846,10 +893,11 @@ tmd_status mlp_split_launch(const char *name, const DevModel &dm, const int32_t 
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     const int grid = std::max(1, std::min(ntile, std::max(1, nsm) * u.blocks_per_sm));
-    TMD_LAUNCH(name, s, k_mlp_split<<<grid, UTHREADS, u.smem, s>>>(dm, u, perm, types, n, G, dG, e_atom, part_e, ntile));
+    TMD_LAUNCH(name, s, k_mlp_split<<<grid, UTHREADS, u.smem, s>>>(dm, u, perm, types, n, G, dG, e_atom, part_e, ntile,
+                                                                  err));
     TMD_CUDA(cudaGetLastError());
     *ntile_out = ntile;
-    return TMD_OK;
+    return giveup_if_armed(dm, perm, n, dG, e_atom, part_e, ntile, err, s);
 }
 
 // FP32 weights split into three BF16 planes in the operand layout of k_mlp_split

@@ -535,6 +535,7 @@ __global__ void __launch_bounds__(PW * 32, desc_min_blocks(S, K)) k_desc(DevMode
         const float4 a = __ldg(m.radial + i);
         return make_float4(-a.x, -a.y, -a.z, 0.f);
     };
+    if (nl.err_clear && blockIdx.x == 0 && threadIdx.x == 0) *nl.err_clear = 0;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, t = lane & 3;   // operand row (channel) / column (pairs 2t, 2t + 1)
     const unsigned lt = (1u << lane) - 1u;

@@ -738,20 +738,22 @@ __global__ void __cluster_dims__(RED_CL, 1, 1) __launch_bounds__(256)
     }
 }
 
-__global__ void k_forces_out(const long long *__restrict__ Fq, int64_t n, float *__restrict__ forces) {
+// (NaN where the evaluation is invalid: the fixed-point sums cannot hold it)
+__global__ void k_forces_out(const long long *__restrict__ Fq, int64_t n, const int32_t *__restrict__ err,
+                             float *__restrict__ forces) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < 3 * n) forces[i] = (float)((double)Fq[i] * FQ_INV);
+    if (i < 3 * n) forces[i] = *err ? NAN : (float)((double)Fq[i] * FQ_INV);
 }
 
 // forces of the atoms listed in perm (batched: only the active systems' atoms)
 __global__ void k_forces_out_perm(const long long *__restrict__ Fq, const int32_t *__restrict__ perm, int64_t n,
-                                  float *__restrict__ forces) {
+                                  const int32_t *__restrict__ err, float *__restrict__ forces) {
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= n) return;
     const int64_t a = perm[p];
-    forces[3 * a] = (float)((double)Fq[3 * a] * FQ_INV);
-    forces[3 * a + 1] = (float)((double)Fq[3 * a + 1] * FQ_INV);
-    forces[3 * a + 2] = (float)((double)Fq[3 * a + 2] * FQ_INV);
+    const bool bad = *err != 0;
+#pragma unroll
+    for (int x = 0; x < 3; ++x) forces[3 * a + x] = bad ? NAN : (float)((double)Fq[3 * a + x] * FQ_INV);
 }
 
 // Per-system FP64 sums over each active system's atom range (one cluster per
@@ -952,10 +954,10 @@ static tmd_status set_mlp_smem(const DevModel &dm, bool bf16) {
 
 static tmd_status launch_network(const DevModel &dm, const int32_t *perm, const int32_t *types, int64_t n,
                                  const float *G, float *dG, float *e_atom, double *part_e, int *ntile_out,
-                                 cudaStream_t s) {
+                                 int32_t *err, cudaStream_t s) {
     tmd_status st;
     if (dm.precision == TMD_PREC_BF16 && network_kernel() != 2 && mlp_umma_supported(dm))
-        return mlp_umma_launch(dm, perm, types, n, G, dG, e_atom, part_e, ntile_out, s);
+        return mlp_umma_launch(dm, perm, types, n, G, dG, e_atom, part_e, ntile_out, err, s);
     if (dm.precision == TMD_PREC_BF16 && network_kernel() == 1) {
         set_error("the tcgen05 network kernel does not support these network shapes");
         return TMD_ERR_UNIMPLEMENTED;
@@ -971,7 +973,7 @@ static tmd_status launch_network(const DevModel &dm, const int32_t *perm, const 
     // 128 stands for 128-atom tiles, else "k_mlp".
     if (mlp_split_ok(dm))
         return mlp_split_launch(mlp_all64(dm) && (dm.tile_rows == 0 || dm.tile_rows == 128) ? "k_mlp_res" : "k_mlp", dm,
-                               perm, types, n, G, dG, e_atom, part_e, ntile_out, s);
+                               perm, types, n, G, dG, e_atom, part_e, ntile_out, err, s);
     if ((st = set_mlp_smem(dm, dm.precision == TMD_PREC_BF16)) != TMD_OK) return st;
     if (dm.precision == TMD_PREC_BF16) {
         const int ntile = (int)((n + BT - 1) / BT);
@@ -993,6 +995,9 @@ static tmd_status launch_network(const DevModel &dm, const int32_t *perm, const 
     TMD_CUDA(cudaGetLastError());
     return TMD_OK;
 }
+
+// the word in which an evaluation on this table records that it is invalid
+static tmd_status err_word(tmd_nlist *nl) { return nl->err_ext ? TMD_OK : grow(&nl->err, &nl->cap_err, 1); }
 
 static tmd_status split_positions(tmd_nlist *nl, const double *pos, int64_t n, cudaStream_t s) {
     tmd_status st;
@@ -1024,6 +1029,7 @@ tmd_status reserve_compute(const DevModel &dm, tmd_nlist *nl, int64_t n_total, i
     if ((st = grow(&nl->Fq, &nl->cap_Fq, 3 * nt)) != TMD_OK) return st;
     if ((st = grow(&nl->ph, &nl->cap_ph, nt)) != TMD_OK) return st;
     if ((st = grow(&nl->pl, &nl->cap_pl, nt)) != TMD_OK) return st;
+    if ((st = err_word(nl)) != TMD_OK) return st;
     const int64_t nblk = pair_blocks(dm, na), ntile = (na + MT - 1) / MT;
     if ((st = grow(&nl->part, &nl->cap_part, ntile + 9 * nblk + 16)) != TMD_OK) return st;
     return pair_cache(nl, nt, nullptr);
@@ -1031,6 +1037,8 @@ tmd_status reserve_compute(const DevModel &dm, tmd_nlist *nl, int64_t n_total, i
 
 static DevNlist dev_nlist(const tmd_nlist *nl, int64_t n, const double box[3]) {
     DevNlist dn;
+    dn.err = nl->err_ext ? nl->err_ext : nl->err;
+    dn.err_clear = nl->err_ext ? nullptr : nl->err;
     dn.beg = nl->beg;
     dn.end = nl->end;
     dn.nbr = nl->nbr;
@@ -1057,6 +1065,7 @@ tmd_status run_descriptors(const tmd_model *model, tmd_nlist *nl, const double *
     if (dEdG && (st = grow(&nl->dG, &nl->cap_dG, n * dm.Dd)) != TMD_OK) return st;
     const int nblk = pair_blocks(dm, n);
     if ((st = split_positions(nl, pos, n, s)) != TMD_OK) return st;
+    if ((st = err_word(nl)) != TMD_OK) return st;
     const DevNlist dn = dev_nlist(nl, n, box);
     if ((st = dispatch_pair(dm, dn, pos, types, nl, nullptr, nblk, s, true)) != TMD_OK) return st;
     // the workspaces hold rows in perm order; the caller's arrays are per atom
@@ -1067,7 +1076,7 @@ tmd_status run_descriptors(const tmd_model *model, tmd_nlist *nl, const double *
     const int ntile = (int)((n + MT - 1) / MT);
     if ((st = grow(&nl->part, &nl->cap_part, ntile + 16)) != TMD_OK) return st;
     int nt = 0;
-    if ((st = launch_network(dm, nl->perm, types, n, nl->G, nl->dG, nullptr, nl->part, &nt, s)) != TMD_OK) return st;
+    if ((st = launch_network(dm, nl->perm, types, n, nl->G, nl->dG, nullptr, nl->part, &nt, dn.err, s)) != TMD_OK) return st;
     TMD_LAUNCH("k_rows_to_atoms", s, k_rows_to_atoms<<<gb, 256, 0, s>>>(nl->dG, nl->perm, n, dm.Dd, dEdG));
     TMD_CUDA(cudaGetLastError());
     return TMD_OK;
@@ -1099,6 +1108,7 @@ tmd_status run_compute(const tmd_model *model, tmd_nlist *nl, const double *pos,
     if (!(pos_split && nl->cap_ph >= n && nl->cap_pl >= n))
         if ((st = split_positions(nl, pos, n, s)) != TMD_OK) return st;
     if ((st = pair_cache(nl, n, s)) != TMD_OK) return st;
+    if ((st = err_word(nl)) != TMD_OK) return st;
     DevNlist dn = dev_nlist(nl, n, box);
     dn.pq = nl->pq;
     dn.pq2 = nl->pq2;
@@ -1107,13 +1117,13 @@ tmd_status run_compute(const tmd_model *model, tmd_nlist *nl, const double *pos,
     TMD_CUDA(cudaMemsetAsync(nl->Fq, 0, sizeof(long long) * 3 * n, s));
     if ((st = dispatch_pair(dm, dn, pos, types, nl, part_w, nblk, s, true)) != TMD_OK) return st;
     int ne = 0;
-    if ((st = launch_network(dm, nl->perm, types, n, nl->G, nl->dG, e_atom, part_e, &ne, s)) != TMD_OK) return st;
+    if ((st = launch_network(dm, nl->perm, types, n, nl->G, nl->dG, e_atom, part_e, &ne, dn.err, s)) != TMD_OK) return st;
     if ((st = dispatch_pair(dm, dn, pos, types, nl, part_w, nblk, s, false)) != TMD_OK) return st;
     TMD_LAUNCH("k_reduce", s, k_reduce<<<RED_CL, 256, 0, s>>>(part_e, ne, part_w, nblk, energy, virial));
     TMD_CUDA(cudaGetLastError());
     if (forces) {
         TMD_LAUNCH("k_forces_out", s, k_forces_out<<<(unsigned)((3 * n + 255) / 256), 256, 0, s>>>(
-                                           reinterpret_cast<const long long *>(nl->Fq), n, forces));
+                                           reinterpret_cast<const long long *>(nl->Fq), n, dn.err, forces));
         TMD_CUDA(cudaGetLastError());
     }
     return TMD_OK;
@@ -1191,14 +1201,14 @@ tmd_status run_compute_owned(const tmd_model *model, tmd_nlist *nl, const double
     TMD_CUDA(cudaMemsetAsync(nl->Fq, 0, sizeof(long long) * 3 * n, s));
     if ((st = dispatch_pair(dm, dn, pos, types, nl, part_w, nblk, s, true)) != TMD_OK) return st;
     int ne = 0;
-    if ((st = launch_network(dm, nl->perm_own, types, n_owned, nl->G, nl->dG, e_atom, part_e, &ne, s)) != TMD_OK)
+    if ((st = launch_network(dm, nl->perm_own, types, n_owned, nl->G, nl->dG, e_atom, part_e, &ne, dn.err, s)) != TMD_OK)
         return st;
     if ((st = dispatch_pair(dm, dn, pos, types, nl, part_w, nblk, s, false)) != TMD_OK) return st;
     TMD_LAUNCH("k_reduce", s, k_reduce<<<RED_CL, 256, 0, s>>>(part_e, ne, part_w, nblk, energy, virial));
     TMD_CUDA(cudaGetLastError());
     if (forces) {
         TMD_LAUNCH("k_forces_out", s, k_forces_out<<<(unsigned)((3 * n + 255) / 256), 256, 0, s>>>(
-                                           reinterpret_cast<const long long *>(nl->Fq), n, forces));
+                                           reinterpret_cast<const long long *>(nl->Fq), n, dn.err, forces));
         TMD_CUDA(cudaGetLastError());
     }
     return TMD_OK;
@@ -1351,7 +1361,7 @@ tmd_status run_compute_noalloc(const tmd_model *model, const int64_t *off, const
     int32_t *flag = static_cast<int32_t *>(take(sizeof(int32_t) * 4));
 
     // validate the caller's table on the device, then read the result
-    TMD_CUDA(cudaMemsetAsync(flag, 0, sizeof(int32_t), s));
+    TMD_CUDA(cudaMemsetAsync(flag, 0, 2 * sizeof(int32_t), s));   // the check's, the evaluation's
     const int cb = (int)std::min<int64_t>((std::max(n, nnz) + 255) / 256, 4096);
     TMD_LAUNCH("k_noalloc_check", s, k_noalloc_check<<<cb, 256, 0, s>>>(off, nbr, reinterpret_cast<const char4 *>(shift4),
                                                                         types, n, nnz, dm.S, box[0], box[1], box[2],
@@ -1376,6 +1386,7 @@ tmd_status run_compute_noalloc(const tmd_model *model, const int64_t *off, const
     dn.nbr = nbr;
     dn.shift = reinterpret_cast<const char4 *>(shift4);
     dn.perm = w.perm;
+    dn.err = flag + 1;
     dn.ph = w.ph;
     dn.pl = w.pl;
     dn.n = n;
@@ -1390,13 +1401,13 @@ tmd_status run_compute_noalloc(const tmd_model *model, const int64_t *off, const
     TMD_CUDA(cudaMemsetAsync(w.Fq, 0, sizeof(unsigned long long) * 3 * n, s));
     if ((st = dispatch_pair(dm, dn, pos, types, &w, part_w, nblk, s, true)) != TMD_OK) return st;
     int ne = 0;
-    if ((st = launch_network(dm, w.perm, types, n, w.G, w.dG, e_atom, part_e, &ne, s)) != TMD_OK) return st;
+    if ((st = launch_network(dm, w.perm, types, n, w.G, w.dG, e_atom, part_e, &ne, dn.err, s)) != TMD_OK) return st;
     if ((st = dispatch_pair(dm, dn, pos, types, &w, part_w, nblk, s, false)) != TMD_OK) return st;
     TMD_LAUNCH("k_reduce", s, k_reduce<<<RED_CL, 256, 0, s>>>(part_e, ne, part_w, nblk, energy, virial));
     TMD_CUDA(cudaGetLastError());
     if (forces) {
         TMD_LAUNCH("k_forces_out", s, k_forces_out<<<(unsigned)((3 * n + 255) / 256), 256, 0, s>>>(
-                                           reinterpret_cast<const long long *>(w.Fq), n, forces));
+                                           reinterpret_cast<const long long *>(w.Fq), n, dn.err, forces));
         TMD_CUDA(cudaGetLastError());
     }
     return TMD_OK;
@@ -1438,6 +1449,7 @@ tmd_status run_compute_batch(const tmd_model *model, tmd_nlist *nl, const double
         if ((st = grow(&nl->part, &nl->cap_part, ntile + 9 * (int64_t)nblk + 16)) != TMD_OK) return st;
         if ((st = split_positions(nl, pos, n_total, s)) != TMD_OK) return st;
         if ((st = pair_cache(nl, n_total, s)) != TMD_OK) return st;
+        if ((st = err_word(nl)) != TMD_OK) return st;
         DevNlist dn = dev_nlist(nl, na, nl->box);
         dn.sp = nl->sp;
         dn.sys_of = sys_of;
@@ -1447,12 +1459,12 @@ tmd_status run_compute_batch(const tmd_model *model, tmd_nlist *nl, const double
         TMD_CUDA(cudaMemsetAsync(nl->Fq, 0, sizeof(long long) * 3 * n_total, s));
         if ((st = dispatch_pair(dm, dn, pos, types, nl, nullptr, nblk, s, true)) != TMD_OK) return st;
         int ne = 0;
-        if ((st = launch_network(dm, nl->perm, types, na, nl->G, nl->dG, e_atom, nl->part, &ne, s)) != TMD_OK)
+        if ((st = launch_network(dm, nl->perm, types, na, nl->G, nl->dG, e_atom, nl->part, &ne, dn.err, s)) != TMD_OK)
             return st;
         if ((st = dispatch_pair(dm, dn, pos, types, nl, nl->part + ntile, nblk, s, false, w_atom)) != TMD_OK)
             return st;
         TMD_LAUNCH("k_forces_out_perm", s, k_forces_out_perm<<<(unsigned)((na + 255) / 256), 256, 0, s>>>(
-                                               reinterpret_cast<const long long *>(nl->Fq), nl->perm, na, forces));
+                                               reinterpret_cast<const long long *>(nl->Fq), nl->perm, na, dn.err, forces));
         TMD_CUDA(cudaGetLastError());
     }
     if (n_act > 0 && sys_out) {

@@ -74,11 +74,12 @@ size_t mlp_bf16_smem_bytes(const DevModel &dm);
 // tcgen05 form of the BF16 network (mlp_umma.cu)
 bool mlp_umma_supported(const DevModel &dm);
 tmd_status mlp_umma_launch(const DevModel &dm, const int32_t *perm, const int32_t *types, int64_t n, const float *G,
-                           float *dG, float *e_atom, double *part_e, int *ntile_out, cudaStream_t s);
+                           float *dG, float *e_atom, double *part_e, int *ntile_out, int32_t *err, cudaStream_t s);
 // tcgen05 form of the FP32 network on split operands (mlp_split.cuh)
 bool mlp_split_ok(const DevModel &dm);
 tmd_status mlp_split_launch(const char *name, const DevModel &dm, const int32_t *perm, const int32_t *types, int64_t n,
-                           const float *G, float *dG, float *e_atom, double *part_e, int *ntile_out, cudaStream_t s);
+                           const float *G, float *dG, float *e_atom, double *part_e, int *ntile_out, int32_t *err,
+                           cudaStream_t s);
 // network kernel of the BF16 form: 0 = tcgen05 when the shapes allow it, else
 // mma.sync; 1 = tcgen05 only; 2 = mma.sync only
 int network_kernel();
@@ -130,6 +131,12 @@ struct DevNlist {
     float4 *pq = nullptr;
     float2 *pq2 = nullptr;
     int32_t *npair = nullptr;
+    // DEV_ERR_TIMEOUT when a bounded wait of the network kernel gave up in this
+    // evaluation (forces are then NaN, as are the energies and virials through
+    // the network's outputs); err_clear: the same word where the evaluation
+    // starts by clearing it (the descriptor pass), or nullptr
+    int32_t *err = nullptr;
+    int32_t *err_clear = nullptr;
 };
 
 }  // namespace tmd
@@ -195,6 +202,8 @@ struct tmd_nlist {
     int32_t *npair = nullptr; int64_t cap_npair = 0; // [n] in-cutoff pairs per atom
     int32_t *perm_own = nullptr; int64_t cap_perm_own = 0; // [n_owned] evaluation order of owned centres
     int32_t *own_count = nullptr; int64_t cap_own_count = 0; // [MAX_SPECIES] owned atoms per species
+    int32_t *err = nullptr;   int64_t cap_err = 0;  // [1] DevNlist::err of a table of its own
+    int32_t *err_ext = nullptr;   // the owner's word instead (System, Batch): set here, cleared by the owner
 
     // staging for the host-buffer entry point
     double *io_pos = nullptr;   int64_t cap_io_pos = 0;
@@ -228,7 +237,9 @@ struct tmd_system {
     double *pos = nullptr, *vel = nullptr, *pos_ref = nullptr, *inv_mass = nullptr, *mass = nullptr;
     int32_t *types = nullptr;
     float *forces = nullptr;
-    double *red = nullptr;       // [32] device reduction outputs (E, W, KE, max disp)
+    // [32] device reduction outputs: 0-9 E and W, 10-15 kinetic; then 20 the skin
+    // flag of a step, 21 the time-out word (nl.err_ext), 24-31 the skin flags of a run
+    double *red = nullptr;
     double *part = nullptr;      int64_t cap_part = 0;
     double *h_red = nullptr;     // host pinned mirror of red
     tmd_nlist nl;
@@ -236,11 +247,10 @@ struct tmd_system {
     int need_rebuild = 1, have_forces = 0;
     tmd::GraphCache g_step;      // force evaluation + second half kick
     // runs of steps as one launch sequence (tmd_step): state at the start of
-    // the run (for an exact rerun), skin-check flag of each step, host mirror
+    // the run (for an exact rerun), host mirror of its flags
     double *snap_pos = nullptr, *snap_vel = nullptr;
     float *snap_forces = nullptr;
-    int32_t *run_flags = nullptr;
-    int64_t *h_run = nullptr;    // pinned: flags, entry counter, status
+    int64_t *h_run = nullptr;    // pinned: red[21..31], entry counter, status
     tmd::GraphCache g_run;
     int64_t runs = 0, reruns = 0;
     int near_skin = 0;           // an atom moved more than 0.7 skin/2 since the last build
@@ -348,6 +358,7 @@ tmd_status mlp_umma_build(tmd_model *m, const double *const *weights);
 tmd_status mlp_split_build(tmd_model *m, const double *const *weights);
 tmd_status umma_status(int32_t *bits);
 tmd_status wait_probe(int32_t *gave_up);
+void arm_network_timeout();   // tmd_selftest_network_timeout
 extern int g_network_kernel;
 // pos_split: the table's split positions (nl->ph, nl->pl) already hold pos
 // (the MD step writes them in its drift); otherwise they are formed here

@@ -72,6 +72,7 @@ _SIGS = {
     "tmd_set_force_kernel": (C.c_int, [C.c_int32]),
     "tmd_device_status": (C.c_int, [C.POINTER(C.c_int32)]),
     "tmd_selftest_bounded_wait": (C.c_int, [C.POINTER(C.c_int32)]),
+    "tmd_selftest_network_timeout": (C.c_int, []),
     "tmd_model_get_tuning": (C.c_int, [_P, C.POINTER(Tuning)]),
     "tmd_autotune": (C.c_int, [_P, _P, _P, _P, C.c_int64, C.POINTER(C.c_double), C.POINTER(Tuning), _P]),
     "tmd_batch_autotune": (C.c_int, [_P, _P, _P, C.c_int32, C.POINTER(Tuning), _P]),
@@ -166,6 +167,11 @@ def selftest_bounded_wait():
     g = C.c_int32(0)
     check(lib().tmd_selftest_bounded_wait(C.byref(g)))
     return g.value == 1
+
+
+def selftest_network_timeout():
+    """Treat the next tensor-core network launched (outside a capture) as one that gave up waiting."""
+    check(lib().tmd_selftest_network_timeout())
 
 
 def set_graphs(on=True):
