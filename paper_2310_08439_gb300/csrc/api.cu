@@ -204,9 +204,10 @@ __global__ void k_vv_second_fq(double *__restrict__ vel, const long long *__rest
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const double h = 0.5 * dt * inv_mass[i] * ACC_CONV;
+    const float bad = *err ? NAN : 0.f;   // (as k_forces_out)
 #pragma unroll
     for (int x = 0; x < 3; ++x) {
-        const float f = *err ? NAN : (float)((double)Fq[3 * i + x] * FQ_UNIT);   // (as k_forces_out)
+        const float f = (float)((double)Fq[3 * i + x] * FQ_UNIT) + bad;
         F[3 * i + x] = f;
         vel[3 * i + x] += h * (double)f;
     }

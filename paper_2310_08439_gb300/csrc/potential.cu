@@ -742,7 +742,7 @@ __global__ void __cluster_dims__(RED_CL, 1, 1) __launch_bounds__(256)
 __global__ void k_forces_out(const long long *__restrict__ Fq, int64_t n, const int32_t *__restrict__ err,
                              float *__restrict__ forces) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < 3 * n) forces[i] = *err ? NAN : (float)((double)Fq[i] * FQ_INV);
+    if (i < 3 * n) forces[i] = (float)((double)Fq[i] * FQ_INV) + (*err ? NAN : 0.f);
 }
 
 // forces of the atoms listed in perm (batched: only the active systems' atoms)
@@ -751,9 +751,9 @@ __global__ void k_forces_out_perm(const long long *__restrict__ Fq, const int32_
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= n) return;
     const int64_t a = perm[p];
-    const bool bad = *err != 0;
+    const float bad = *err ? NAN : 0.f;
 #pragma unroll
-    for (int x = 0; x < 3; ++x) forces[3 * a + x] = bad ? NAN : (float)((double)Fq[3 * a + x] * FQ_INV);
+    for (int x = 0; x < 3; ++x) forces[3 * a + x] = (float)((double)Fq[3 * a + x] * FQ_INV) + bad;
 }
 
 // Per-system FP64 sums over each active system's atom range (one cluster per
