@@ -789,11 +789,7 @@ tmd_status mlp_umma_launch(const DevModel &dm, const int32_t *perm, const int32_
         set_error("network shapes outside the tcgen05 kernel");
         return TMD_ERR_UNIMPLEMENTED;
     }
-    static int smem_set = 0;
-    if (u.smem > 48 * 1024 && u.smem > smem_set) {
-        TMD_CUDA(cudaFuncSetAttribute(k_mlp_umma, cudaFuncAttributeMaxDynamicSharedMemorySize, u.smem));
-        smem_set = u.smem;
-    }
+    TMD_CUDA(smem_opt_in<k_mlp_umma>(u.smem));
     const int ntile = (int)((n + UM - 1) / UM);
     int dev = 0, nsm = 0;
     cudaGetDevice(&dev);
@@ -885,9 +881,7 @@ tmd_status mlp_split_launch(const char *name, const DevModel &dm, const int32_t 
         set_error("network shapes outside the split-operand kernel");
         return TMD_ERR_UNIMPLEMENTED;
     }
-    static const cudaError_t set =
-        cudaFuncSetAttribute(k_mlp_split, cudaFuncAttributeMaxDynamicSharedMemorySize, SN_SMEM_MAX);
-    TMD_CUDA(set);
+    TMD_CUDA(smem_opt_in<k_mlp_split>(u.smem));
     const int ntile = (int)((n + UM - 1) / UM);
     int dev = 0, nsm = 0;
     cudaGetDevice(&dev);

@@ -926,28 +926,17 @@ static tmd_status validate(const tmd_model *model, tmd_nlist *nl, int64_t n, con
 // opt-in shared memory of the network kernel that runs: the FP32 k_mlp<TR>,
 // or (bf16 = true) the mma.sync kernel of the BF16 form
 static tmd_status set_mlp_smem(const DevModel &dm, bool bf16) {
-    static size_t smem_set[2] = {0, 0}, smem_bf_set = 0;
     if (bf16) {
         const size_t sb = mlp_bf16_smem_bytes(dm);
         if (sb > 227 * 1024) {
             set_error("network too wide for the mma.sync BF16 kernel (%zu bytes of shared memory)", sb);
             return TMD_ERR_UNIMPLEMENTED;
         }
-        if (sb > 48 * 1024 && sb > smem_bf_set) {
-            TMD_CUDA(cudaFuncSetAttribute(k_mlp_bf16, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sb));
-            smem_bf_set = sb;
-        }
-        return TMD_OK;
-    }
-    const int tr = mlp_tr(dm);
-    const size_t smem = mlp_smem_bytes(dm);
-    size_t &done = smem_set[tr == 64 ? 1 : 0];
-    if (smem > 48 * 1024 && smem > done) {
-        if (tr == 64)
-            TMD_CUDA(cudaFuncSetAttribute(k_mlp<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        else
-            TMD_CUDA(cudaFuncSetAttribute(k_mlp<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        done = smem;
+        TMD_CUDA(smem_opt_in<k_mlp_bf16>(sb));
+    } else if (mlp_tr(dm) == 64) {
+        TMD_CUDA(smem_opt_in<k_mlp<64>>(mlp_smem_bytes(dm)));
+    } else {
+        TMD_CUDA(smem_opt_in<k_mlp<32>>(mlp_smem_bytes(dm)));
     }
     return TMD_OK;
 }

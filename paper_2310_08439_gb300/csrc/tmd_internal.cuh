@@ -3,6 +3,8 @@
 
 #include <cuda_runtime.h>
 
+#include <atomic>
+#include <mutex>
 #include <vector>
 #include <cstdint>
 #include <cstdio>
@@ -310,6 +312,25 @@ tmd_status grow(T **ptr, int64_t *cap, int64_t need) {
     }
     *cap = n;
     return TMD_OK;
+}
+
+// Dynamic shared memory of a kernel above what it may have without asking: the
+// opt-in, once per device and size.  (Its static arrays count against the 48 KB
+// that need none: asked for from 32 KB on.)
+template <auto KERNEL>
+cudaError_t smem_opt_in(size_t bytes) {
+    constexpr int DEVICES = 64;
+    static std::atomic<size_t> granted[DEVICES];   // by device
+    static std::mutex mu;
+    if (bytes <= 32 * 1024) return cudaSuccess;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess || (dev < DEVICES && bytes <= granted[dev].load())) return e;
+    std::lock_guard<std::mutex> lk(mu);   // (a smaller size set later would take back a larger one)
+    if (dev < DEVICES && bytes <= granted[dev].load()) return cudaSuccess;
+    e = cudaFuncSetAttribute(KERNEL, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess && dev < DEVICES) granted[dev].store(bytes);
+    return e;
 }
 
 void nlist_free(tmd_nlist *nl);
