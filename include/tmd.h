@@ -251,14 +251,17 @@ int64_t tmd_graph_replays(void);
 /*
  * Tile shapes of this implementation's kernels (the paper has no counterpart:
  * they are launch choices of the GPU path).  The results are the same up to
- * the order of FP64 partial sums.
+ * the order of FP64 partial sums, but for tile_rows on networks whose descriptor
+ * length and hidden widths are all 64 (one or two hidden layers), where it
+ * chooses between two kernels that agree to FP32 rounding.
  *  tile_rows           atoms per tile of the FP32 network kernel on the FP32
- *                      pipes: 32 or 64; 128 (networks whose descriptor length
- *                      and hidden widths are all 64, one or two hidden layers)
- *                      and 0 = built-in choice.  Networks that run on the
- *                      tensor cores (hidden widths multiples of 16 up to 128,
- *                      activations of a tile within an SM's shared memory)
- *                      have 128-atom tiles with each of them;
+ *                      pipes: 32 or 64; 128: tiles of the tensor-core kernel
+ *                      (all widths 64); 0 = built-in choice: the tensor-core
+ *                      kernel where it runs (hidden widths multiples of 16 up
+ *                      to 128, activations of a tile within an SM's shared
+ *                      memory), whose tiles have 128 atoms, else 32.  Networks
+ *                      of other widths than 64 that run on the tensor cores do
+ *                      so with every tile_rows;
  *  pair_blocks_per_sm  blocks per SM of the persistent descriptor / force
  *                      grids (0 = built-in 16);
  *  ms                  output of the tuners: measured milliseconds of one

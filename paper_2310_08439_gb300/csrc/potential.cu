@@ -958,11 +958,13 @@ static tmd_status launch_network(const DevModel &dm, const int32_t *perm, const 
     // us against 461, 32,000 x 640-64-64 148 us against 342; and the errors of
     // forces and dE/dG are smaller (0.93 and 0.80 times over 113 and 23 random models
     // of more than 192 columns).
-    // Two labels, as tile_rows has two kinds of tile: "k_mlp_res" where 0 or
-    // 128 stands for 128-atom tiles, else "k_mlp".
-    if (mlp_split_ok(dm))
-        return mlp_split_launch(mlp_all64(dm) && (dm.tile_rows == 0 || dm.tile_rows == 128) ? "k_mlp_res" : "k_mlp", dm,
-                               perm, types, n, G, dG, e_atom, part_e, ntile_out, err, s);
+    // Where tile_rows has always chosen between two kernels (all widths 64), 32 and
+    // 64 are k_mlp's tiles; on other networks tile_rows changes no result.  The
+    // profile's "k_mlp_res" (all widths 64) and "k_mlp" (others) are the network
+    // stage, whose kernel here is k_mlp_split.
+    const bool all64 = mlp_all64(dm);
+    if (mlp_split_ok(dm) && !(all64 && (dm.tile_rows == 32 || dm.tile_rows == 64)))
+        return mlp_split_launch(all64 ? "k_mlp_res" : "k_mlp", dm, perm, types, n, G, dG, e_atom, part_e, ntile_out, err, s);
     if ((st = set_mlp_smem(dm, dm.precision == TMD_PREC_BF16)) != TMD_OK) return st;
     if (dm.precision == TMD_PREC_BF16) {
         const int ntile = (int)((n + BT - 1) / BT);

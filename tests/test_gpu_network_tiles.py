@@ -1,7 +1,9 @@
 """The FP32 network on the FP32 pipes (k_mlp, tiles of 32 and 64 atoms) against
 the FP64 oracle, on networks that run there: hidden widths that are no multiples
-of 16 or above 128.  The two tiles sum the products in one order and give the
-same bits."""
+of 16 or above 128, and all widths 64 with tile_rows 32 or 64.  The two tiles sum
+the products in one order and give the same bits; where tile_rows selects the
+kernel (all widths 64), the tensor cores' result is another one within FP32
+rounding."""
 import numpy as np
 import pytest
 
@@ -14,6 +16,8 @@ NETS = {   # species, K, hidden widths, activation, runs on the tensor cores by 
     "w36_20": (2, 8, [36, 20], "tanh", False),
     "w160": (1, 16, [160], "squareplus", False),
     "dd256_w60": (1, 64, [60], "tanh", False),
+    "all64": (1, 16, [64, 64], "tanh", True),
+    "all64_2sp": (2, 8, [64], "squareplus", True),
 }
 
 
