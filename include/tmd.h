@@ -262,8 +262,8 @@ int64_t tmd_graph_replays(void);
  *                      memory), whose tiles have 128 atoms, else 32.  Networks
  *                      of other widths than 64 that run on the tensor cores do
  *                      so with every tile_rows;
- *  pair_blocks_per_sm  blocks per SM of the persistent descriptor / force
- *                      grids (0 = built-in 16);
+ *  pair_blocks_per_sm  blocks per SM of the persistent force grid (0 = built-in
+ *                      16); the descriptor pass sizes its grid by itself;
  *  ms                  output of the tuners: measured milliseconds of one
  *                      evaluation with these shapes (ignored on input).
  */

@@ -1521,17 +1521,17 @@ __global__ void __launch_bounds__(PW * 32, 4) k_force(DevModel m, DevNlist nl, c
     }
 }
 
-// Blocks of the descriptor pass (or the caller's tuning): what the GPU holds at
-// once, and more once every warp would run over 512 channels (atoms x S x K),
-// so that blocks that finish early are replaced (1M atoms, K = 16: 1.12 ms with
-// the resident 7 blocks per SM, 1.04 with 4 times, 1.02 with 8 times and 1.05
-// with 64 times as many; 39,366 atoms, K = 128: 0.51 ms with the resident
-// blocks, 0.34 with 4 atoms per warp; 16,384 atoms, K = 16: 0.041 ms with the
-// resident blocks, 0.045 with 8 times as many).
+// Blocks of the descriptor pass: what the GPU holds at once, and more once every
+// warp would run over 512 channels (atoms x S x K), so that blocks that finish early
+// are replaced (1M atoms, K = 16, when the pass took 1.02 ms: 1.12 ms with the
+// resident 7 blocks per SM, 1.04 with 4 times, 1.02 with 8 times and 1.05 with 64
+// times as many; 39,366 atoms, K = 128: 0.51 ms with the resident blocks, 0.34 with 4
+// atoms per warp; 16,384 atoms, K = 16: 0.041 ms with the resident blocks, 0.045 with
+// 8 times as many).  In tuned models, too: their pair_bps, 4 to 32 blocks per SM, is
+// the force pass's (here 4 to 16 took 1.27 to 1.49 ms at 1M atoms instead of 1.20).
 constexpr int CHANNELS_PER_WARP = 512;
 template <auto KERNEL>
-int desc_blocks(const DevModel &dm, int64_t n, int nblk) {
-    if (dm.pair_bps > 0) return nblk;
+int desc_blocks(const DevModel &dm, int64_t n) {
     static const int resident = [] {
         int dev = 0, nsm = 0, per_sm = 0;
         cudaGetDevice(&dev);
@@ -1545,8 +1545,8 @@ int desc_blocks(const DevModel &dm, int64_t n, int nblk) {
 
 template <int K, int S, bool TAB, bool CACHED>
 void launch_desc(const DevModel &dm, const DevNlist &dn, const double *pos, const int32_t *types, tmd_nlist *nl,
-                 int nblk, cudaStream_t s) {
-    const int nb = desc_blocks<k_desc<K, S, TAB, CACHED>>(dm, dn.n, nblk);
+                 cudaStream_t s) {
+    const int nb = desc_blocks<k_desc<K, S, TAB, CACHED>>(dm, dn.n);
     TMD_LAUNCH("k_desc", s, k_desc<K, S, TAB, CACHED><<<nb, PW * 32, 0, s>>>(dm, dn, pos, types, nl->G, nl->P));
 }
 
@@ -1564,12 +1564,12 @@ tmd_status launch_pair_kernels(const DevModel &dm, const DevNlist &dn, const dou
     if (forward && dn.pq) {   // screen into the pair cache, then stream it
         const tmd_status st = launch_screen(dm, dn, s);
         if (st != TMD_OK) return st;
-        if (dm.rtab) launch_desc<K, S, true, true>(dm, dn, pos, types, nl, nblk, s);
-        else launch_desc<K, S, false, true>(dm, dn, pos, types, nl, nblk, s);
+        if (dm.rtab) launch_desc<K, S, true, true>(dm, dn, pos, types, nl, s);
+        else launch_desc<K, S, false, true>(dm, dn, pos, types, nl, s);
     } else if (forward && dm.rtab)
-        launch_desc<K, S, true, false>(dm, dn, pos, types, nl, nblk, s);
+        launch_desc<K, S, true, false>(dm, dn, pos, types, nl, s);
     else if (forward)
-        launch_desc<K, S, false, false>(dm, dn, pos, types, nl, nblk, s);
+        launch_desc<K, S, false, false>(dm, dn, pos, types, nl, s);
     else if (w_atom && dm.rtab)   // batched evaluations always run with the pair cache
         launch_force<K, S, true, true, true>(dm, dn, pos, types, nl, part_w, nblk, s, w_atom);
     else if (w_atom)
