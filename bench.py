@@ -97,7 +97,7 @@ class ClockSampler:
             os.makedirs(os.path.dirname(self.path), exist_ok=True)
             self.f = open(self.path, "w")
             self.proc = subprocess.Popen(["nvidia-smi", f"--id={self.index}", f"--query-gpu={self.Q}",
-                                          "--format=csv,noheader,nounits", "-lms", "200"],
+                                          "--format=csv,noheader,nounits", "-lms", "20"],
                                          stdout=self.f, stderr=subprocess.DEVNULL)
         except Exception:
             self.proc = None
@@ -149,6 +149,40 @@ class ClockSampler:
             return None
         return {"sm_mhz": statistics.median(sm), "sm_max_mhz": mx, "reasons": sorted(reasons),
                 "samples": len(sm)}
+
+
+def short(x):
+    """A copy with floats rounded to six significant digits."""
+    if isinstance(x, dict):
+        return {k: short(v) for k, v in x.items()}
+    if isinstance(x, (list, tuple)):
+        return [short(v) for v in x]
+    return float(f"{x:.6g}") if isinstance(x, float) else x
+
+
+def compact(line):
+    """The result line as it is printed: whole but for the extra measurements,
+    of which it keeps the headline numbers (a reader of the last few kilobytes
+    of the output gets all of it)."""
+    out = {k: v for k, v in line.items() if k not in ("kernels", "forms", "batch", "radial_table", "paper_models", "graphs",
+                                                     "serving")}
+    if line.get("cpu_baseline"):
+        out["cpu_baseline"] = {k: v for k, v in line["cpu_baseline"].items() if k != "split"}
+    out["ms_per_launch"] = {k: v["ms_per_launch"] for k, v in list(line.get("kernels", {}).items())[:5]}
+    out["forms_ms_per_step"] = {k: v["ms_per_step"] for k, v in line.get("forms", {}).items()}
+    if "batch" in line:
+        out["batch"] = {}
+        for k in ("fp32", "bf16"):
+            e = line["batch"][k].get("errors") or {}
+            out["batch"][k] = {"atom_evals_per_s": line["batch"][k]["atom_evals_per_s"],
+                               **{q: e[q] for q in ("max_dE_rel", "max_dF_over_rms") if q in e}}
+    if "paper_models" in line:
+        out["paper_models_ms"] = {k: {p: v[p]["ms_per_eval"] for p in ("fp32", "bf16")}
+                                  for k, v in line["paper_models"].items() if isinstance(v, dict)}
+    if "serving" in line:
+        keep = ("p50_ms", "p99_ms", "atom_steps_per_s")
+        out["serving_2000_per_s"] = {k: {q: v[q] for q in keep} for k, v in line["serving"]["at_2000_per_s"].items()}
+    return short(out)
 
 
 def kernel_traffic(name):
@@ -735,6 +769,8 @@ def main():
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--reps", type=int, default=64, help="fcc repeats of the large cell (64 = 1,048,576 atoms)")
     ap.add_argument("--no-extras", action="store_true", help="skip the batch and serving measurements")
+    ap.add_argument("--details", default=os.path.join(ROOT, "bench_details.json"),
+                    help="file for what the printed line leaves out: sweeps, per-system errors, every kernel ('' = none)")
     ap.add_argument("--serve-seconds", type=float, default=1.0, help="arrival window of each serving load point")
     ap.add_argument("--size-sweep", default="",
                     help="instead of the bench line: the FP32 MD step of the large lattice at these fcc repeats "
@@ -956,26 +992,41 @@ def main():
     entries = nl.size()[1]        # table entries screened per step (rc + skin)
     K = w.model.n_radial
     dims = [w.model.n_desc] + list(w.model.widths) + [1]
-    per_launch_flops = {"k_force": pairs * bwd_flops_per_pair(K), "k_desc": pairs * fwd_flops_per_pair(K),
-                        "k_mlp": n * mlp_flops_per_atom(dims), "k_mlp_res": n * mlp_flops_per_atom(dims)}
+    # k_force (and k_mlp where it is the FP32-pipe kernel) against the FP32 pipes; the
+    # split products of the network (six on BF16 parts) and of the descriptor (four on
+    # TF32 parts, half the BF16 rate) against the tensor cores, with the rest of the
+    # descriptor pass, the radial functions and geometry, against the FP32 pipes beside
+    bf16_peak = float(peaks["bf16_tflops_sustained"])
+    fp32_src = (f"FP32 FMA peak {nsm} SMs x 128 lanes x 2 flops x {clk_mhz:.0f} MHz (max SM clock, "
+                f"{peaks['source']} peaks file)")
+    bf16_src = f"sustained BF16 tensor rate, {peaks['source']} peaks file"
+    all64 = all(d == 64 for d in dims[:-1]) and len(dims) <= 4
+    split = (all(d % 16 == 0 for d in dims[:-1]) and max(dims[1:-1]) <= 128 and
+             not (all64 and tuning["tile_rows"] in (32, 64)))
+    mlp = n * mlp_flops_per_atom(dims)
+    net = {"flops": 6 * mlp, "peak": bf16_peak, "bound": "tensor", "src": bf16_src} if split else \
+        {"flops": mlp, "peak": fp32_peak, "bound": "alu", "src": fp32_src}
+    per_launch_flops = {
+        "k_force": {"flops": pairs * bwd_flops_per_pair(K), "peak": fp32_peak, "bound": "alu", "src": fp32_src},
+        "k_desc": {"flops": pairs * 4 * 2 * 16 * K, "peak": bf16_peak / 2, "bound": "tensor", "src": bf16_src + ", half",
+                   "alu_flops": pairs * (fwd_flops_per_pair(K) - 2 * 16 * K)},
+        "k_mlp": net, "k_mlp_res": net}
+
+    def figures(kn):
+        q, t = per_launch_flops[kn], kstats[kn][1] / max(kstats[kn][0], 1) * 1e-3
+        a = q["flops"] / t / 1e12
+        r = {"bound": q["bound"], "achieved": a, "peak": q["peak"], "unit": "TFLOP/s", "frac": a / q["peak"],
+             "traffic": kernel_traffic(kn)}
+        if "alu_flops" in q:
+            r["alu_frac"] = q["alu_flops"] / t / 1e12 / fp32_peak
+        return r
     ranked = sorted(kstats.items(), key=lambda kv: -kv[1][1])
-    dom, (dl, dms) = ranked[0]
-    avg_ms = dms / max(dl, 1)
+    dom = ranked[0][0]
     roof = None
     if dom in per_launch_flops:
-        ach = per_launch_flops[dom] / (avg_ms * 1e-3) / 1e12
-        roof = {"bound": "alu", "kernel": dom, "achieved": ach, "peak": fp32_peak, "unit": "TFLOP/s",
-                "frac": ach / fp32_peak, "traffic": kernel_traffic(dom),
-                "peak_source": f"FP32 FMA peak {nsm} SMs x 128 lanes x 2 flops x {clk_mhz:.0f} MHz "
-                               f"(max SM clock, {peaks['source']} peaks file)"}
-        # the descriptor and force passes take nearly equal time, so the
-        # dominant one can change between runs: every pair/network kernel's
-        # figures, the same way
-        roof["all"] = {}
-        for kn, fl in per_launch_flops.items():
-            if kn in kstats:
-                a = fl / (kstats[kn][1] / max(kstats[kn][0], 1) * 1e-3) / 1e12
-                roof["all"][kn] = {"achieved": a, "frac": a / fp32_peak, "traffic": kernel_traffic(kn)}
+        roof = {"kernel": dom, **figures(dom), "peak_source": per_launch_flops[dom]["src"]}
+        # every pair / network kernel's figures, the same way
+        roof["all"] = {kn: figures(kn) for kn in per_launch_flops if kn in kstats}
         # the in-cutoff screen is a stream: table entries in (nbr int32 +
         # shift char4), pair-cache entries out (float4 + float2 per pair), per
         # atom its split position (2 float4), segment bounds and pair count
@@ -1018,7 +1069,10 @@ def main():
             "forms": forms, "compute_only": compute_only, "tuning": tuning, "roofline": roof, "kernels": kernels,
             "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": launches, "clocks": clk}
     line.update(extras)
-    print(json.dumps(line), flush=True)
+    if args.details:
+        with open(args.details, "w") as fh:
+            json.dump(line, fh)
+    print(json.dumps(compact(line)), flush=True)
     if dist is not None:
         dist.destroy_process_group()
 
