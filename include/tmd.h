@@ -251,17 +251,19 @@ int64_t tmd_graph_replays(void);
 /*
  * Tile shapes of this implementation's kernels (the paper has no counterpart:
  * they are launch choices of the GPU path).  The results are the same up to
- * the order of FP64 partial sums, but for tile_rows on networks whose descriptor
- * length and hidden widths are all 64 (one or two hidden layers), where it
- * chooses between two kernels that agree to FP32 rounding.
+ * the order of FP64 partial sums, but for tile_rows 128 and, on networks whose
+ * descriptor length and hidden widths are all 64 (one or two hidden layers), any:
+ * there it chooses between two kernels that agree to FP32 rounding.
  *  tile_rows           atoms per tile of the FP32 network kernel on the FP32
  *                      pipes: 32 or 64; 128: tiles of the tensor-core kernel
- *                      (all widths 64); 0 = built-in choice: the tensor-core
- *                      kernel where it runs (hidden widths multiples of 16 up
- *                      to 128, activations of a tile within an SM's shared
- *                      memory), whose tiles have 128 atoms, else 32.  Networks
- *                      of other widths than 64 that run on the tensor cores do
- *                      so with every tile_rows;
+ *                      wherever it runs (hidden widths multiples of 16 up to
+ *                      128, activations of a tile within an SM's shared
+ *                      memory); 0 = built-in choice: the tensor-core kernel
+ *                      where it runs and the descriptor has at most 192
+ *                      columns (of at most four species, where no hidden layer
+ *                      is wider than 64) or more of one or two species before
+ *                      layers of more than 64; else 32.  Networks of other
+ *                      widths than 64 make that choice with 32 and 64, too;
  *  pair_blocks_per_sm  blocks per SM of the persistent force grid (0 = built-in
  *                      16); the descriptor pass sizes its grid by itself;
  *  ms                  output of the tuners: measured milliseconds of one

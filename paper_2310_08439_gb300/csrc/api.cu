@@ -791,7 +791,7 @@ tmd_status tune_shapes(tmd_model *m, cudaStream_t s, tmd_tuning *best, F &&run) 
     for (int r = 0; r < nrows && st == TMD_OK; ++r) {
         m->dm.tile_rows = (m->dm.precision == TMD_PREC_FP32) ? rows_fp32[r] : 0;
         if (m->dm.tile_rows && !tmd::mlp_rows_ok(m->dm, m->dm.tile_rows)) continue;
-        // (64 runs the same code as 32 on the tensor cores, unless all widths are 64)
+        // (32 and 64 are the same code where 128 is no choice and the tensor cores run)
         if (m->dm.tile_rows == 64 && tmd::mlp_split_ok(m->dm) && !tmd::mlp_rows_ok(m->dm, 128)) continue;
         for (int b = 0; b < 4 && st == TMD_OK; ++b) {
             m->dm.pair_bps = bps[b];

@@ -483,9 +483,9 @@ __device__ __forceinline__ Split2 split2(const float2 x) {
 // A lane stages two pairs (2 l, 2 l + 1 of a batch of 64) on packed FP32x2
 // arithmetic, so that most atoms need one batch.
 //
-// What bounds it: instruction issue (with three products and the sum of H on the
-// tensor cores 61 % of the slots, 760 warp instructions per atom at 53 pairs and K
-// = 16, FMA pipe 41 %, ALU 35 %, tensor 27 %).  The pass before it (packed FP32
+// What bounds it: instruction issue (59 % of the slots; 880 warp instructions per
+// atom at 54 pairs and K = 16; FMA pipe 36 %, ALU 34 %, tensor 30 %; waits on results
+// of the steps before it).  The pass before it (packed FP32
 // multiply-adds on a (K/8 x 4) block per lane) staged H as well, read 6 shared
 // float4 per 16 multiply-add instructions and waited on shared memory.  1,048,576
 // atoms, K = 16: 1.60 -> 1.20 ms; 148,176 atoms, K = 32: 0.356 -> 0.330; 39,366
@@ -1020,9 +1020,11 @@ __device__ __forceinline__ void virial_flush(float (&wacc)[9], double *acc, int 
 // contiguous run of atoms (perm order) and fills every batch of 32 lanes with
 // the rest of the current atom's pairs followed by the first pairs of the
 // next atom (two P' slots per warp, two self-force accumulators).
-// For one species: there it is the faster one (1,048,576 atoms, K = 16, 54
-// pairs: 2.06 ms, k_force 2.10; 39,366 atoms, K = 128: 0.63, k_force 0.70; only
-// K = 32 is 4 % the other way).  Two pairs per lane in this form: 2.37 ms.
+// For one species: there it is the faster one on the whole (1,048,576 atoms, K = 16,
+// 54 pairs: 2.04 ms, k_force 2.10; 128,000 atoms of the dense bcc lattice, 82 pairs:
+// 0.34 and 0.39; 39,366 atoms, K = 128: 0.63 and 0.70; K = 32 and 64 are 2 % the other
+// way: 0.530 and 0.517, 0.447 and 0.437), for its batches are full.  Two pairs per
+// lane in this form: 2.37 ms.
 template <int K, int S, bool TAB>
 __global__ void __launch_bounds__(PW * 32, 4) k_force_merged(DevModel m, DevNlist nl, const int32_t *__restrict__ types,
                                                           const float *__restrict__ Pin, const float *__restrict__ dG,
@@ -1200,7 +1202,7 @@ __global__ void __launch_bounds__(PW * 32, 4) k_force_tc(DevModel m, DevNlist nl
         const int a = nl.perm[p];
         pprime_setup<K, 1>(Pin, dG, p, sPd, kg, g, Wg);
         __syncwarp();
-        // B fragments of P' (k x 24), hi and lo parts: b0 = (k = t, n = g), b1 = (k = t + 4, n = g)
+        // B fragments of P' (k x 16), hi and lo parts: b0 = (k = t, n = g), b1 = (k = t + 4, n = g)
         uint32_t bh[KS][2][2], bl[KS][2][2];
 #pragma unroll
         for (int ks = 0; ks < KS; ++ks)
@@ -1364,9 +1366,9 @@ __global__ void __launch_bounds__(PW * 32, 4) k_force_tc(DevModel m, DevNlist nl
 // atoms, K = 16).  A batch passes through shared memory also with one species:
 // pairs read from global memory stay in registers over the channel loop, which
 // then spills (2.99 ms against 2.10).  Measured, one pair per lane -> two:
-// 16,384 atoms, 2 species, K = 16, 78 pairs: 87 -> 66 us; 225,008 atoms in 128
-// systems, 3 species, 54 pairs: 0.76 -> 0.67 ms; 93,802 atoms in 24 systems, 2
-// species: 0.40 -> 0.33 ms; table screened in the pass, 8,160 atoms: 46 -> 41 us.
+// 16,384 atoms, 2 species, K = 16, 78 pairs: 87 -> 64 us; 225,008 atoms in 128
+// systems, 3 species, 54 pairs: 0.76 -> 0.69 ms; 93,802 atoms in 24 systems, 2
+// species: 0.40 -> 0.33 ms; table screened in the pass, 8,160 atoms: 46 -> 39 us.
 //
 // CACHED: the pairs are those of the pair cache, else the table is screened
 // here.  PAW (batched): each atom's virial is summed over its own pairs and

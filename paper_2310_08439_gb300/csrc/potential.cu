@@ -890,8 +890,28 @@ static bool mlp_all64(const DevModel &dm) {
     return true;
 }
 
+// Whether the tensor cores are the built-in choice for a network that they can run.
+// It is made by the network alone: a system has the same bits evaluated by itself and
+// in a batch.  They are for descriptors of up to 192 columns (of at most four species
+// before narrow layers, of up to 64) and for longer ones of one or two species before
+// wider layers: k_mlp and tensor cores at 864 atoms, 16,384 and more: 64-64-64 20 and
+// 20 us, 1M atoms 850 and 420; 128-128-128 (2 species) 84 and 68, 128 and 68;
+// 256-128-128-128 (2 species) 149 and 119, 316 and 121; 70,304 atoms x 256-128-128 461
+// and 143.  With more species or narrow layers behind a longer descriptor it depends
+// on the number of atoms, for a tile runs the whole chain once for each species that
+// it holds and k_mlp's 32-atom tile of a narrow network is soon done: at 108, 864 and
+// 16,384 atoms 5 species x 160-64-64 take 59, 43, 72 us in k_mlp and 110, 51, 53; 5 x
+// 640-64-64 127, 90, 199 and 253, 112, 123; 512-64-64 43, 44, 165 and 52, 54, 62; 5 x
+// 320-128-128 139, 96, 203 and 187, 82, 88.  These stay in k_mlp; tile_rows 128 selects
+// the tensor cores, and the tuners try it.
+static bool split_default(const DevModel &dm) {
+    int maxw = 0;
+    for (int l = 1; l <= dm.L; ++l) maxw = std::max(maxw, dm.dims[l]);
+    return maxw > 64 ? dm.Dd <= 192 || dm.S <= 2 : dm.Dd <= 192 && dm.S <= 4;
+}
+
 bool mlp_rows_ok(const DevModel &dm, int tr) {
-    if (tr == 128) return mlp_all64(dm);
+    if (tr == 128) return mlp_all64(dm) || (mlp_split_ok(dm) && !split_default(dm));
     return (tr == 32 || tr == 64) && mlp_smem_tr(dm, tr) <= 227 * 1024;
 }
 
@@ -951,19 +971,17 @@ static tmd_status launch_network(const DevModel &dm, const int32_t *perm, const 
         set_error("the tcgen05 network kernel does not support these network shapes");
         return TMD_ERR_UNIMPLEMENTED;
     }
-    // FP32: the tensor cores wherever the widths are multiples of 16 up to 128 and
-    // a tile fits on chip; k_mlp has the rest.  At every size: one 32-atom tile
-    // 16.3 us against 15.6 in k_mlp, 1,048,576 atoms x 64-64 420 us against 850,
-    // 147,456 atoms x 128-128-128 247 us against 922, 70,304 atoms x 256-128-128 143
-    // us against 461, 32,000 x 640-64-64 148 us against 342; and the errors of
-    // forces and dE/dG are smaller (0.93 and 0.80 times over 113 and 23 random models
-    // of more than 192 columns).
+    // FP32: the tensor cores where the widths are multiples of 16 up to 128 and a
+    // tile fits on chip, where split_default says so; k_mlp has the rest.
+    // (The errors of forces and dE/dG are smaller there, too: 0.93 and 0.80 times
+    // over 113 and 23 random models of more than 192 columns.)
     // Where tile_rows has always chosen between two kernels (all widths 64), 32 and
     // 64 are k_mlp's tiles; on other networks tile_rows changes no result.  The
     // profile's "k_mlp_res" (all widths 64) and "k_mlp" (others) are the network
     // stage, whose kernel here is k_mlp_split.
     const bool all64 = mlp_all64(dm);
-    if (mlp_split_ok(dm) && !(all64 && (dm.tile_rows == 32 || dm.tile_rows == 64)))
+    if (mlp_split_ok(dm) && !(all64 && (dm.tile_rows == 32 || dm.tile_rows == 64)) &&
+        (dm.tile_rows == 128 || split_default(dm)))
         return mlp_split_launch(all64 ? "k_mlp_res" : "k_mlp", dm, perm, types, n, G, dG, e_atom, part_e, ntile_out, err, s);
     if ((st = set_mlp_smem(dm, dm.precision == TMD_PREC_BF16)) != TMD_OK) return st;
     if (dm.precision == TMD_PREC_BF16) {

@@ -52,3 +52,29 @@ def test_tiles_on_the_fp32_pipes(tmdlib, net, n_cells):
     assert np.array_equal(res[32]["forces"], res[64]["forces"])
     assert np.array_equal(res[32]["e_atom"], res[64]["e_atom"])
     assert np.array_equal(res[0]["forces"], res[32]["forces"]) != split
+
+
+@pytest.mark.parametrize("n", [1, 127, 128, 129, 300])
+@pytest.mark.parametrize("shape", ["dd96_w64x4", "dd192_w32_16", "dd512_2sp_w64"])
+def test_tensor_core_tiles_of_few_atoms(tmdlib, shape, n):
+    """The tensor-core kernel selected by tile_rows 128, at the edges of its tiles,
+    also where the built-in choice is k_mlp (narrow layers behind a long
+    descriptor); and the built-in choice beside it, within the same bars."""
+    import torch
+
+    import test_gpu_network_split as split
+    S, K, _, _ = split.SHAPES[shape]
+    s = split._system(n, S, seed=n + K)
+    p, o = split._model(shape, s.pos, s.types, s.box, s.pbc)
+    m = tmdlib.Model(p)
+    nl = tmdlib.NeighborList()
+    x, t = torch.as_tensor(s.pos, device="cuda"), torch.as_tensor(s.types, device="cuda")
+    nl.build(x, t, s.box, s.pbc, p.rc)
+    for rows in (128, 0):
+        m.tuning = {"tile_rows": rows, "pair_blocks_per_sm": 0}
+        out = {k: v.double().cpu().numpy() for k, v in tmdlib.evaluate(m, nl, x, t, s.box).items()}
+        assert abs(out["energy"].item() - o["energy"]) <= 1e-6 * abs(o["energy"])
+        assert np.abs(out["e_atom"] - o["e_atom"]).max() <= 1e-5 * np.abs(o["e_atom"]).max()
+        rms = float(np.sqrt((o["forces"] ** 2).mean()))
+        assert np.abs(out["forces"] - o["forces"]).max() <= 1e-5 * rms if rms else not out["forces"].any()
+        assert np.abs(out["virial"].reshape(3, 3) - o["virial"]).max() <= 1e-5 * np.abs(o["virial"]).max()

@@ -29,6 +29,12 @@ def _case(n_species=2, seed=3):
     return I.random_model(n_species, 16, 4.5, [64, 64], seed=seed), s
 
 
+def _model(tmd, p, **kw):
+    m = tmd.Model(p, **kw)
+    m.tuning = {"tile_rows": 128, "pair_blocks_per_sm": 0}   # on the tensor cores
+    return m
+
+
 def _dev(s):
     import torch
     return torch.as_tensor(s.pos, device="cuda"), torch.as_tensor(s.types, device="cuda")
@@ -38,7 +44,7 @@ def _dev(s):
 def test_enqueued_calls_give_nan(tmdlib, precision):
     import torch
     p, s = _case()
-    m = tmdlib.Model(p, precision=precision)
+    m = _model(tmdlib, p, precision=precision)
     nl = tmdlib.NeighborList()
     pos, types = _dev(s)
     nl.build(pos, types, s.box, s.pbc, p.rc)
@@ -67,7 +73,7 @@ def test_enqueued_calls_give_nan(tmdlib, precision):
 
 def test_single_steps_report_it(tmdlib):
     p, s = _case()
-    m = tmdlib.Model(p)
+    m = _model(tmdlib, p)
     g = tmdlib.System(s.n, s.box, s.pbc, skin=0.0)
     g.set_state(s.pos, s.vel, s.types, s.masses)
     ref = g.step(m, 1.0, 3)
@@ -88,7 +94,7 @@ def test_single_steps_report_it(tmdlib):
 @pytest.mark.parametrize("rebuild_every", [0, 5])
 def test_a_run_of_steps_is_stepped_again(tmdlib, rebuild_every):
     p, s = _case()
-    m = tmdlib.Model(p)
+    m = _model(tmdlib, p)
     out = []
     for armed in (False, True):
         g = tmdlib.System(s.n, s.box, s.pbc, skin=1.0)
@@ -106,7 +112,7 @@ def test_a_run_of_steps_is_stepped_again(tmdlib, rebuild_every):
 
 def test_a_step_before_a_run_is_not_taken_for_one_of_it(tmdlib):
     p, s = _case()
-    m = tmdlib.Model(p)
+    m = _model(tmdlib, p)
     g = tmdlib.System(s.n, s.box, s.pbc, skin=1.0)
     g.set_state(s.pos, s.vel, s.types, s.masses)
     tmdlib.selftest_network_timeout()
@@ -119,7 +125,7 @@ def test_a_step_before_a_run_is_not_taken_for_one_of_it(tmdlib):
 
 def test_host_state_and_host_evaluation_report_it(tmdlib):
     p, s = _case()
-    m = tmdlib.Model(p)
+    m = _model(tmdlib, p)
     g = tmdlib.System(s.n, s.box, s.pbc, skin=0.0)
     g.set_state(s.pos, s.vel, s.types, s.masses)
     first = None
@@ -147,7 +153,7 @@ def test_host_state_and_host_evaluation_report_it(tmdlib):
 
 def test_batches_report_it(tmdlib):
     p, s = _case()
-    m = tmdlib.Model(p)
+    m = _model(tmdlib, p)
     b = tmdlib.Batch([s, s, s], skin=1.0)
     ids = [0, 1, 2]
     E, W = b.compute(m, ids)

@@ -113,7 +113,9 @@ def test_network_sums_are_as_exact_as_their_rounding(tmdlib, S, K, widths, act, 
         return I.random_model(S, K, RC, widths, seed=K + len(widths), activation=act, feature_scale=scale, scale_floor=floor)
     G0 = O.evaluate(O.OracleModel(model(None)), s.pos, s.types, s.box, s.pbc, want_G=True)["G"]
     p = model([np.sqrt((G0[s.types == t] ** 2).mean(axis=0)) for t in range(S)])
-    G, dG = _descriptors(tmdlib, tmdlib.Model(p), s)
+    m = tmdlib.Model(p)
+    m.tuning = {"tile_rows": 128, "pair_blocks_per_sm": 0}   # on the tensor cores
+    G, dG = _descriptors(tmdlib, m, s)
     ref = _gradient64(p, G, s.types)
     err = float(np.linalg.norm(dG - ref) / np.linalg.norm(ref))
     with capsys.disabled():
