@@ -742,11 +742,16 @@ uint16_t bf16_bits(double x) {
     return (uint16_t)((v + 0x7fffu + ((v >> 16) & 1u)) >> 16);   // round to nearest even
 }
 
-double bf16_value(uint16_t b) {
+inline float bf16_value(uint16_t b) {
     const uint32_t v = (uint32_t)b << 16;
     float f;
     std::memcpy(&f, &v, 4);
     return f;
+}
+inline uint16_t bf16_round(float f) {   // (finite)
+    uint32_t v;
+    std::memcpy(&v, &f, 4);
+    return (uint16_t)((v + 0x7fffu + ((v >> 16) & 1u)) >> 16);   // round to nearest even
 }
 
 #include "mlp_split.cuh"
@@ -870,14 +875,14 @@ tmd_status mlp_umma_build(tmd_model *m, const double *const *weights) {
 
 bool mlp_split_ok(const DevModel &dm) {
     SplitNet u;
-    return dm.precision == TMD_PREC_FP32 && split_plan(dm, u);
+    return dm.precision == TMD_PREC_FP32 && dm.tb[0] && split_plan(dm, u);
 }
 
 tmd_status mlp_split_launch(const char *name, const DevModel &dm, const int32_t *perm, const int32_t *types, int64_t n,
                            const float *G, float *dG, float *e_atom, double *part_e, int *ntile_out, int32_t *err,
                            cudaStream_t s) {
     SplitNet u;
-    if (!split_plan(dm, u)) {
+    if (!dm.tb[0] || !split_plan(dm, u)) {
         set_error("network shapes outside the split-operand kernel");
         return TMD_ERR_UNIMPLEMENTED;
     }
@@ -906,7 +911,8 @@ tmd_status mlp_split_build(tmd_model *m, const double *const *weights) {
     }
     for (int s = 0; s < TMD_MAX_SPECIES; ++s) dm.tb[s] = nullptr;
     SplitShape sh;
-    if (!split_shape(dm, sh)) return TMD_OK;
+    SplitNet plan;
+    if (!split_shape(dm, sh) || !split_plan(dm, plan)) return TMD_OK;   // (k_mlp runs it: no planes)
     size_t off = 0, toff[2 * MAX_LAYERS];   // in BF16 values
     for (int pr = 0; pr < 2 * L; ++pr) {
         toff[pr] = off;
@@ -936,28 +942,41 @@ tmd_status mlp_split_build(tmd_model *m, const double *const *weights) {
             const int K = fwd ? dm.dims[l] : dm.dims[l + 1], N = fwd ? dm.dims[l + 1] : dm.dims[l];
             uint16_t *b = h.data() + per * s + toff[pr];
             const int np = sh.np[pr];
-            for (int nn = 0; nn < N; ++nn)
+            const size_t plane = (size_t)np * SN_KC;
+            for (int nn = 0; nn < N; ++nn) {
+                const int P = nn / np, r = nn % np;
+                const double *row = w + lo[l] + (fwd ? (size_t)nn * in : (size_t)nn);
+                const size_t step = fwd ? 1 : in;   // between the k of this n
                 for (int k0 = 0; k0 < K; k0 += 16) {   // the K of one MMA
                     double v[16], mx = 0.0;
                     for (int i = 0; i < 16; ++i) {
-                        const int k = k0 + i;
-                        v[i] = fwd ? w[lo[l] + (size_t)nn * in + k] : w[lo[l] + (size_t)k * in + nn];
-                        if (pr == 0) v[i] /= scale[(size_t)s * dm.Dd + k];
+                        v[i] = row[(k0 + i) * step];
+                        if (pr == 0) v[i] /= scale[(size_t)s * dm.Dd + k0 + i];
                         mx = std::max(mx, std::fabs(v[i]));
                     }
-                    const double unit = mx > 0.0 ? std::ldexp(1.0, std::ilogb(mx) - 7) : 1.0;
+                    // x_1 is a multiple of 2^-7 of the power of two at the largest
+                    // (added to 3 2^51 units and taken off again)
+                    const double big = mx > 0.0 ? std::ldexp(3.0, std::ilogb(mx) - 7 + 51) : 0.0;
+                    uint16_t *d = b + ((size_t)P * sh.nk[pr] + k0 / SN_KC) * plane * SN_PL + (size_t)(r >> 3) * (8 * SN_KC) +
+                                  (size_t)((k0 % SN_KC) >> 3) * 64 + (r & 7) * 8;
+                    float x[16];
+                    uint16_t h[16];
                     for (int i = 0; i < 16; ++i) {
-                        const int P = nn / np, r = nn % np, c = (k0 + i) / SN_KC, kk = (k0 + i) % SN_KC;
-                        const size_t plane = (size_t)np * SN_KC;
-                        const size_t idx = ((size_t)P * sh.nk[pr] + c) * plane * SN_PL + (size_t)(r >> 3) * (8 * SN_KC) +
-                                           (size_t)(kk >> 3) * 64 + (r & 7) * 8 + (kk & 7);
-                        double x = v[i];
-                        for (int q = 0; q < SN_PL; ++q) {
-                            b[idx + q * plane] = bf16_bits(q == 0 ? std::nearbyint(x / unit) * unit : x);
-                            x -= bf16_value(b[idx + q * plane]);
+                        const double y = (v[i] + big) - big;
+                        h[i] = bf16_round((float)y);
+                        x[i] = (float)(v[i] - y);
+                    }
+                    for (int q = 0;; ++q, d += plane) {
+                        std::memcpy(d, h, 16);
+                        std::memcpy(d + 64, h + 8, 16);   // (the next core matrix along K)
+                        if (q == SN_PL - 1) break;
+                        for (int i = 0; i < 16; ++i) {
+                            if (q > 0) x[i] -= bf16_value(h[i]);
+                            h[i] = bf16_round(x[i]);
                         }
                     }
                 }
+            }
         }
     }
     // the copies of a species in the order in which the kernel takes them
