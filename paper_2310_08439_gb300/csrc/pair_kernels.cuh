@@ -474,7 +474,7 @@ __device__ __forceinline__ Split2 split2(const float2 x) {
 // one sign, is not left to them: every lane adds the H that it forms, in FP32.
 // Errors against FP64 over 543 evaluations of the workloads and of random models,
 // lattices and sizes, as multiples of those with FP32 multiply-adds in sequence
-// and k_mlp (rms, K up to 64): G 0.95 to 0.99, forces 0.85 to 1.00.  Without x_l y_l
+// and k_mlp (rms, K up to 64): G 0.95 to 1.00, forces 0.85 to 1.00.  Without x_l y_l
 // and the rounding of x_l the forces of a 32-atom fcc and an 8,160-atom bcc cell are
 // 1.04 and 1.05 (now 0.99 and 1.00).
 // K = 128 (FINE false): three products and no separate sum, whose registers and
