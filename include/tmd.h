@@ -259,10 +259,9 @@ int64_t tmd_graph_replays(void);
  *                      wherever it runs (hidden widths multiples of 16 up to
  *                      128, activations of a tile within an SM's shared
  *                      memory); 0 = built-in choice: the tensor-core kernel
- *                      where it runs and the descriptor has at most 192
- *                      columns (of at most four species, where no hidden layer
- *                      is wider than 64) or more of one or two species before
- *                      layers of more than 64; else 32.  Networks of other
+ *                      where it runs, but for hidden layers of up to 64
+ *                      behind more than 192 descriptor columns of one species
+ *                      (of several in tmd_compute_noalloc); else 32.  Networks of other
  *                      widths than 64 make that choice with 32 and 64, too;
  *  pair_blocks_per_sm  blocks per SM of the persistent force grid (0 = built-in
  *                      16); the descriptor pass sizes its grid by itself;

@@ -92,6 +92,7 @@ void nlist_key(const tmd_nlist &nl, std::vector<uintptr_t> &k) {
                        nl.ph, nl.pl, nl.pq, nl.pq2, nl.npair, nl.sp};
     for (const void *q : p) k.push_back((uintptr_t)q);
     k.push_back((uintptr_t)nl.n_active);
+    for (int t = 0; t < TMD_MAX_SPECIES; ++t) k.push_back((uintptr_t)nl.type_count[t]);   // (the network's tiles)
 }
 
 void model_key(const tmd_model *m, std::vector<uintptr_t> &k) {

@@ -127,11 +127,13 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, uint32_t
 }
 // The outputs of the tiles tile0, tile0 + step, ... of a network that gave up:
 // NaN, and the evaluation's error word set (all threads of a block).
-__device__ __forceinline__ void net_invalid(const int32_t *perm, int64_t n, int Dd, float *dG, float *e_atom,
-                                            double *part_e, int tile0, int step, int ntile, int32_t *err) {
+// rows_of(tile, p0): the tile's number of rows, p0 its first.
+template <typename F>
+__device__ __forceinline__ void net_invalid(const int32_t *perm, int Dd, float *dG, float *e_atom, double *part_e, int tile0,
+                                            int step, int ntile, int32_t *err, F &&rows_of) {
     for (int tile = tile0; tile < ntile; tile += step) {
-        const int64_t p0 = (int64_t)tile * UM;
-        const int rows = (int)min((int64_t)UM, n - p0);
+        int64_t p0;
+        const int rows = rows_of(tile, p0);
         for (int i = threadIdx.x; i < rows * Dd; i += blockDim.x) dG[(size_t)p0 * Dd + i] = NAN;
         if (e_atom)
             for (int r = threadIdx.x; r < rows; r += blockDim.x) e_atom[perm[p0 + r]] = NAN;
@@ -600,7 +602,10 @@ __global__ void __launch_bounds__(UTHREADS, 2)
             mbar_drain(bar_done, pd & 1);
         }
         __syncthreads();
-        net_invalid(perm, n, Dd, dG, e_atom, part_e, blockIdx.x, gridDim.x, ntile, err);
+        net_invalid(perm, Dd, dG, e_atom, part_e, blockIdx.x, gridDim.x, ntile, err, [&](int t, int64_t &p0) {
+            p0 = (int64_t)t * UM;
+            return (int)min((int64_t)UM, n - p0);
+        });
     }
     tc_fence_before();
     __syncthreads();
@@ -637,11 +642,14 @@ __global__ void __launch_bounds__(32, 1) k_wait_probe(int32_t *__restrict__ gave
 }
 
 // net_invalid by itself (the self-test of what follows a time-out)
-__global__ void __launch_bounds__(256) k_net_invalid(const int32_t *__restrict__ perm, int64_t n, int Dd,
+__global__ void __launch_bounds__(256) k_net_invalid(const int32_t *__restrict__ perm, int rows, int Dd,
                                                      float *__restrict__ dG, float *__restrict__ e_atom,
-                                                     double *__restrict__ part_e, int ntile, int32_t *__restrict__ err) {
-    net_invalid(perm, n, Dd, dG, e_atom, part_e, blockIdx.x, gridDim.x, ntile, err);
-    if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&g_umma_status, DEV_ERR_TIMEOUT);
+                                                     double *__restrict__ part_e, int32_t *__restrict__ err) {
+    net_invalid(perm, Dd, dG, e_atom, part_e, 0, 1, 1, err, [&](int, int64_t &p0) {
+        p0 = 0;
+        return rows;
+    });
+    if (threadIdx.x == 0) atomicOr(&g_umma_status, DEV_ERR_TIMEOUT);
 }
 
 // launch plan for a model, or false when the shapes do not fit
@@ -758,8 +766,9 @@ inline uint16_t bf16_round(float f) {   // (finite)
 
 std::atomic<int> g_net_timeout{0};   // tmd_selftest_network_timeout
 
-// armed: the network just enqueued on s is treated as one that gave up in its
-// last tile (not within a capture: the graph would keep it)
+// armed: the network just enqueued on s is treated as one that gave up in the
+// last of its n atoms, up to 128 of them (not within a capture: the graph would
+// keep it)
 tmd_status giveup_if_armed(const DevModel &dm, const int32_t *perm, int64_t n, float *dG, float *e_atom, double *part_e,
                            int ntile, int32_t *err, cudaStream_t s) {
     if (!g_net_timeout.load()) return TMD_OK;
@@ -769,8 +778,8 @@ tmd_status giveup_if_armed(const DevModel &dm, const int32_t *perm, int64_t n, f
         return TMD_OK;
     }
     if (!g_net_timeout.exchange(0)) return TMD_OK;
-    const int64_t p0 = (int64_t)(ntile - 1) * UM;
-    k_net_invalid<<<1, 256, 0, s>>>(perm + p0, n - p0, dm.Dd, dG + (size_t)p0 * dm.Dd, e_atom, part_e + (ntile - 1), 1, err);
+    const int64_t p0 = (n - 1) / UM * UM;
+    k_net_invalid<<<1, 256, 0, s>>>(perm + p0, (int)(n - p0), dm.Dd, dG + (size_t)p0 * dm.Dd, e_atom, part_e + (ntile - 1), err);
     TMD_CUDA(cudaGetLastError());
     return TMD_OK;
 }
@@ -880,20 +889,30 @@ bool mlp_split_ok(const DevModel &dm) {
 
 tmd_status mlp_split_launch(const char *name, const DevModel &dm, const int32_t *perm, const int32_t *types, int64_t n,
                            const float *G, float *dG, float *e_atom, double *part_e, int *ntile_out, int32_t *err,
-                           cudaStream_t s) {
+                           const int32_t *count, cudaStream_t s) {
     SplitNet u;
     if (!dm.tb[0] || !split_plan(dm, u)) {
         set_error("network shapes outside the split-operand kernel");
         return TMD_ERR_UNIMPLEMENTED;
     }
     TMD_CUDA(smem_opt_in<k_mlp_split>(u.smem));
-    const int ntile = (int)((n + UM - 1) / UM);
+    // tiles: of each species for itself where its atoms lie together
+    SplitTiles tl = {};
+    int64_t sum = 0;
+    for (int q = 0; count && q < dm.S; ++q) sum += count[q];
+    const bool grouped = count && sum == n;
+    tl.ng = grouped ? dm.S : 1;
+    for (int q = 0; q < tl.ng; ++q) {
+        const int64_t c = grouped ? count[q] : n;
+        tl.off[q + 1] = tl.off[q] + c;
+        tl.first[q + 1] = tl.first[q] + (int)((c + UM - 1) / UM);
+    }
+    const int ntile = tl.first[tl.ng];
     int dev = 0, nsm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     const int grid = std::max(1, std::min(ntile, std::max(1, nsm) * u.blocks_per_sm));
-    TMD_LAUNCH(name, s, k_mlp_split<<<grid, UTHREADS, u.smem, s>>>(dm, u, perm, types, n, G, dG, e_atom, part_e, ntile,
-                                                                  err));
+    TMD_LAUNCH(name, s, k_mlp_split<<<grid, UTHREADS, u.smem, s>>>(dm, u, tl, perm, types, G, dG, e_atom, part_e, ntile, err));
     TMD_CUDA(cudaGetLastError());
     *ntile_out = ntile;
     return giveup_if_armed(dm, perm, n, dG, e_atom, part_e, ntile, err, s);

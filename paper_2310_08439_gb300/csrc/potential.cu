@@ -23,6 +23,8 @@ namespace {
 
 constexpr int PW = PAIR_WARPS;  // warps per block in the pair kernels
 constexpr int MT = 32;          // smallest network tile (sizes the per-tile energy partials)
+// per-tile energy partials at most: of 32-atom tiles, or of larger ones by species
+__host__ inline int part_tiles(int64_t n) { return (int)((n + MT - 1) / MT) + TMD_MAX_SPECIES; }
 constexpr int MLP_THREADS = 256;
 constexpr double FQ_INV = 1.0 / 4294967296.0;   // forces accumulate in units of 2^-32 eV/A
 
@@ -891,27 +893,25 @@ static bool mlp_all64(const DevModel &dm) {
 }
 
 // Whether the tensor cores are the built-in choice for a network that they can run.
-// It is made by the network alone: a system has the same bits evaluated by itself and
-// in a batch.  They are for descriptors of up to 192 columns (of at most four species
-// before narrow layers, of up to 64) and for longer ones of one or two species before
-// wider layers: k_mlp and tensor cores at 864 atoms, 16,384 and more: 64-64-64 20 and
-// 20 us, 1M atoms 850 and 420; 128-128-128 (2 species) 84 and 68, 128 and 68;
-// 256-128-128-128 (2 species) 149 and 119, 316 and 121; 70,304 atoms x 256-128-128 461
-// and 143.  With more species or narrow layers behind a longer descriptor it depends
-// on the number of atoms, for a tile runs the whole chain once for each species that
-// it holds and k_mlp's 32-atom tile of a narrow network is soon done: at 108, 864 and
-// 16,384 atoms 5 species x 160-64-64 take 59, 43, 72 us in k_mlp and 110, 51, 53; 5 x
-// 640-64-64 127, 90, 199 and 253, 112, 123; 512-64-64 43, 44, 165 and 52, 54, 62; 5 x
-// 320-128-128 139, 96, 203 and 187, 82, 88.  These stay in k_mlp; tile_rows 128 selects
-// the tensor cores, and the tuners try it.
-static bool split_default(const DevModel &dm) {
+// It is made by the network alone (and by whether tiles hold one species, `grouped`):
+// a system has the same bits evaluated by itself and in a batch.  k_mlp and tensor
+// cores at 108, 500 and 16,384 atoms: 3 species x 192-64-64 45, 45, 77 us and 27, 30, 32;
+// 5 x 160-64-64 58, 43, 74 and 29, 31, 33; 5 x 320-128-128 138, 96, 203 and 43, 47, 53;
+// 5 x 640-64-64 126, 90, 198 and 55, 61, 72.  Of one species, narrow layers behind a
+// long descriptor are sooner done in k_mlp's 32-atom tiles up to some 5,000 atoms:
+// 256-64-64 30, 31, 74 and 33, 34, 37; 512-64-64 43, 43, 164 and 51, 53, 62.  They stay
+// there, and so do those of several species where a tile holds them all and runs the
+// chain once for each (the allocation-free call at 108 and 4,000 atoms: 5 x 320-64-64 129
+// and 130 us, on the tensor cores 143 and 149; 3 x 384-64-64 88 and 90, 102 and 107; but 5
+// x 320-128-128 225 and 227, 182 and 188).  tile_rows 128 selects the tensor cores.
+static bool split_default(const DevModel &dm, bool grouped) {
     int maxw = 0;
     for (int l = 1; l <= dm.L; ++l) maxw = std::max(maxw, dm.dims[l]);
-    return maxw > 64 ? dm.Dd <= 192 || dm.S <= 2 : dm.Dd <= 192 && dm.S <= 4;
+    return maxw > 64 || (dm.Dd <= 192 && dm.S <= 4) || (grouped && dm.S > 1);
 }
 
 bool mlp_rows_ok(const DevModel &dm, int tr) {
-    if (tr == 128) return mlp_all64(dm) || (mlp_split_ok(dm) && !split_default(dm));
+    if (tr == 128) return mlp_all64(dm) || (mlp_split_ok(dm) && !split_default(dm, true));
     return (tr == 32 || tr == 64) && mlp_smem_tr(dm, tr) <= 227 * 1024;
 }
 
@@ -963,7 +963,7 @@ static tmd_status set_mlp_smem(const DevModel &dm, bool bf16) {
 
 static tmd_status launch_network(const DevModel &dm, const int32_t *perm, const int32_t *types, int64_t n,
                                  const float *G, float *dG, float *e_atom, double *part_e, int *ntile_out,
-                                 int32_t *err, cudaStream_t s) {
+                                 int32_t *err, const int32_t *count, cudaStream_t s) {
     tmd_status st;
     if (dm.precision == TMD_PREC_BF16 && network_kernel() != 2 && mlp_umma_supported(dm))
         return mlp_umma_launch(dm, perm, types, n, G, dG, e_atom, part_e, ntile_out, err, s);
@@ -981,8 +981,8 @@ static tmd_status launch_network(const DevModel &dm, const int32_t *perm, const 
     // stage, whose kernel here is k_mlp_split.
     const bool all64 = mlp_all64(dm);
     if (mlp_split_ok(dm) && !(all64 && (dm.tile_rows == 32 || dm.tile_rows == 64)) &&
-        (dm.tile_rows == 128 || split_default(dm)))
-        return mlp_split_launch(all64 ? "k_mlp_res" : "k_mlp", dm, perm, types, n, G, dG, e_atom, part_e, ntile_out, err, s);
+        (dm.tile_rows == 128 || split_default(dm, count != nullptr)))
+        return mlp_split_launch(all64 ? "k_mlp_res" : "k_mlp", dm, perm, types, n, G, dG, e_atom, part_e, ntile_out, err, count, s);
     if ((st = set_mlp_smem(dm, dm.precision == TMD_PREC_BF16)) != TMD_OK) return st;
     if (dm.precision == TMD_PREC_BF16) {
         const int ntile = (int)((n + BT - 1) / BT);
@@ -1039,7 +1039,7 @@ tmd_status reserve_compute(const DevModel &dm, tmd_nlist *nl, int64_t n_total, i
     if ((st = grow(&nl->ph, &nl->cap_ph, nt)) != TMD_OK) return st;
     if ((st = grow(&nl->pl, &nl->cap_pl, nt)) != TMD_OK) return st;
     if ((st = err_word(nl)) != TMD_OK) return st;
-    const int64_t nblk = pair_blocks(dm, na), ntile = (na + MT - 1) / MT;
+    const int64_t nblk = pair_blocks(dm, na), ntile = part_tiles(na);
     if ((st = grow(&nl->part, &nl->cap_part, ntile + 9 * nblk + 16)) != TMD_OK) return st;
     return pair_cache(nl, nt, nullptr);
 }
@@ -1082,10 +1082,11 @@ tmd_status run_descriptors(const tmd_model *model, tmd_nlist *nl, const double *
     TMD_LAUNCH("k_rows_to_atoms", s, k_rows_to_atoms<<<gb, 256, 0, s>>>(nl->G, nl->perm, n, dm.Dd, G));
     TMD_CUDA(cudaGetLastError());
     if (!dEdG) return TMD_OK;
-    const int ntile = (int)((n + MT - 1) / MT);
-    if ((st = grow(&nl->part, &nl->cap_part, ntile + 16)) != TMD_OK) return st;
+    if ((st = grow(&nl->part, &nl->cap_part, part_tiles(n) + 16)) != TMD_OK) return st;
     int nt = 0;
-    if ((st = launch_network(dm, nl->perm, types, n, nl->G, nl->dG, nullptr, nl->part, &nt, dn.err, s)) != TMD_OK) return st;
+    if ((st = launch_network(dm, nl->perm, types, n, nl->G, nl->dG, nullptr, nl->part, &nt, dn.err, nl->type_count, s)) !=
+        TMD_OK)
+        return st;
     TMD_LAUNCH("k_rows_to_atoms", s, k_rows_to_atoms<<<gb, 256, 0, s>>>(nl->dG, nl->perm, n, dm.Dd, dEdG));
     TMD_CUDA(cudaGetLastError());
     return TMD_OK;
@@ -1109,7 +1110,7 @@ tmd_status run_compute(const tmd_model *model, tmd_nlist *nl, const double *pos,
     if ((st = grow(&nl->P, &nl->cap_P, n * dm.S * dm.K * NHAR)) != TMD_OK) return st;
     if ((st = grow(&nl->Fq, &nl->cap_Fq, 3 * n)) != TMD_OK) return st;
     const int nblk = pair_blocks(dm, n);
-    const int ntile = (int)((n + MT - 1) / MT);
+    const int ntile = part_tiles(n);
     if ((st = grow(&nl->part, &nl->cap_part, ntile + 9 * (int64_t)nblk + 16)) != TMD_OK) return st;
     double *part_e = nl->part;
     double *part_w = nl->part + ntile;
@@ -1126,7 +1127,9 @@ tmd_status run_compute(const tmd_model *model, tmd_nlist *nl, const double *pos,
     TMD_CUDA(cudaMemsetAsync(nl->Fq, 0, sizeof(long long) * 3 * n, s));
     if ((st = dispatch_pair(dm, dn, pos, types, nl, part_w, nblk, s, true)) != TMD_OK) return st;
     int ne = 0;
-    if ((st = launch_network(dm, nl->perm, types, n, nl->G, nl->dG, e_atom, part_e, &ne, dn.err, s)) != TMD_OK) return st;
+    if ((st = launch_network(dm, nl->perm, types, n, nl->G, nl->dG, e_atom, part_e, &ne, dn.err, nl->type_count, s)) !=
+        TMD_OK)
+        return st;
     if ((st = dispatch_pair(dm, dn, pos, types, nl, part_w, nblk, s, false)) != TMD_OK) return st;
     TMD_LAUNCH("k_reduce", s, k_reduce<<<RED_CL, 256, 0, s>>>(part_e, ne, part_w, nblk, energy, virial));
     TMD_CUDA(cudaGetLastError());
@@ -1198,7 +1201,7 @@ tmd_status run_compute_owned(const tmd_model *model, tmd_nlist *nl, const double
     }
     if ((st = reserve_compute(dm, nl, n, n_owned)) != TMD_OK) return st;
     const int nblk = pair_blocks(dm, n_owned);
-    const int ntile = (int)((n_owned + MT - 1) / MT);
+    const int ntile = part_tiles(n_owned);
     double *part_e = nl->part;
     double *part_w = nl->part + ntile;
     if ((st = split_positions(nl, pos, n, s)) != TMD_OK) return st;
@@ -1210,7 +1213,7 @@ tmd_status run_compute_owned(const tmd_model *model, tmd_nlist *nl, const double
     TMD_CUDA(cudaMemsetAsync(nl->Fq, 0, sizeof(long long) * 3 * n, s));
     if ((st = dispatch_pair(dm, dn, pos, types, nl, part_w, nblk, s, true)) != TMD_OK) return st;
     int ne = 0;
-    if ((st = launch_network(dm, nl->perm_own, types, n_owned, nl->G, nl->dG, e_atom, part_e, &ne, dn.err, s)) != TMD_OK)
+    if ((st = launch_network(dm, nl->perm_own, types, n_owned, nl->G, nl->dG, e_atom, part_e, &ne, dn.err, own, s)) != TMD_OK)
         return st;
     if ((st = dispatch_pair(dm, dn, pos, types, nl, part_w, nblk, s, false)) != TMD_OK) return st;
     TMD_LAUNCH("k_reduce", s, k_reduce<<<RED_CL, 256, 0, s>>>(part_e, ne, part_w, nblk, energy, virial));
@@ -1410,7 +1413,7 @@ tmd_status run_compute_noalloc(const tmd_model *model, const int64_t *off, const
     TMD_CUDA(cudaMemsetAsync(w.Fq, 0, sizeof(unsigned long long) * 3 * n, s));
     if ((st = dispatch_pair(dm, dn, pos, types, &w, part_w, nblk, s, true)) != TMD_OK) return st;
     int ne = 0;
-    if ((st = launch_network(dm, w.perm, types, n, w.G, w.dG, e_atom, part_e, &ne, dn.err, s)) != TMD_OK) return st;
+    if ((st = launch_network(dm, w.perm, types, n, w.G, w.dG, e_atom, part_e, &ne, dn.err, nullptr, s)) != TMD_OK) return st;
     if ((st = dispatch_pair(dm, dn, pos, types, &w, part_w, nblk, s, false)) != TMD_OK) return st;
     TMD_LAUNCH("k_reduce", s, k_reduce<<<RED_CL, 256, 0, s>>>(part_e, ne, part_w, nblk, energy, virial));
     TMD_CUDA(cudaGetLastError());
@@ -1454,7 +1457,7 @@ tmd_status run_compute_batch(const tmd_model *model, tmd_nlist *nl, const double
         if ((st = grow(&nl->P, &nl->cap_P, na * dm.S * dm.K * NHAR)) != TMD_OK) return st;
         if ((st = grow(&nl->Fq, &nl->cap_Fq, 3 * n_total)) != TMD_OK) return st;
         const int nblk = pair_blocks(dm, na);
-        const int ntile = (int)((na + MT - 1) / MT);
+        const int ntile = part_tiles(na);
         if ((st = grow(&nl->part, &nl->cap_part, ntile + 9 * (int64_t)nblk + 16)) != TMD_OK) return st;
         if ((st = split_positions(nl, pos, n_total, s)) != TMD_OK) return st;
         if ((st = pair_cache(nl, n_total, s)) != TMD_OK) return st;
@@ -1468,7 +1471,8 @@ tmd_status run_compute_batch(const tmd_model *model, tmd_nlist *nl, const double
         TMD_CUDA(cudaMemsetAsync(nl->Fq, 0, sizeof(long long) * 3 * n_total, s));
         if ((st = dispatch_pair(dm, dn, pos, types, nl, nullptr, nblk, s, true)) != TMD_OK) return st;
         int ne = 0;
-        if ((st = launch_network(dm, nl->perm, types, na, nl->G, nl->dG, e_atom, nl->part, &ne, dn.err, s)) != TMD_OK)
+        if ((st = launch_network(dm, nl->perm, types, na, nl->G, nl->dG, e_atom, nl->part, &ne, dn.err, nl->type_count, s)) !=
+            TMD_OK)
             return st;
         if ((st = dispatch_pair(dm, dn, pos, types, nl, nl->part + ntile, nblk, s, false, w_atom)) != TMD_OK)
             return st;

@@ -77,11 +77,12 @@ size_t mlp_bf16_smem_bytes(const DevModel &dm);
 bool mlp_umma_supported(const DevModel &dm);
 tmd_status mlp_umma_launch(const DevModel &dm, const int32_t *perm, const int32_t *types, int64_t n, const float *G,
                            float *dG, float *e_atom, double *part_e, int *ntile_out, int32_t *err, cudaStream_t s);
-// tcgen05 form of the FP32 network on split operands (mlp_split.cuh)
+// tcgen05 form of the FP32 network on split operands (mlp_split.cuh); count: atoms
+// of each species, which perm has one species after the other (nullptr: it has not)
 bool mlp_split_ok(const DevModel &dm);
 tmd_status mlp_split_launch(const char *name, const DevModel &dm, const int32_t *perm, const int32_t *types, int64_t n,
                            const float *G, float *dG, float *e_atom, double *part_e, int *ntile_out, int32_t *err,
-                           cudaStream_t s);
+                           const int32_t *count, cudaStream_t s);
 // network kernel of the BF16 form: 0 = tcgen05 when the shapes allow it, else
 // mma.sync; 1 = tcgen05 only; 2 = mma.sync only
 int network_kernel();

@@ -58,8 +58,7 @@ def test_tiles_on_the_fp32_pipes(tmdlib, net, n_cells):
 @pytest.mark.parametrize("shape", ["dd96_w64x4", "dd192_w32_16", "dd512_2sp_w64"])
 def test_tensor_core_tiles_of_few_atoms(tmdlib, shape, n):
     """The tensor-core kernel selected by tile_rows 128, at the edges of its tiles,
-    also where the built-in choice is k_mlp (narrow layers behind a long
-    descriptor); and the built-in choice beside it, within the same bars."""
+    species by species; the built-in choice beside it, within the same bars."""
     import torch
 
     import test_gpu_network_split as split
@@ -78,3 +77,29 @@ def test_tensor_core_tiles_of_few_atoms(tmdlib, shape, n):
         rms = float(np.sqrt((o["forces"] ** 2).mean()))
         assert np.abs(out["forces"] - o["forces"]).max() <= 1e-5 * rms if rms else not out["forces"].any()
         assert np.abs(out["virial"].reshape(3, 3) - o["virial"]).max() <= 1e-5 * np.abs(o["virial"]).max()
+
+
+@pytest.mark.parametrize("counts", [(1, 0, 5), (128, 129, 127), (0, 0, 256), (3, 260, 1)])
+def test_tiles_begin_where_a_species_begins(tmdlib, counts):
+    """Species of none, one, and around 128 atoms: more tiles than 32-atom ones in
+    the smallest case (their energies have room of their own), tiles of a species
+    that end short of 128, and the per-atom energies that add up to the total."""
+    import torch
+    rng = np.random.default_rng(sum(counts))
+    n = sum(counts)
+    reps = int(np.ceil((n / 4) ** (1 / 3)))
+    pos, box = I.lattice("fcc", (reps, reps, reps), 3.8)
+    pos = I.jitter_and_wrap(pos, box, 0.1, rng)[:n]
+    types = rng.permutation(np.repeat(np.arange(3), counts)).astype(np.int32)
+    p = I.random_model(3, 8, 4.5, [64, 32], seed=5)
+    pbc = np.zeros(3, np.int32)
+    o = O.evaluate(O.OracleModel(p), pos, types, box, pbc)
+    nl = tmdlib.NeighborList()
+    x, t = torch.as_tensor(pos, device="cuda"), torch.as_tensor(types, device="cuda")
+    nl.build(x, t, box, pbc, p.rc)
+    out = {k: v.double().cpu().numpy() for k, v in tmdlib.evaluate(tmdlib.Model(p), nl, x, t, box).items()}
+    assert np.abs(out["e_atom"] - o["e_atom"]).max() <= 1e-5 * np.abs(o["e_atom"]).max()
+    assert abs(out["energy"].item() - out["e_atom"].sum()) <= 1e-12 * abs(o["energy"])
+    rms = float(np.sqrt((o["forces"] ** 2).mean()))
+    assert np.abs(out["forces"] - o["forces"]).max() <= 1e-5 * rms
+    assert np.abs(out["virial"].reshape(3, 3) - o["virial"]).max() <= 1e-5 * np.abs(o["virial"]).max()
